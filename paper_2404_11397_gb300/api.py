@@ -18,9 +18,16 @@ from . import _lib
 from ._lib import MODES, NPAR, check, load
 
 
-def _stream_handle(stream: Optional[torch.cuda.Stream]) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
+    """The cudaStream_t of the given stream, or of the current one.  Addresses are
+    passed to the C ABI as plain ints (its prototypes convert them): a Stream
+    object for the current stream and a c_void_p per argument cost a batch call
+    about a third of its host time."""
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _mode(mode) -> int:
@@ -34,6 +41,8 @@ def _theta_dev(theta: torch.Tensor) -> torch.Tensor:
         raise TypeError("theta must be a CUDA tensor [W, 13]")
     if theta.dim() != 2 or theta.shape[1] != NPAR:
         raise ValueError("theta must have shape [W, 13]")
+    if theta.dtype is torch.float64 and theta.is_contiguous():
+        return theta
     return theta.to(torch.float64).contiguous()
 
 
@@ -108,7 +117,7 @@ def _check_mala_shapes(z, logp, gz, xi, u) -> int:
         raise ValueError("z must have shape [W, 13]")
     W = z.shape[0]
     for name, t, shape in (("logp", logp, (W,)), ("gz", gz, (W, NPAR)), ("xi", xi, (W, NPAR)), ("u", u, (W,))):
-        if t is not None and tuple(t.shape) != shape:
+        if t is not None and t.shape != shape:
             raise ValueError(f"{name} must have shape {list(shape)}, got {list(t.shape)}")
     return W
 
@@ -160,7 +169,7 @@ class Event:
         th = np.asarray(theta_ref, dtype=np.float64).reshape(NPAR)
         for j in range(NPAR):
             desc.theta_ref[j] = float(th[j])
-        desc.cuda_stream = _stream_handle(stream).value if torch.cuda.is_available() else None
+        desc.cuda_stream = _stream_handle(stream) if torch.cuda.is_available() else None
         handle = ctypes.c_void_p()
         check(lib.rb_build_summary(ctypes.byref(desc), ctypes.byref(handle)), "rb_build_summary")
         del keep
@@ -283,9 +292,8 @@ def loglike(event: Event, theta: torch.Tensor, mode="mixed", stream=None) -> tor
     """Batched RB log-likelihood [W] (float64, on theta's device)."""
     th = _theta_dev(theta)
     out = torch.empty(th.shape[0], dtype=torch.float64, device=th.device)
-    check(load().rb_loglike_batch(event.handle, ctypes.c_void_p(th.data_ptr()), th.shape[0],
-                                  ctypes.c_void_p(out.data_ptr()), _mode(mode), _stream_handle(stream)),
-          "rb_loglike_batch")
+    check(load().rb_loglike_batch(event.handle, th.data_ptr(), th.shape[0], out.data_ptr(), _mode(mode),
+                                  _stream_handle(stream)), "rb_loglike_batch")
     return out
 
 
@@ -297,9 +305,8 @@ def rebuild_loglike_grad(event: Event, theta: torch.Tensor, mode="mixed", stream
     W = th.shape[0]
     out = torch.empty(W, dtype=torch.float64, device=th.device)
     g = torch.empty(W, NPAR, dtype=torch.float64, device=th.device) if grad else None
-    check(load().rb_rebuild_loglike_grad(event.handle, ctypes.c_void_p(th.data_ptr()), W,
-                                         ctypes.c_void_p(out.data_ptr()),
-                                         ctypes.c_void_p(g.data_ptr()) if g is not None else None, _mode(mode),
+    check(load().rb_rebuild_loglike_grad(event.handle, th.data_ptr(), W, out.data_ptr(),
+                                         g.data_ptr() if g is not None else None, _mode(mode),
                                          _stream_handle(stream)), "rb_rebuild_loglike_grad")
     return (out, g) if grad else out
 
@@ -331,9 +338,8 @@ def loglike_full(event: Event, theta: torch.Tensor, mode="mixed", stream=None) -
     """Full-grid (un-binned) log-likelihood [W] (float64, on theta's device)."""
     th = _theta_dev(theta)
     out = torch.empty(th.shape[0], dtype=torch.float64, device=th.device)
-    check(load().rb_loglike_full_batch(event.handle, ctypes.c_void_p(th.data_ptr()), th.shape[0],
-                                       ctypes.c_void_p(out.data_ptr()), _mode(mode), _stream_handle(stream)),
-          "rb_loglike_full_batch")
+    check(load().rb_loglike_full_batch(event.handle, th.data_ptr(), th.shape[0], out.data_ptr(), _mode(mode),
+                                       _stream_handle(stream)), "rb_loglike_full_batch")
     return out
 
 
@@ -343,14 +349,13 @@ def loglike_grad(event: Event, theta: torch.Tensor, mode="mixed", stream=None):
     W = th.shape[0]
     out = torch.empty(W, dtype=torch.float64, device=th.device)
     grad = torch.empty(W, NPAR, dtype=torch.float64, device=th.device)
-    check(load().rb_loglike_grad_batch(event.handle, ctypes.c_void_p(th.data_ptr()), W,
-                                       ctypes.c_void_p(out.data_ptr()), ctypes.c_void_p(grad.data_ptr()),
-                                       _mode(mode), _stream_handle(stream)), "rb_loglike_grad_batch")
+    check(load().rb_loglike_grad_batch(event.handle, th.data_ptr(), W, out.data_ptr(), grad.data_ptr(), _mode(mode),
+                                       _stream_handle(stream)), "rb_loglike_grad_batch")
     return out, grad
 
 
 def _host_ptr(a) -> int:
-    return a.data_ptr() if isinstance(a, torch.Tensor) else a.ctypes.data
+    return a.data_ptr() if isinstance(a, torch.Tensor) else a.__array_interface__["data"][0]
 
 
 def loglike_grad_host(event: Event, theta: np.ndarray, logl_out, grad_out=None, mode="mixed", stream=None) -> None:
@@ -374,7 +379,7 @@ def strain(geom, gmst: float, theta, T: float, kmin: int, n_freq: int, device="c
     th = np.ascontiguousarray(theta, dtype=np.float64).reshape(NPAR)
     out = torch.empty(n_freq, 2, dtype=torch.float64, device=device)
     check(load().rb_strain(g.ctypes.data_as(_lib.c_double_p), float(gmst), th.ctypes.data_as(_lib.c_double_p),
-                           float(T), int(kmin), int(n_freq), ctypes.c_void_p(out.data_ptr()),
+                           float(T), int(kmin), int(n_freq), out.data_ptr(),
                            _stream_handle(stream)), "rb_strain")
     return torch.view_as_complex(out)
 
@@ -392,9 +397,8 @@ def mala_init(event: Event, z: torch.Tensor, lo, hi, mode="mixed", stream=None):
     logp = torch.empty(W, dtype=torch.float64, device=zz.device)
     gz = torch.empty(W, NPAR, dtype=torch.float64, device=zz.device)
     lo_, hi_ = _host13(lo), _host13(hi)
-    check(load().rb_mala_init(event.handle, ctypes.c_void_p(zz.data_ptr()), W, ctypes.c_void_p(lo_.ctypes.data),
-                              ctypes.c_void_p(hi_.ctypes.data), ctypes.c_void_p(logp.data_ptr()),
-                              ctypes.c_void_p(gz.data_ptr()), _mode(mode), _stream_handle(stream)), "rb_mala_init")
+    check(load().rb_mala_init(event.handle, zz.data_ptr(), W, _host_ptr(lo_), _host_ptr(hi_), logp.data_ptr(),
+                              gz.data_ptr(), _mode(mode), _stream_handle(stream)), "rb_mala_init")
     return logp, gz
 
 
@@ -403,16 +407,14 @@ def mala_step(event: Event, z: torch.Tensor, logp: torch.Tensor, gz: torch.Tenso
     """One MALA step of every chain; z, logp, gz are updated in place (they
     must be contiguous float64 device tensors).  Returns accepted [W] (int32)."""
     for t in (z, logp, gz, xi, u):
-        if not (t.is_cuda and t.dtype == torch.float64 and t.is_contiguous()):
+        if not (t.is_cuda and t.dtype is torch.float64 and t.is_contiguous()):
             raise ValueError("mala_step: z, logp, gz, xi, u must be contiguous float64 CUDA tensors")
     W = _check_mala_shapes(z, logp, gz, xi, u)
     acc = torch.empty(W, dtype=torch.int32, device=z.device)
     eps_, lo_, hi_ = _host13(eps), _host13(lo), _host13(hi)
-    check(load().rb_mala_step(event.handle, ctypes.c_void_p(z.data_ptr()), ctypes.c_void_p(logp.data_ptr()),
-                              ctypes.c_void_p(gz.data_ptr()), W, ctypes.c_void_p(eps_.ctypes.data),
-                              ctypes.c_void_p(lo_.ctypes.data), ctypes.c_void_p(hi_.ctypes.data),
-                              ctypes.c_void_p(xi.data_ptr()), ctypes.c_void_p(u.data_ptr()),
-                              ctypes.c_void_p(acc.data_ptr()), _mode(mode), _stream_handle(stream)), "rb_mala_step")
+    check(load().rb_mala_step(event.handle, z.data_ptr(), logp.data_ptr(), gz.data_ptr(), W, _host_ptr(eps_),
+                              _host_ptr(lo_), _host_ptr(hi_), xi.data_ptr(), u.data_ptr(), acc.data_ptr(),
+                              _mode(mode), _stream_handle(stream)), "rb_mala_step")
     return acc
 
 
