@@ -24,7 +24,7 @@ cudaError_t launch_ref_values(const double* theta_ref_dev, const EventConst& ec,
 cudaError_t launch_setup(int mode, const double* theta, int64_t W, const EventConst& ec, const RefValues* ref,
                          void* ws, void* tan, bool grad, cudaStream_t s);
 cudaError_t launch_rb_mixed(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl,
-                            double* grad, bool phase64, cudaStream_t s, int n_sm, const MalaArgs* mala);
+                            double* grad, bool phase64, bool spread, cudaStream_t s, int n_sm, const MalaArgs* mala);
 cudaError_t launch_rb_f64(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl, double* grad,
                           cudaStream_t s, int n_sm, const MalaArgs* mala);
 cudaError_t launch_bin_edges(double f_low, double f_high, double T, int64_t kmin, int64_t N, int B, int64_t* edges,
@@ -1183,7 +1183,7 @@ size_t walker_ws_bytes(int mode, bool grad) {
 // Set-up kernel + likelihood kernel for one batch.  If `scratch` is NULL the
 // per-walker workspace is taken from the stream-ordered pool of `s`.
 int run_batch(const EventEntry* e, const double* theta, int64_t W, double* logl, double* grad, int mode,
-              cudaStream_t s, void* scratch, const MalaArgs* mala) {
+              cudaStream_t s, void* scratch, const MalaArgs* mala, bool spread) {
   if (!e) return set_error(RB_EINVAL, "NULL event");
   if (W < 0) return set_error(RB_EINVAL, "W < 0");
   if (mode != RB_MIXED && mode != RB_FP64 && mode != RB_MIXED_F64PHASE) return set_error(RB_EINVAL, "bad mode %d", mode);
@@ -1202,7 +1202,7 @@ int run_batch(const EventEntry* e, const double* theta, int64_t W, double* logl,
   void* tan = want_grad ? static_cast<void*>(static_cast<char*>(buf) + ws_bytes) : nullptr;
   int rc = RB_OK;
   err = launch_setup(mode, theta, W, e->ec, e->d_ref, ws, tan, want_grad, s);
-  if (err == cudaSuccess) err = launch_batch_main(e, ws, tan, W, logl, grad, mode, s, mala);
+  if (err == cudaSuccess) err = launch_batch_main(e, ws, tan, W, logl, grad, mode, spread, s, mala);
   if (err != cudaSuccess) rc = cuda_fail(err, "likelihood kernels");
   else count_launches(2);
   if (!scratch) cudaFreeAsync(buf, s);
@@ -1250,7 +1250,7 @@ int rebuild_and_batch(EventEntry& e, const double* theta, int64_t W, double* log
   const SideSetup ss{theta, W, buf, tan, want_grad, data_ready};
   int rc = rebuild_event(e, nullptr, mode, s, &ss);
   if (rc == RB_OK) {
-    if ((err = launch_batch_main(&e, buf, tan, W, logl, grad, mode, s, nullptr)) != cudaSuccess)
+    if ((err = launch_batch_main(&e, buf, tan, W, logl, grad, mode, true, s, nullptr)) != cudaSuccess)
       rc = cuda_fail(err, "likelihood kernel");
     else
       count_launches(1);
@@ -1263,7 +1263,7 @@ int rebuild_and_batch(EventEntry& e, const double* theta, int64_t W, double* log
 }
 
 cudaError_t launch_batch_main(const EventEntry* e, void* ws, void* tan, int64_t W, double* logl, double* grad, int mode,
-                              cudaStream_t s, const MalaArgs* mala) {
+                              bool spread, cudaStream_t s, const MalaArgs* mala) {
   const int n_sm = sm_count();
   cudaEvent_t tb = static_cast<cudaEvent_t>(g_trace_before.load());
   cudaEvent_t ta = static_cast<cudaEvent_t>(g_trace_after.load());
@@ -1272,7 +1272,7 @@ cudaError_t launch_batch_main(const EventEntry* e, void* ws, void* tan, int64_t 
     if (mode == RB_FP64)
       err = launch_rb_f64(e->dev, ws, tan, W, logl, grad, s, n_sm, mala);
     else
-      err = launch_rb_mixed(e->dev, ws, tan, W, logl, grad, mode == RB_MIXED_F64PHASE, s, n_sm, mala);
+      err = launch_rb_mixed(e->dev, ws, tan, W, logl, grad, mode == RB_MIXED_F64PHASE, spread, s, n_sm, mala);
   }
   if (err == cudaSuccess && ta) err = cudaEventRecord(ta, s);
   return err;

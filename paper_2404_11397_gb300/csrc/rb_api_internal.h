@@ -118,8 +118,10 @@ size_t walker_ws_bytes(int mode, bool grad);
 // Set-up + likelihood kernels for one batch; scratch = NULL takes the
 // workspace from the stream-ordered allocator.  With mala, the likelihood
 // kernel finishes each walker with the MALA accept step (logl, grad unused).
+// spread = false for launches that share the GPU with others (the server's):
+// few, dense blocks instead of a small batch spread over every SM.
 int run_batch(const EventEntry* e, const double* theta, int64_t W, double* logl, double* grad, int mode,
-              cudaStream_t s, void* scratch, const MalaArgs* mala = nullptr);
+              cudaStream_t s, void* scratch, const MalaArgs* mala = nullptr, bool spread = true);
 
 // Fiducial values, summary data, tables and base of an event from the given
 // device strain/PSD (NULL: the event's resident copy); no allocation, no
@@ -144,7 +146,7 @@ int rebuild_and_batch(EventEntry& e, const double* theta, int64_t W, double* log
                       cudaStream_t s, cudaEvent_t data_ready);
 // The likelihood kernel of a batch whose set-up has been done (trace events around it).
 cudaError_t launch_batch_main(const EventEntry* e, void* ws, void* tan, int64_t W, double* logl, double* grad, int mode,
-                              cudaStream_t s, const MalaArgs* mala);
+                              bool spread, cudaStream_t s, const MalaArgs* mala);
 
 // Events recorded on the launch stream right before / after the main
 // likelihood kernel of every batch (NULL disables).

@@ -1023,8 +1023,10 @@ static cudaError_t blocks_per_sm(const void* fn, int threads, size_t smem, int* 
   return cudaSuccess;
 }
 
+constexpr int64_t kThinWalkers = 4;  // an SM's sub-partitions
+
 template <int ND, bool GRAD, bool PHASE64, bool MALA>
-static cudaError_t launch_mixed_nd(const LaunchArgs& a, cudaStream_t s, int n_sm) {
+static cudaError_t launch_mixed_nd(const LaunchArgs& a, bool spread, cudaStream_t s, int n_sm) {
   // the kernel copies records in 16-byte and tangents in 8-byte asynchronous copies
   if (reinterpret_cast<uintptr_t>(a.ws) % 16 != 0 || (GRAD && reinterpret_cast<uintptr_t>(a.tan) % 8 != 0))
     return cudaErrorMisalignedAddress;
@@ -1034,31 +1036,38 @@ static cudaError_t launch_mixed_nd(const LaunchArgs& a, cudaStream_t s, int n_sm
   cudaError_t err = blocks_per_sm(fn, kThreads, smem, &per_sm);
   if (err != cudaSuccess) return err;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int64_t blocks_needed = (a.W * 32 + kThreads - 1) / kThreads;
-  const int64_t grid = std::min<int64_t>(blocks_needed, (int64_t)per_sm * n_sm);
+  // spread: a batch that does not fill the SMs with 16 walkers per block takes
+  // more of them, down to one walker per SM sub-partition (the warps of a block
+  // share its FP32 pipe; below four walkers nothing is left to share).  GPU time
+  // of a call, 3 detectors, 500 bins, with the gradient: 64 walkers 24.1 -> 16.2
+  // us, 1024 walkers 24.2 -> 18.4 us.  Otherwise (launches that share the GPU
+  // with others) the blocks stay dense: fewer SMs are held, for longer.
+  const int64_t dense = (a.W * 32 + kThreads - 1) / kThreads;
+  const int64_t thin = spread ? std::min<int64_t>((a.W + kThinWalkers - 1) / kThinWalkers, n_sm) : 0;
+  const int64_t grid = std::min<int64_t>(std::max<int64_t>(dense, thin), (int64_t)per_sm * n_sm);
   k_rb_mixed<ND, GRAD, PHASE64, MALA><<<(unsigned)grid, kThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <bool GRAD, bool PHASE64, bool MALA = false>
-static cudaError_t launch_mixed_t(const LaunchArgs& a, cudaStream_t s, int n_sm) {
+static cudaError_t launch_mixed_t(const LaunchArgs& a, bool spread, cudaStream_t s, int n_sm) {
   switch (a.ev.n_det) {
-    case 1: return launch_mixed_nd<1, GRAD, PHASE64, MALA>(a, s, n_sm);
-    case 2: return launch_mixed_nd<2, GRAD, PHASE64, MALA>(a, s, n_sm);
-    case 3: return launch_mixed_nd<3, GRAD, PHASE64, MALA>(a, s, n_sm);
+    case 1: return launch_mixed_nd<1, GRAD, PHASE64, MALA>(a, spread, s, n_sm);
+    case 2: return launch_mixed_nd<2, GRAD, PHASE64, MALA>(a, spread, s, n_sm);
+    case 3: return launch_mixed_nd<3, GRAD, PHASE64, MALA>(a, spread, s, n_sm);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_rb_mixed(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl, double* grad,
-                            bool phase64, cudaStream_t s, int n_sm, const MalaArgs* mala) {
+                            bool phase64, bool spread, cudaStream_t s, int n_sm, const MalaArgs* mala) {
   LaunchArgs a{ev, ws, tan, W, logl, grad, {}};
   if (mala) {
     a.mala = *mala;
-    return phase64 ? launch_mixed_t<true, true, true>(a, s, n_sm) : launch_mixed_t<true, false, true>(a, s, n_sm);
+    return phase64 ? launch_mixed_t<true, true, true>(a, spread, s, n_sm) : launch_mixed_t<true, false, true>(a, spread, s, n_sm);
   }
-  if (grad) return phase64 ? launch_mixed_t<true, true>(a, s, n_sm) : launch_mixed_t<true, false>(a, s, n_sm);
-  return phase64 ? launch_mixed_t<false, true>(a, s, n_sm) : launch_mixed_t<false, false>(a, s, n_sm);
+  if (grad) return phase64 ? launch_mixed_t<true, true>(a, spread, s, n_sm) : launch_mixed_t<true, false>(a, spread, s, n_sm);
+  return phase64 ? launch_mixed_t<false, true>(a, spread, s, n_sm) : launch_mixed_t<false, false>(a, spread, s, n_sm);
 }
 
 cudaError_t launch_rb_f64(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl, double* grad,

@@ -173,7 +173,7 @@ static int enqueue_work(Slot* s, const EventEntry* ev, int64_t W, bool grad, int
   cudaError_t err = cudaMemcpyAsync(s->d_theta, s->h_theta, sizeof(double) * kNPar * W, cudaMemcpyHostToDevice,
                                     s->stream);
   if (err != cudaSuccess) return cuda_fail(err, "server copy-in");
-  int rc = run_batch(ev, s->d_theta, W, s->d_logl, grad ? s->d_grad : nullptr, mode, s->stream, s->d_ws);
+  int rc = run_batch(ev, s->d_theta, W, s->d_logl, grad ? s->d_grad : nullptr, mode, s->stream, s->d_ws, nullptr, false);
   if (rc != RB_OK) return rc;
   if ((err = cudaMemcpyAsync(s->h_logl, s->d_logl, sizeof(double) * W, cudaMemcpyDeviceToHost, s->stream)) !=
       cudaSuccess)
