@@ -436,7 +436,9 @@ RB_API const char* rb_strerror(int status);
 RB_API const char* rb_last_error(void);
 /* Tracing: record the CUDA events before_main / after_main (cudaEvent_t, or
  * NULL to stop) on the launch stream immediately before and after the main
- * likelihood kernel of every subsequent batch call (process-wide). */
+ * likelihood kernel of every subsequent batch call (process-wide).  While
+ * they are set, batches run as a set-up kernel and a likelihood kernel (without
+ * them small batches run both in one kernel). */
 RB_API void rb_set_trace_events(void* before_main, void* after_main);
 /* Number of this library's kernel launches on the calling process so far
  * (all entry points, all threads). */

@@ -25,6 +25,8 @@ cudaError_t launch_setup(int mode, const double* theta, int64_t W, const EventCo
                          void* ws, void* tan, bool grad, cudaStream_t s);
 cudaError_t launch_rb_mixed(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl,
                             double* grad, bool phase64, bool spread, cudaStream_t s, int n_sm, const MalaArgs* mala);
+cudaError_t launch_rb_fused(const EventDev& ev, const EventConst& ec, const double* theta, int64_t W, double* logl,
+                            double* grad, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done);
 cudaError_t launch_rb_f64(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl, double* grad,
                           cudaStream_t s, int n_sm, const MalaArgs* mala);
 cudaError_t launch_bin_edges(double f_low, double f_high, double T, int64_t kmin, int64_t N, int B, int64_t* edges,
@@ -783,8 +785,10 @@ static bool host_batch_graph(EventEntry& e, const double* theta, int64_t W, doub
     cudaGetLastError();
     return false;
   }
+  const uint64_t n0 = g_launches.load();
   const int rc = run_batch(&e, theta, W, logl, grad, mode, e.hg_stream, e.hg_ws);
-  count_launches((uint64_t)0 - 2u);  // the capture launched nothing
+  e.hg_launches = g_launches.load() - n0;
+  count_launches((uint64_t)0 - e.hg_launches);  // the capture launched nothing
   err = cudaStreamEndCapture(e.hg_stream, &g);
   cudaGraphExec_t exec = nullptr;
   if (rc == RB_OK && err == cudaSuccess && g) err = cudaGraphInstantiate(&exec, g, 0);
@@ -835,7 +839,7 @@ int rb_loglike_grad_host(rb_event_t ev, const double* theta_host, int64_t W, dou
       if (replay && (err = cudaGraphLaunch(ev->e.hg_exec, s)) != cudaSuccess) return cuda_fail(err, "graph launch");
     }
     if (replay) {
-      rb::count_launches(2);
+      rb::count_launches(ev->e.hg_launches);
       err = cudaStreamSynchronize(s);
       return err == cudaSuccess ? RB_OK : cuda_fail(err, "synchronise");
     }
@@ -1190,6 +1194,18 @@ int run_batch(const EventEntry* e, const double* theta, int64_t W, double* logl,
   if (W == 0) return RB_OK;
   if (!theta || (!logl && !mala)) return set_error(RB_EINVAL, "NULL theta or logl");
   const bool want_grad = grad != nullptr || mala != nullptr;
+  // set-up and likelihood in one launch where the batch allows it (not with
+  // trace events, which bracket the likelihood kernel alone, nor for launches
+  // that share the GPU with others)
+  if (mode == RB_MIXED && spread && !trace_events_set()) {
+    bool done = false;
+    const cudaError_t ferr = launch_rb_fused(e->dev, e->ec, theta, W, logl, grad, s, sm_count(), mala, &done);
+    if (ferr != cudaSuccess) return cuda_fail(ferr, "likelihood kernel");
+    if (done) {
+      count_launches(1);
+      return RB_OK;
+    }
+  }
   const size_t ws_bytes = (mode == RB_MIXED) ? sizeof(WalkerMixed) * W : sizeof(WalkerF64) * W;
   const size_t tan_bytes = !want_grad ? 0 : (mode == RB_FP64 ? sizeof(WalkerTan<double>) : sizeof(WalkerTan<float>)) * W;
   void* buf = scratch;

@@ -80,6 +80,7 @@ struct EventEntry {
   double* hg_grad = nullptr;
   int64_t hg_W = 0;
   int hg_mode = -1;
+  uint64_t hg_launches = 0;
   void* hg_ws = nullptr;             // the captured launches' workspace
   size_t hg_ws_bytes = 0;
   // host-buffer rebuild + batch with everything pinned: the whole call

@@ -30,7 +30,7 @@
 #define RB_DD_CTOR __host__ __device__
 // the longer routines are kept out of line: the set-up kernels run many
 // warps on different code at once and are otherwise instruction-fetch bound
-#define RB_DD_CALL __host__ __device__ __noinline__
+#define RB_DD_CALL static __host__ __device__ __noinline__
 #else
 #define RB_DD inline
 #define RB_DD_CTOR

@@ -39,6 +39,7 @@
 #include <type_traits>
 
 #include "rb_internal.cuh"
+#include "rb_setup_dd.cuh"
 
 namespace rb {
 
@@ -79,9 +80,8 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // set-up record (its constants, WalkerMixed) and tangents, so that the next
 // walker's are fetched while this one runs.
 constexpr int kTanBytes = 384;
-struct __align__(16) WarpSlot {
-  WalkerMixed rec[2];
-  unsigned char tan[2][kTanBytes];
+// what a warp needs besides its walker's record and tangents
+struct __align__(16) WarpWork {
   float red[32];  // the walker's adjoint sums
   // the current walker's constants, each value in both halves of a pair
   // (float-float path): {hi, hi, lo, lo} of dc_k (k < kNBasis), then per
@@ -93,6 +93,22 @@ struct __align__(16) WarpSlot {
   // record expansion (constant over the launch)
   float lane_gmax[32];
 };
+struct __align__(16) WarpSlot {
+  WalkerMixed rec[2];
+  unsigned char tan[2][kTanBytes];
+  WarpWork work;
+};
+// Shared memory of a FUSED block after the tables: its walkers' records and
+// tangents, then the set-up's values, whose space the warps take over.
+struct __align__(16) FusedRecords {
+  WalkerMixed rec[kSetupWalkers];
+  WalkerTan<float> tan[kSetupWalkers];
+};
+constexpr size_t kFusedWork = sizeof(DdSmem) > (kThreads / 32) * sizeof(WarpWork) ? (sizeof(DdSmem) + 15) / 16 * 16
+                                                                               : (kThreads / 32) * sizeof(WarpWork);
+constexpr size_t kFusedBytes = sizeof(FusedRecords) + kFusedWork;
+static_assert(sizeof(FusedRecords) % 16 == 0, "the set-up's values start on a 16-byte boundary");
+static_assert(kThreads >= kDdRoleThreads + kTanWarps * 32, "a FUSED block has a warp for every set-up role");
 static_assert(sizeof(WalkerMixed) % 16 == 0, "record copied in 16-byte pieces");
 static_assert(sizeof(WalkerTan<float>) <= kTanBytes && sizeof(WalkerTan<float>) % 8 == 0, "tangent buffer");
 
@@ -202,6 +218,11 @@ struct LaunchArgs {
   double* logl;
   double* grad;
   MalaArgs mala;     // MALA kernels only
+};
+// the FUSED kernels form the records themselves
+struct FusedArgs : LaunchArgs {
+  const double* theta;  // [W][13]
+  EventConst ec;
 };
 
 // MALA accept/reject for walker w after its log L and d log L / d theta
@@ -434,9 +455,22 @@ __device__ __forceinline__ void det_edge_slot(float2 y, float4 rho, float4 sig, 
 // detectors, a compile-time constant so that the independent chains of the
 // detector pair and the single detector interleave in one instruction stream.
 // ---------------------------------------------------------------------------
-template <int ND, bool GRAD, bool PHASE64, bool MALA = false>
-__global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
+//
+// FUSED: a block of at most kSetupWalkers walkers runs their set-up itself
+// (roles on its first warps, tangents on the next), into shared memory, while
+// the tables are on their way: one launch, no workspace, no records through
+// memory, and no gap between two kernels.  Small batches are bound by the
+// host's launches and by the set-up's latency: 48 walkers, 1 detector, 100 bins, log L
+// 9.6 -> 8.4 us on the GPU and 15.0 -> 11.4 us per eager call; 3 detectors, 500 bins,
+// with the gradient, on the GPU: 64 walkers 16.2 -> 13.1 us, 4096 walkers 34.9 ->
+// 33.8 us.  More walkers per block than lanes (kSetupWalkers) would run the
+// set-up in turns while the FP32 pipe idles: those batches keep the set-up
+// kernel, whose blocks overlap one another.
+template <int ND, bool GRAD, bool PHASE64, bool MALA, bool FUSED>
+__global__ void __launch_bounds__(kThreads)
+    k_rb_mixed(typename std::conditional<FUSED, FusedArgs, LaunchArgs>::type a) {
   static_assert(!MALA || GRAD, "the MALA step needs the gradient");
+  static_assert(!(FUSED && PHASE64), "the FP64-phase path has FP64 records");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const EventDev& ev = a.ev;
   constexpr int D = ND;
@@ -482,12 +516,20 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
   cp_async_commit();
 
   const int lane = threadIdx.x & 31;
-  WarpSlot* slot;  // this warp's slot, after the tables
+  WarpSlot* slot = nullptr;       // this warp's slot, after the tables
+  FusedRecords* fused = nullptr;  // FUSED: the block's records
+  WarpWork* work;
   {
     const size_t tab_bytes = !PHASE64 ? ev.slot32_floats * sizeof(float)
                                       : (size_t)(kNBasis + 1) * Ep * sizeof(double) +
                                             (ev.tab32_floats - ev.edge32_floats) * sizeof(float);
-    slot = reinterpret_cast<WarpSlot*>(smem_raw + tab_bytes) + (threadIdx.x >> 5);
+    if constexpr (FUSED) {
+      fused = reinterpret_cast<FusedRecords*>(smem_raw + tab_bytes);
+      work = reinterpret_cast<WarpWork*>(smem_raw + tab_bytes + sizeof(FusedRecords)) + (threadIdx.x >> 5);
+    } else {
+      slot = reinterpret_cast<WarpSlot*>(smem_raw + tab_bytes) + (threadIdx.x >> 5);
+      work = &slot->work;
+    }
   }
   // detectors 0 and 1 form a pair when D >= 2; an odd detector count leaves
   // detector D - 1 single (bin table layout in EventDev)
@@ -506,8 +548,18 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
   const int64_t nwarps = blockDim.x >> 5;
   const unsigned char* rec_g = static_cast<const unsigned char*>(a.ws);
   const unsigned char* tan_g = static_cast<const unsigned char*>(a.tan);
+  if constexpr (FUSED) {
+    DdSmem& S = *reinterpret_cast<DdSmem*>(fused + 1);
+    const int warp = threadIdx.x >> 5;
+    if (warp < kDdRoleWarps) {
+      setup_absolute_dd(a.theta, w_begin, w_end, a.ec, S);
+      setup_record_dd(ev.ref->dd, a.ec, S, &fused->rec[lane], w_begin + lane < w_end);
+    } else if (GRAD && warp < kDdRoleWarps + 3 + D) {
+      tangent_warp<float>(a.theta, w_end, w_begin, a.ec, fused->tan, warp - kDdRoleWarps);
+    }
+  }
   // the first walker's record and tangents travel with the tables
-  if (warp0 < w_end)
+  if (!FUSED && warp0 < w_end)
     prefetch_walker<GRAD, PHASE64>(slot, 0, PHASE64 ? nullptr : rec_g + sizeof(WalkerMixed) * RB_IDX(warp0, a.W, 101),
                                    GRAD ? tan_g + sizeof(WalkerTan<float>) * RB_IDX(warp0, a.W, 107) : nullptr, lane);
   cp_async_wait_all();
@@ -521,15 +573,17 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
   if (!PHASE64) {
     const int j = lane - kNBasis;
     const int gk = lane < kNBasis ? lane : (j < 3 * D && j % 3 == 0 ? kNBasis : -1);
-    slot->lane_gmax[lane] = gk >= 0 ? ev.gmax[gk] : 0.f;
+    work->lane_gmax[lane] = gk >= 0 ? ev.gmax[gk] : 0.f;
   }
 
   int buf = 0;
   for (int64_t w = warp0; w < w_end; w += nwarps, buf ^= 1) {
-    cp_async_wait_all();  // this walker's record and tangents
-    __syncwarp();         // ... visible to the warp; the previous walker's reads of wc and of buffer buf ^ 1 done
+    if (!FUSED) cp_async_wait_all();  // this walker's record and tangents
+    __syncwarp();  // ... visible to the warp; the previous walker's reads of wc and of buffer buf ^ 1 done
     // ---- per-walker constants (uniform across the warp), in shared memory ----
-    float4* const wc = slot->rec[buf].q;
+    const int64_t wl = FUSED ? RB_IDX(w - w_begin, kSetupWalkers, 101) : 0;
+    WalkerMixed& rec = FUSED ? fused->rec[wl] : slot->rec[buf];
+    float4* const wc = rec.q;
     double dc64[kNBasis];
     double tau64[kMaxDet];
     pv::DetState<float2> P;  // detectors 0, 1: accumulators (constants come from wc)
@@ -537,7 +591,7 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
     int valid;
     unsigned walker_ex = 0;  // float-float path: exponent field of the walker's phase-term bound
     if (!PHASE64) {
-      valid = slot->rec[buf].valid;
+      valid = rec.valid;
 #pragma unroll
       for (int k = 0; k < kNBasis; ++k) dc64[k] = 0.0;
 #pragma unroll
@@ -562,8 +616,8 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
           iv = iu + (d == ds ? 1 : 2);
         }
         const float u = f[iu], v = f[iv];
-        slot->dup[lane] = make_float4(u, u, v, v);
-        mag = fabsf(u) * slot->lane_gmax[lane];
+        work->dup[lane] = make_float4(u, u, v, v);
+        mag = fabsf(u) * work->lane_gmax[lane];
       }
       // the walker's rounding constant m = 1.5 * 2^23 q with q = 2^-20 of a
       // power of two above every phase term (at least 2^-62 turns): then each
@@ -575,7 +629,7 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
       walker_ex = ex;
       if (lane == 0) {
         const float m = __uint_as_float(((ex + 4u) << 23) | 0x400000u);  // 1.5 * 2^(ex - 123)
-        slot->dup[kNBasis + 3 * kMaxDet] = make_float4(m, m, m, m);
+        work->dup[kNBasis + 3 * kMaxDet] = make_float4(m, m, m, m);
       }
     } else {
       float rho[kMaxDet][2], sg[kMaxDet][2];
@@ -601,7 +655,7 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
       }
     }
     __syncwarp();
-    {
+    if (!FUSED) {
       // the next walker's record and tangents, into the other buffer (issued
       // after this walker's shared-memory reads above)
       const int64_t wn = w + nwarps;
@@ -640,7 +694,7 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
     if constexpr (!PHASE64) {
       // slot loop: both halves of every paired value are edges of this walker
       const int NS = ev.n_slots;
-      const float4* const wd = slot->dup;
+      const float4* const wd = work->dup;
       float2 acc = make_float2(0.f, 0.f), acc_lo = acc;
       // the adjoint sums of a lane's two edges in one float each (as pairs,
       // the extra registers spilled)
@@ -798,16 +852,16 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
       const float two_pi = 6.28318530717958648f;
       // the walker's adjoint sums (basis coefficients, then per detector the
       // delay and the prefactor ratio re/im) by one transposed warp sum
-      warp_transposed_sums<kNV>(v, lane, slot->red);
+      warp_transposed_sums<kNV>(v, lane, work->red);
       __syncwarp();
       float ac[kNBasis], at[kMaxDet], ar[kMaxDet][2];
 #pragma unroll
-      for (int k = 0; k < kNBasis; ++k) ac[k] = two_pi * slot->red[k];
+      for (int k = 0; k < kNBasis; ++k) ac[k] = two_pi * work->red[k];
 #pragma unroll
       for (int d = 0; d < kMaxDet; ++d) {
-        at[d] = d < D ? two_pi * slot->red[kNBasis + d] : 0.f;
-        ar[d][0] = d < D ? slot->red[kNBasis + D + d] : 0.f;
-        ar[d][1] = d < D ? slot->red[kNBasis + 2 * D + d] : 0.f;
+        at[d] = d < D ? two_pi * work->red[kNBasis + d] : 0.f;
+        ar[d][0] = d < D ? work->red[kNBasis + D + d] : 0.f;
+        ar[d][1] = d < D ? work->red[kNBasis + 2 * D + d] : 0.f;
       }
       if constexpr (PHASE64) {
         // this path sums gbar conj(E) = gbar_rho: G_d = conj(gbar_rho) rho
@@ -825,7 +879,7 @@ __global__ void __launch_bounds__(kThreads) k_rb_mixed(LaunchArgs a) {
       }
       double g = 0.0;
       if (lane < kNPar) {
-        const WalkerTan<float>& tn = *reinterpret_cast<const WalkerTan<float>*>(slot->tan[buf]);  // prefetched
+        const WalkerTan<float>& tn = FUSED ? fused->tan[wl] : *reinterpret_cast<const WalkerTan<float>*>(slot->tan[buf]);
         g = f2d_int(chain_rule_lanes<D>(lane, ac, at, ar, tn));
       }
       if (MALA) mala_finish(a.mala, w, lane, logl, g);
@@ -988,8 +1042,21 @@ constexpr int kOccSlots = 256;
 static std::mutex g_occ_mu;
 static OccEntry g_occ[kOccSlots];
 static int g_occ_n = 0;
-static const void* g_smem_raised[16];
+constexpr int kSmemRaised = 64;
+static const void* g_smem_raised[kSmemRaised];
 static int g_smem_raised_n = 0;
+
+static size_t smem_optin_max() {
+  static std::once_flag once;
+  static int n = 0;
+  std::call_once(once, [] {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+      n = 0;
+  });
+  return (size_t)n;
+}
 
 static cudaError_t blocks_per_sm(const void* fn, int threads, size_t smem, int* out) {
   std::lock_guard<std::mutex> lk(g_occ_mu);
@@ -1013,7 +1080,7 @@ static cudaError_t blocks_per_sm(const void* fn, int threads, size_t smem, int* 
     if (err == cudaSuccess)
       err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)fa.sharedSizeBytes);
     if (err != cudaSuccess) return err;
-    if (g_smem_raised_n < 16) g_smem_raised[g_smem_raised_n++] = fn;
+    if (g_smem_raised_n < kSmemRaised) g_smem_raised[g_smem_raised_n++] = fn;
   }
   int n = 0;
   err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, smem);
@@ -1025,27 +1092,31 @@ static cudaError_t blocks_per_sm(const void* fn, int threads, size_t smem, int* 
 
 constexpr int64_t kThinWalkers = 4;  // an SM's sub-partitions
 
+// Blocks of a batch of W walkers, at most n_max.  spread: a batch that does not
+// fill the SMs with 16 walkers per block takes more of them, down to one walker
+// per SM sub-partition (the warps of a block share its FP32 pipe; below four
+// walkers nothing is left to share).  GPU time of a call, 3 detectors, 500
+// bins, with the gradient: 64 walkers 24.1 -> 16.2 us, 1024 walkers 24.2 -> 18.4
+// us.  Otherwise (launches that share the GPU with others) the blocks stay
+// dense: fewer SMs are held, for longer.
+static int64_t mixed_grid(int64_t W, bool spread, int n_sm, int64_t n_max) {
+  const int64_t dense = (W * 32 + kThreads - 1) / kThreads;
+  const int64_t thin = spread ? std::min<int64_t>((W + kThinWalkers - 1) / kThinWalkers, n_sm) : 0;
+  return std::min<int64_t>(std::max<int64_t>(dense, thin), n_max);
+}
+
 template <int ND, bool GRAD, bool PHASE64, bool MALA>
 static cudaError_t launch_mixed_nd(const LaunchArgs& a, bool spread, cudaStream_t s, int n_sm) {
   // the kernel copies records in 16-byte and tangents in 8-byte asynchronous copies
   if (reinterpret_cast<uintptr_t>(a.ws) % 16 != 0 || (GRAD && reinterpret_cast<uintptr_t>(a.tan) % 8 != 0))
     return cudaErrorMisalignedAddress;
   const size_t smem = mixed_smem_bytes(a.ev, PHASE64);
-  const void* fn = reinterpret_cast<const void*>(k_rb_mixed<ND, GRAD, PHASE64, MALA>);
+  auto* fn = k_rb_mixed<ND, GRAD, PHASE64, MALA, false>;
   int per_sm = 0;
-  cudaError_t err = blocks_per_sm(fn, kThreads, smem, &per_sm);
+  cudaError_t err = blocks_per_sm(reinterpret_cast<const void*>(fn), kThreads, smem, &per_sm);
   if (err != cudaSuccess) return err;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  // spread: a batch that does not fill the SMs with 16 walkers per block takes
-  // more of them, down to one walker per SM sub-partition (the warps of a block
-  // share its FP32 pipe; below four walkers nothing is left to share).  GPU time
-  // of a call, 3 detectors, 500 bins, with the gradient: 64 walkers 24.1 -> 16.2
-  // us, 1024 walkers 24.2 -> 18.4 us.  Otherwise (launches that share the GPU
-  // with others) the blocks stay dense: fewer SMs are held, for longer.
-  const int64_t dense = (a.W * 32 + kThreads - 1) / kThreads;
-  const int64_t thin = spread ? std::min<int64_t>((a.W + kThinWalkers - 1) / kThinWalkers, n_sm) : 0;
-  const int64_t grid = std::min<int64_t>(std::max<int64_t>(dense, thin), (int64_t)per_sm * n_sm);
-  k_rb_mixed<ND, GRAD, PHASE64, MALA><<<(unsigned)grid, kThreads, smem, s>>>(a);
+  fn<<<(unsigned)mixed_grid(a.W, spread, n_sm, (int64_t)per_sm * n_sm), kThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -1068,6 +1139,49 @@ cudaError_t launch_rb_mixed(const EventDev& ev, const void* ws, const void* tan,
   }
   if (grad) return phase64 ? launch_mixed_t<true, true>(a, spread, s, n_sm) : launch_mixed_t<true, false>(a, spread, s, n_sm);
   return phase64 ? launch_mixed_t<false, true>(a, spread, s, n_sm) : launch_mixed_t<false, false>(a, spread, s, n_sm);
+}
+
+// Set-up and likelihood in one launch, where it applies (*done): every block
+// gets at most kSetupWalkers walkers, and the tables leave room for their
+// records beside them.
+template <int ND, bool GRAD, bool MALA>
+static cudaError_t launch_fused_nd(const FusedArgs& a, cudaStream_t s, int n_sm, bool* done) {
+  auto* fn = k_rb_mixed<ND, GRAD, false, MALA, true>;
+  const size_t smem = a.ev.slot32_floats * sizeof(float) + kFusedBytes;
+  *done = false;
+  if (smem > smem_optin_max()) return cudaSuccess;
+  int per_sm = 0;
+  const cudaError_t err = blocks_per_sm(reinterpret_cast<const void*>(fn), kThreads, smem, &per_sm);
+  if (err != cudaSuccess) return err;
+  if (per_sm < 1) return cudaSuccess;
+  const int64_t grid = mixed_grid(a.W, true, n_sm, (int64_t)per_sm * n_sm);
+  if ((a.W + grid - 1) / grid > kSetupWalkers) return cudaSuccess;
+  fn<<<(unsigned)grid, kThreads, smem, s>>>(a);
+  *done = true;
+  return cudaGetLastError();
+}
+
+template <bool GRAD, bool MALA>
+static cudaError_t launch_fused_t(const FusedArgs& a, cudaStream_t s, int n_sm, bool* done) {
+  switch (a.ev.n_det) {
+    case 1: return launch_fused_nd<1, GRAD, MALA>(a, s, n_sm, done);
+    case 2: return launch_fused_nd<2, GRAD, MALA>(a, s, n_sm, done);
+    case 3: return launch_fused_nd<3, GRAD, MALA>(a, s, n_sm, done);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_rb_fused(const EventDev& ev, const EventConst& ec, const double* theta, int64_t W, double* logl,
+                            double* grad, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done) {
+  FusedArgs a;
+  static_cast<LaunchArgs&>(a) = LaunchArgs{ev, nullptr, nullptr, W, logl, grad, {}};
+  a.theta = theta;
+  a.ec = ec;
+  if (mala) {
+    a.mala = *mala;
+    return launch_fused_t<true, true>(a, s, n_sm, done);
+  }
+  return grad ? launch_fused_t<true, false>(a, s, n_sm, done) : launch_fused_t<false, false>(a, s, n_sm, done);
 }
 
 cudaError_t launch_rb_f64(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl, double* grad,
