@@ -42,6 +42,9 @@ cudaError_t launch_summary(const DataPtrs& in, int64_t kmin, int64_t N, double T
                            cudaStream_t s);
 cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t kmin, int64_t N, double T, int D, int B,
                                   const int64_t* edges, const SummaryOut& so, int n_parts, cudaStream_t s);
+cudaError_t launch_summary_chunk64(const DataPtrs& in, double* h0_out, void* scratch, int64_t kmin, int64_t N, double T, int D,
+                                   int B, const int64_t* edges, const RefValues* ref, const SummaryOut& so, int n_parts,
+                                   cudaStream_t s);
 cudaError_t launch_edge_tables(int64_t kmin, double T, int D, int B, int Ep, int Bp, const int64_t* edges,
                                float* tab32, size_t edge32_floats, double* tab64, double* inv_df, float* slot32,
                                int n_slots, cudaStream_t s);
@@ -50,7 +53,7 @@ size_t chunk_q_bytes(int64_t N);
 cudaError_t launch_strain(const RefValues* src, int64_t kmin, int64_t N, double T, double* h, cudaStream_t s);
 cudaError_t launch_summary_parts(const void* w32, const float* is32, const int* exps, int64_t N, double T, int D, int B,
                                  const int64_t* edges, const RefValues* ref, const void* chunk_q, const void* recs,
-                                 const SummaryOut& so, int p0, int p1, cudaStream_t s);
+                                 const SummaryOut& so, cudaStream_t s);
 cudaError_t launch_ref_dd(const double* theta_ref_dev, const EventConst& ec, RefValues* out, SummarySync* base_reset,
                           cudaStream_t s);
 cudaError_t launch_tangents(const double* theta, int64_t W, const EventConst& ec, void* tan, cudaStream_t s);
@@ -539,7 +542,7 @@ int rb_event_rebuild(rb_event_t ev, const double* theta_ref_host, const double* 
       }
     }
   }
-  return rebuild_event(e, have ? &in : nullptr, mode, s);
+  return rebuild_event(e, have ? &in : nullptr, mode, s, nullptr, theta_ref_host != nullptr);
 }
 
 void rb_set_trace_events(void* before_main, void* after_main) { set_trace_events(before_main, after_main); }
@@ -1062,7 +1065,7 @@ int rb_strain(const double* geom, double gmst, const double* theta_host, double 
 
 namespace rb {
 
-int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t s, const SideSetup* ss) {
+int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t s, const SideSetup* ss, bool new_ref) {
   cudaError_t err;
   DataPtrs in{};
   if (in_opt) {
@@ -1074,6 +1077,12 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     }
   }
   const bool fast = mode != RB_FP64 && e.kmin >= 1024 && e.N <= (int64_t(1) << 30);
+  // FP64 sums with h0 generated: for a theta_ref given with the call from FP64
+  // Taylor chunks; otherwise (the event's creation, or a rebuild behind a change of
+  // theta_ref that kept h0 away) directly at every point, so that a saved event
+  // loads to the bits it has after an FP64 rebuild
+  const bool chunk64 = mode == RB_FP64 && new_ref && !e.h0_valid && e.kmin >= 1024 && e.N <= (int64_t(1) << 30) &&
+                       e.kmin <= (int64_t(1) << 30);
   if (ss && !(fast && mode == RB_MIXED)) return set_error(RB_EINVAL, "overlapped set-up needs the mixed fast rebuild");
   // Both sets of reference values are rebuilt: the float-float set (mixed
   // path, fast summary) and the FP64 set (FP64 paths, FP64 summary).  The
@@ -1144,15 +1153,22 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     }
     e.w32_current = true;
     err = launch_summary_parts(e.d_w32, e.d_is32, e.d_wexp, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref,
-                               e.d_chunkq, ss ? e.d_chunks : nullptr, e.out(), 0, e.n_parts, s);
-  } else if (e.h0_valid) {
+                               e.d_chunkq, ss ? e.d_chunks : nullptr, e.out(), s);
+  } else if (e.h0_valid || chunk64) {
     // FP64 sums from the fiducial waveform stored by the last inline build
     // for this theta_ref: strain, PSD and h0 streamed, no waveform arithmetic;
     // its fixed-point sum starts from zero (a fast build leaves it set)
     if ((err = cudaMemsetAsync(&e.d_sync->base_acc, 0, sizeof(unsigned long long), s)) != cudaSuccess ||
         (err = cudaMemsetAsync(&e.d_sync->overflow, 0, sizeof(unsigned), s)) != cudaSuccess)
       return cuda_fail(err, "zero counters");
-    err = launch_summary_stored(in, e.d_h0, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.out(), e.n_parts, s);
+    if (chunk64) {
+      err = launch_summary_chunk64(in, e.d_h0, e.d_chunks, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref, e.out(),
+                                   e.n_parts, s);
+      e.h0_valid = err == cudaSuccess;
+      ++launches;
+    } else {
+      err = launch_summary_stored(in, e.d_h0, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.out(), e.n_parts, s);
+    }
     e.w32_current = !in_opt && e.w32_resident;
   } else {
     // FP64 waveform generated inline, and stored for the next builds

@@ -425,43 +425,19 @@ __device__ __forceinline__ double rcp_newton(double S) {
   return r;
 }
 
+// Blocks take the parts from the last one down: the bins widen with frequency,
+// so the full parts start first and the short ones fill the gaps at the end.
+__device__ __forceinline__ int part_of_block(int n_parts) { return n_parts - 1 - (int)blockIdx.x; }
+
+// The end of the FP64 builds that take one block per part of a bin: the block's
+// sums of the per-thread sums acc (six per detector, terms over S without the
+// factor 4 df), the parts of a bin added in index order by the last of them to
+// finish, which runs the FP64 epilogue (base log L by the fixed-point sum).
 template <int ND>
-__global__ void __launch_bounds__(kStoredThreads) k_summary_stored(DataPtrs in, const double* __restrict__ h0,
-                                                                   int64_t kmin, int64_t N, double T, int B,
-                                                                   const int64_t* __restrict__ edges, SummaryOut so) {
-  __shared__ double red[6 * ND][kStoredThreads];  // per-thread sums, one row per quantity
-  __shared__ double qsum[6 * kMaxDet];
-  __shared__ double sblock[6 * kMaxDet];
+__device__ __forceinline__ void stored_part_sums(const double (&acc)[ND][6], double inv_T, int pid, const PartDesc& pd, int b, int B, const SummaryOut& so,
+                                                 double (*red)[kStoredThreads], double* qsum, double* sblock) {
   __shared__ bool s_last;
-  const int pid = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
-  const int b = pd.bin;
-  const double fm = 0.5 * (grid_f(kmin, edges[b], T) + grid_f(kmin, edges[b + 1], T));
-  const double inv_T = 1.0 / T;
-  double acc[ND][6];
-#pragma unroll
-  for (int d = 0; d < ND; ++d)
-#pragma unroll
-    for (int j = 0; j < 6; ++j) acc[d][j] = 0.0;
-  // sums of the terms over S; the factor 4 df = 4 / T is applied to the sums
-  for (int64_t k = pd.start + tid; k < pd.end; k += kStoredThreads) {
-    const double f = (double)(kmin + k) * inv_T;
-    const double df = f - fm;
-#pragma unroll
-    for (int d = 0; d < ND; ++d) {
-      const double2 dv = __ldcs(reinterpret_cast<const double2*>(in.data[d]) + RB_IDX(k, N, 222));
-      const double2 hv = __ldcs(reinterpret_cast<const double2*>(h0) + (size_t)d * N + RB_IDX(k, N, 222));
-      const double w = rcp_newton(__ldcs(in.psd[d] + k));
-      const double hr = hv.x, hi = hv.y, dr = dv.x, di = dv.y;
-      const double xr = dr * hr + di * hi, xi = di * hr - dr * hi, hh = hr * hr + hi * hi;
-      acc[d][0] += w * xr;
-      acc[d][1] += w * xi;
-      acc[d][2] += w * xr * df;
-      acc[d][3] += w * xi * df;
-      acc[d][4] += w * hh;
-      acc[d][5] += w * hh * df;
-    }
-  }
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   // block sums in a fixed order: warp w takes quantities w, w + 4, ...; each
   // lane adds the 4 threads l, l + 32, l + 64, l + 96, then a shuffle tree
 #pragma unroll
@@ -503,10 +479,344 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_stored(DataPtrs in, 
   summary_epilogue(so, b, 0, ND, B, ND, sblock, nullptr, false, (unsigned)B, so.inv_df[b], true);
 }
 
+template <int ND>
+__global__ void __launch_bounds__(kStoredThreads) k_summary_stored(DataPtrs in, const double* __restrict__ h0,
+                                                                   int64_t kmin, int64_t N, double T, int B,
+                                                                   const int64_t* __restrict__ edges, SummaryOut so) {
+  __shared__ double red[6 * ND][kStoredThreads];  // per-thread sums, one row per quantity
+  __shared__ double qsum[6 * kMaxDet];
+  __shared__ double sblock[6 * kMaxDet];
+  const int pid = blockIdx.x, tid = threadIdx.x;
+  const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
+  const int b = pd.bin;
+  const double fm = 0.5 * (grid_f(kmin, edges[b], T) + grid_f(kmin, edges[b + 1], T));
+  const double inv_T = 1.0 / T;
+  double acc[ND][6];
+#pragma unroll
+  for (int d = 0; d < ND; ++d)
+#pragma unroll
+    for (int j = 0; j < 6; ++j) acc[d][j] = 0.0;
+  // sums of the terms over S; the factor 4 df = 4 / T is applied to the sums
+  for (int64_t k = pd.start + tid; k < pd.end; k += kStoredThreads) {
+    const double f = (double)(kmin + k) * inv_T;
+    const double df = f - fm;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      const double2 dv = __ldcs(reinterpret_cast<const double2*>(in.data[d]) + RB_IDX(k, N, 222));
+      const double2 hv = __ldcs(reinterpret_cast<const double2*>(h0) + (size_t)d * N + RB_IDX(k, N, 222));
+      const double w = rcp_newton(__ldcs(in.psd[d] + k));
+      const double hr = hv.x, hi = hv.y, dr = dv.x, di = dv.y;
+      const double xr = dr * hr + di * hi, xi = di * hr - dr * hi, hh = hr * hr + hi * hi;
+      acc[d][0] += w * xr;
+      acc[d][1] += w * xi;
+      acc[d][2] += w * xr * df;
+      acc[d][3] += w * xi * df;
+      acc[d][4] += w * hh;
+      acc[d][5] += w * hh * df;
+    }
+  }
+  stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, red, qsum, sblock);
+}
+
 cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t kmin, int64_t N, double T, int D, int B,
                                   const int64_t* edges, const SummaryOut& so, int n_parts, cudaStream_t s) {
   auto kf = D == 1 ? k_summary_stored<1> : D == 2 ? k_summary_stored<2> : k_summary_stored<3>;
   kf<<<(unsigned)n_parts, kStoredThreads, 0, s>>>(in, h0, kmin, N, T, B, edges, so);
+  return cudaGetLastError();
+}
+
+// ===========================================================================
+// FP64 build with a new fiducial point: h0 from FP64 Taylor chunks.
+//
+// k_summary evaluates h0_d at every grid point and detector from scratch (log, cbrt,
+// ten basis terms, sincos: ~500 FP64 operations per point with three
+// detectors, and an FP64 warp instruction holds its SM sub-partition's FP64
+// unit for ~65 clocks).  Here the phase in turns is expanded about the centre
+// of every 32-point chunk, as in the fast build but in FP64 and to order 9,
+// and the detectors share the point's sine and cosine:
+//   h_d(f) = K_d f^-7/6 exp(-2 pi i [x(f) + f tau_d]),  f = f_c (1 + j u),
+//   exp(-2 pi i f tau_d) = exp(-2 pi i f_c tau_d) exp(-2 pi i j df tau_d),
+// the first factor (times K_d f_c^-7/6) from the chunk's record, the second from
+// a 32-entry table.  ~115 FP64 operations per point: 519,169 points, 3 detectors,
+// 1000 bins: k_summary 605 us, this kernel 161 us (FP64 pipe 84 % busy) and the
+// records 19 us; the whole rebuild call 615 -> 194 us.  Errors against 80-bit
+// sums (2-norm): A0 8.2e-13 (k_summary 8.3e-13), A1 5.5e-13 (5.5e-13), B0, B1 below 2.5e-15.  A record keeps the orders
+// that reach 2^-48 turns at the chunk's ends (up to 9 of them); X_0, up to
+// thousands of turns, is reduced to [-1/2, 1/2] before it is rounded, so the phase's
+// error stays that of the basis functions, as in k_summary.
+// Needs kmin >= 1024 (|j u| <= 1/64: order 10 is below 2^-46 turns).  The records
+// take the place of the rebuild + batch step's (128 B per chunk).
+// ===========================================================================
+constexpr int kOrd64 = 9;
+constexpr int kAmp64 = 9;  // binomial orders of (1 + j u)^-7/6: (1/64)^10 < 2^-53
+struct __align__(16) ChunkRec64 {
+  double X[kOrd64 + 1];  // phase in turns, X[0] reduced, zero beyond the orders kept
+  double G[kMaxDet][2];  // K_d f_c^-7/6 exp(-2 pi i f_c tau_d)
+};
+
+struct TaylorTables64 {
+  double alpha[kNBasis][kOrd64 + 1];  // binom(p_k, n); ln(1+x) series for k = 4, 6 (see make_taylor_tables)
+  double beta6[kOrd64 + 1];
+};
+struct AmpSeries64 {
+  double c[kAmp64 + 1];  // binom(-7/6, n)
+};
+
+__device__ __forceinline__ void two_sum64(double a, double b, double& s, double& e) {  // Knuth
+  s = a + b;
+  const double bb = s - a;
+  e = (a - (s - bb)) + (b - bb);
+}
+
+// One thread per chunk; the last block forms the offset table
+// etab[d][j] = exp(-2 pi i (j - 16) df tau_d).
+__global__ void __launch_bounds__(64) k_chunk64(const RefValues* __restrict__ ref, int64_t kmin, double T, int n_chunks, int D,
+                                                TaylorTables64 tt, ChunkRec64* __restrict__ recs,
+                                                double2* __restrict__ etab) {
+  const Values& v = ref->v;
+  if (blockIdx.x == gridDim.x - 1) {
+    for (int i = threadIdx.x; i < D * kChunk; i += blockDim.x) {
+      double s, c;
+      sincospi(2.0 * (((double)(i % kChunk - kChunk / 2) / T) * v.tau[i / kChunk]), &s, &c);
+      etab[i] = make_double2(c, -s);
+    }
+    return;
+  }
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= n_chunks) return;
+  const double nc = (double)(kmin + (int64_t)c * kChunk + kChunk / 2), fc = nc / T, u = 1.0 / nc;
+  const double cf = cbrt(fc), lf = log(fc), icf = 1.0 / cf, icf2 = icf * icf;
+  const double P[kNBasis] = {icf2 * icf2 * icf, 1.0 / fc, icf2, icf, 1.0, cf, cf, cf * cf, fc * cf * cf, fc * fc * cf};
+  ChunkRec64& r = recs[c];
+  // X_0 = [Phi0 + sum_k c_k g_k(f_c)] / 2 pi: the two largest terms (up to ~1e4 rad)
+  // added last, in double-double, and the quotient rounded after the whole turns go
+  double cp[kNBasis], sh = v.phi0, sl = 0.0;
+#pragma unroll
+  for (int k = kNBasis - 1; k >= 0; --k) {
+    cp[k] = v.c[k] * P[k];
+    const double g = k == 4 ? lf : k == 6 ? P[k] * lf : P[k];
+    if (k >= 2) {
+      sh = fma(v.c[k], g, sh);
+    } else {
+      const double p = v.c[k] * g, pe = fma(v.c[k], g, -p);
+      double e;
+      two_sum64(sh, p, sh, e);
+      sl += e + pe;
+    }
+  }
+  const double inv2pi = 1.0 / kTwoPi;
+  constexpr double inv2pi_lo = -9.839338337591243e-18;  // 1/2pi - fl(1/2pi)
+  const double xh = sh * inv2pi, xl = fma(sh, inv2pi, -xh) + (sh * inv2pi_lo + sl * inv2pi);
+  r.X[0] = (xh - rint(xh)) + xl;
+  // orders kept: |X_n j^n| <= 6 sum_k |c_k P_k| (1 + |ln f_c|) / 2 pi (16 u)^n
+  // (every |alpha_kn|, |beta_n| <= 5.2 up to order 10), below 2^-48 turns beyond n_ord
+  double bound = 0.0;
+#pragma unroll
+  for (int k = 0; k < kNBasis; ++k) bound += fabs(cp[k]);
+  bound *= (1.0 + fabs(lf)) * (16.0 * u) * (16.0 * u);
+  int n_ord = 1;
+  while (bound >= 3.552713678800501e-15 && n_ord < kOrd64) {
+    bound *= 16.0 * u;
+    ++n_ord;
+  }
+  double un = u * inv2pi;
+  for (int n = n_ord + 1; n <= kOrd64; ++n) r.X[n] = 0.0;
+  for (int n = 1; n <= n_ord; ++n) {
+    double x = 0.0;
+#pragma unroll
+    for (int k = 0; k < kNBasis; ++k) x = fma(cp[k], k == 6 ? fma(tt.beta6[n], lf, tt.alpha[k][n]) : tt.alpha[k][n], x);
+    r.X[n] = x * un;
+    un *= u;
+  }
+  const double kamp = 8.035028173395984e-06 / kMpcS;
+#pragma unroll
+  for (int d = 0; d < kMaxDet; ++d) {
+    if (d >= D) {
+      r.G[d][0] = r.G[d][1] = 0.0;
+      continue;
+    }
+    double s, co;
+    const double y = fc * v.tau[d];
+    sincospi(2.0 * (y - rint(y)), &s, &co);
+    const double a = kamp * v.amp * (sqrt(icf) / fc), Kr = a * v.P64[d][0], Ki = a * v.P64[d][1];
+    r.G[d][0] = Kr * co + Ki * s;  // K exp(-2 pi i y)
+    r.G[d][1] = Ki * co - Kr * s;
+  }
+}
+
+// Integer -> double, exactly, by one FP64 addition (the conversion instruction
+// issues on the FP64 pipe too, and the 64-bit one more than once): 1.5 2^52 + i
+// put together with integer operations.
+__device__ __forceinline__ double small_int_double(int i) {
+  return __hiloint2double(0x43380000 + (i >> 31), i) - 6755399441055744.0;
+}
+
+// exp(-2 pi i x): x reduced to a quarter turn, r in [-1/8, 1/8], and the
+// Taylor series of sine and cosine of 2 pi r (|2 pi r| <= pi/4: the first
+// dropped terms are below 2^-54).  20 FP64 operations; the quadrant is applied with
+// integer selects.
+__device__ __forceinline__ double2 cis_neg_turns64(double x) {
+  const double magic = 6755399441055744.0;  // 1.5 * 2^52
+  const double t = fma(x, 4.0, magic);
+  const int q = __double2loint(t);
+  const double r = fma(t - magic, -0.25, x);
+  const double w = r * r;
+  double ps = -0.7181223017785006;       // -(2 pi)^15 / 15!
+  ps = fma(ps, w, 3.819952584848282);   // (2 pi)^13 / 13!
+  ps = fma(ps, w, -15.09464257682299);  // -(2 pi)^11 / 11!
+  ps = fma(ps, w, 42.058693944897655);   // (2 pi)^9 / 9!
+  ps = fma(ps, w, -76.70585975306139);   // -(2 pi)^7 / 7!
+  ps = fma(ps, w, 81.60524927607506);    // (2 pi)^5 / 5!
+  ps = fma(ps, w, -41.34170224039976);  // -(2 pi)^3 / 3!
+  ps = fma(ps, w, 6.283185307179586);
+  const double sn = r * ps;
+  double pc = 0.28200596845579123;       // (2 pi)^16 / 16!
+  pc = fma(pc, w, -1.714390711088672);  // -(2 pi)^14 / 14!
+  pc = fma(pc, w, 7.903536371318469);    // (2 pi)^12 / 12!
+  pc = fma(pc, w, -26.4262567833744);   // -(2 pi)^10 / 10!
+  pc = fma(pc, w, 60.24464137187666);   // (2 pi)^8 / 8!
+  pc = fma(pc, w, -85.45681720669373);   // -(2 pi)^6 / 6!
+  pc = fma(pc, w, 64.9393940226683);    // (2 pi)^4 / 4!
+  pc = fma(pc, w, -19.739208802178716);  // -(2 pi)^2 / 2
+  const double cs = fma(pc, w, 1.0);
+  // theta = 2 pi r + q pi/2: (cos theta, -sin theta)
+  const double a = (q & 1) ? sn : cs, b = (q & 1) ? cs : sn;
+  const unsigned fa = ((unsigned)(q + 1) & 2u) << 30, fb = ((unsigned)~q & 2u) << 30;  // signs: - for q = 1, 2; - for q = 0, 1
+  return make_double2(__hiloint2double(__double2hiint(a) ^ (int)fa, __double2loint(a)),
+                      __hiloint2double(__double2hiint(b) ^ (int)fb, __double2loint(b)));
+}
+
+// One block per part of a bin, all detectors, as k_summary_stored; h0 goes to
+// h0_out for the builds that follow.
+template <int ND>
+__global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in, double* __restrict__ h0_out, int64_t kmin,
+                                                                    int64_t N, double T, int B,
+                                                                    const int64_t* __restrict__ edges,
+                                                                    const ChunkRec64* __restrict__ recs,
+                                                                    const double2* __restrict__ etab, AmpSeries64 as,
+                                                                    SummaryOut so) {
+  constexpr int kRecDoubles = sizeof(ChunkRec64) / sizeof(double);
+  constexpr int kRecs = kPartPoints / kChunk + 1;  // chunk records a part can touch
+  __shared__ double red[6 * ND][kStoredThreads];
+  __shared__ double qsum[6 * kMaxDet];
+  __shared__ double sblock[6 * kMaxDet];
+  __shared__ ChunkRec64 srec[kRecs];
+  __shared__ double su[kRecs], sg2[ND][kRecs];  // u and |G_d|^2 of the part's chunks
+  __shared__ int sord[kRecs], samp[kRecs];      // orders of the phase and of the amplitude series
+  __shared__ double2 se[ND * kChunk];
+  const int pid = part_of_block(so.n_parts), tid = threadIdx.x;
+  const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
+  const int b = pd.bin, c0 = pd.start / kChunk, nrec = (pd.end - 1) / kChunk - c0 + 1;
+  {
+    const double* src = reinterpret_cast<const double*>(recs + c0);
+    double* dst = reinterpret_cast<double*>(srec);
+    for (int i = tid; i < nrec * kRecDoubles; i += kStoredThreads) dst[RB_IDX(i, kRecs * kRecDoubles, 204)] = __ldg(src + i);
+    for (int i = tid; i < ND * kChunk; i += kStoredThreads) se[i] = etab[i];
+  }
+  const int64_t e0 = edges[b], e1 = edges[b + 1];
+  const double inv_T = 1.0 / T, half_df = 0.5 * inv_T;
+  double acc[ND][6];
+#pragma unroll
+  for (int d = 0; d < ND; ++d)
+#pragma unroll
+    for (int j = 0; j < 6; ++j) acc[d][j] = 0.0;
+  __syncthreads();
+  if (tid < nrec) {
+    const int nc = (int)kmin + (c0 + tid) * kChunk + kChunk / 2;
+    su[tid] = 1.0 / (double)nc;
+    int n = kOrd64;
+    while (n > 1 && __double_as_longlong(srec[tid].X[n]) == 0) --n;
+    sord[tid] = n;
+    // binomial orders of the amplitude: (16 u)^(n + 1) below 2^-53
+    const float u16 = 16.f / (float)nc;
+    int m = 2;
+    for (float t = u16 * u16 * u16; t >= 1.1e-16f && m < kAmp64; t *= u16) ++m;
+    samp[tid] = m;
+  } else if (tid >= 32 && tid < 32 + nrec) {
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      const double gr = srec[tid - 32].G[d][0], gi = srec[tid - 32].G[d][1];
+      sg2[d][tid - 32] = gr * gr + gi * gi;
+    }
+  }
+  __syncthreads();
+  for (int64_t k = pd.start + tid; k < pd.end; k += kStoredThreads) {
+    double2 dv[ND];
+    double S[ND];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      dv[d] = __ldcs(reinterpret_cast<const double2*>(in.data[d]) + RB_IDX(k, N, 222));
+      S[d] = __ldcs(in.psd[d] + k);
+    }
+    const int ci = RB_IDX((int)(k / kChunk) - c0, kRecs, 203), jj = (int)(k % kChunk);
+    const ChunkRec64& r = srec[ci];
+    const double j = small_int_double(jj - kChunk / 2);
+    double x = 0.0;
+    for (int n = sord[ci]; n >= 0; --n) x = fma(x, j, r.X[n]);
+    const double2 z = cis_neg_turns64(x);
+    const double ju = j * su[ci];
+    double a = as.c[samp[ci]];
+    for (int n = samp[ci] - 1; n >= 0; --n) a = fma(a, ju, as.c[n]);  // (1 + j u)^-7/6
+    const double zr = a * z.x, zi = a * z.y, a2 = a * a;
+    const double df = small_int_double((int)(2 * k - e0 - e1)) * half_df;  // f - f_m
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+      const double2 e = se[d * kChunk + jj];
+      const double Fr = r.G[d][0] * e.x - r.G[d][1] * e.y, Fi = r.G[d][0] * e.y + r.G[d][1] * e.x;
+      const double hr = zr * Fr - zi * Fi, hi = zr * Fi + zi * Fr;
+      __stcs(reinterpret_cast<double2*>(h0_out) + (size_t)d * N + k, make_double2(hr, hi));
+      const double w = rcp_newton(S[d]);
+      const double xr = w * (dv[d].x * hr + dv[d].y * hi), xi = w * (dv[d].y * hr - dv[d].x * hi), hh = w * (a2 * sg2[d][ci]);
+      acc[d][0] += xr;
+      acc[d][1] += xi;
+      acc[d][2] += xr * df;
+      acc[d][3] += xi * df;
+      acc[d][4] += hh;
+      acc[d][5] += hh * df;
+    }
+  }
+  stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, red, qsum, sblock);
+}
+
+cudaError_t launch_summary_chunk64(const DataPtrs& in, double* h0_out, void* scratch, int64_t kmin, int64_t N, double T, int D,
+                                   int B, const int64_t* edges, const RefValues* ref, const SummaryOut& so, int n_parts,
+                                   cudaStream_t s) {
+  struct Tables {
+    TaylorTables64 tt;
+    AmpSeries64 as;
+  };
+  static const Tables t = [] {
+    Tables r{};
+    const double p[kNBasis] = {-5.0 / 3.0, -1.0, -2.0 / 3.0, -1.0 / 3.0, 0.0, 1.0 / 3.0, 1.0 / 3.0, 2.0 / 3.0, 5.0 / 3.0, 7.0 / 3.0};
+    for (int k = 0; k < kNBasis; ++k) {
+      double b = 1.0;
+      for (int n = 0; n <= kOrd64; ++n) {
+        r.tt.alpha[k][n] = b;
+        b *= (p[k] - n) / (n + 1);
+      }
+    }
+    for (int n = 0; n <= kOrd64; ++n) {
+      r.tt.beta6[n] = r.tt.alpha[6][n];                               // f^1/3 (ln f_c + ln(1 + j u))
+      r.tt.alpha[4][n] = n == 0 ? 0.0 : ((n % 2) ? 1.0 : -1.0) / n;  // ln(1 + j u)
+    }
+    for (int n = 0; n <= kOrd64; ++n) {
+      double c = 0.0;
+      for (int m = 1; m <= n; ++m) c += r.tt.beta6[n - m] * (((m % 2) ? 1.0 : -1.0) / m);
+      r.tt.alpha[6][n] = c;
+    }
+    double b = 1.0;
+    for (int n = 0; n <= kAmp64; ++n) {
+      r.as.c[n] = b;
+      b *= (-7.0 / 6.0 - n) / (n + 1);
+    }
+    return r;
+  }();
+  const int nc = (int)((N + kChunk - 1) / kChunk);
+  ChunkRec64* recs = static_cast<ChunkRec64*>(scratch);
+  double2* etab = reinterpret_cast<double2*>(recs + nc);
+  k_chunk64<<<(unsigned)((nc + 63) / 64 + 1), 64, 0, s>>>(ref, kmin, T, nc, D, t.tt, recs, etab);
+  auto kf = D == 1 ? k_summary_chunk64<1> : D == 2 ? k_summary_chunk64<2> : k_summary_chunk64<3>;
+  kf<<<(unsigned)n_parts, kStoredThreads, 0, s>>>(in, h0_out, kmin, N, T, B, edges, recs, etab, t.as, so);
   return cudaGetLastError();
 }
 
@@ -815,7 +1125,7 @@ template <int ND, bool INBLOCK>
 __global__ void __launch_bounds__(kSumFastThreads, INBLOCK ? 6 : 8)
     k_summary_fast(const float2* __restrict__ w32, const float* __restrict__ is32, const int* __restrict__ exps,
                    int N, const float* __restrict__ q, double T, float invT_hi, float invT_lo, int B, int D,
-                   const int64_t* __restrict__ edges, const RefValues* __restrict__ ref, SummaryOut so, int p_off) {
+                   const int64_t* __restrict__ edges, const RefValues* __restrict__ ref, SummaryOut so) {
   __shared__ __align__(16) float srec[kPartRecs * kRec];
   // exp(2 pi i j df tau_d), indexed by k mod 32: detectors 0 and 1 as
   // {re_0, re_1, im_0, im_1}, the single detector D-1 as {re, im}
@@ -828,7 +1138,7 @@ __global__ void __launch_bounds__(kSumFastThreads, INBLOCK ? 6 : 8)
   __shared__ double scale[kMaxDet][4];
   __shared__ double s_inv_df;
   __shared__ bool s_last;
-  const int pid = (int)blockIdx.x + p_off;  // this block's part
+  const int pid = blockIdx.x;
   const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
   const int b = pd.bin;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1080,7 +1390,11 @@ static TaylorTables make_taylor_tables() {
 
 int64_t n_chunks_of(int64_t N) { return (N + kChunk - 1) / kChunk; }
 size_t chunk_q_bytes(int64_t N) { return sizeof(float) * 128 * (size_t)n_chunks_of(N); }
-size_t chunk_coef_bytes(int64_t N) { return sizeof(float) * kRec * (size_t)n_chunks_of(N); }
+// Chunk records of one build: k_chunk_coef's, or k_chunk64's and its offset table.
+static_assert(sizeof(ChunkRec64) == sizeof(float) * kRec, "the FP64 records take the place of the float ones");
+size_t chunk_coef_bytes(int64_t N) {
+  return sizeof(float) * kRec * (size_t)n_chunks_of(N) + sizeof(double2) * kMaxDet * kChunk;
+}
 
 cudaError_t launch_chunk_coef(int64_t N, int D, const RefValues* ref, const void* cq, void* chunk_coef, cudaStream_t s) {
   const int nc = (int)n_chunks_of(N);
@@ -1115,16 +1429,15 @@ cudaError_t launch_data32(const DataPtrs& in, int64_t N, int D, void* w32, float
 // from the chunk matrices chunk_q.
 cudaError_t launch_summary_parts(const void* w32, const float* is32, const int* exps, int64_t N, double T, int D, int B,
                                  const int64_t* edges, const RefValues* ref, const void* chunk_q, const void* recs,
-                                 const SummaryOut& so, int p0, int p1, cudaStream_t s) {
-  if (p0 < 0 || p1 <= p0) return cudaErrorInvalidValue;
+                                 const SummaryOut& so, cudaStream_t s) {
   const double invT = 1.0 / T;
   const float ih = (float)invT, il = (float)(invT - (double)ih);
   const bool inblock = recs == nullptr;
   auto kf = inblock ? (D == 1 ? k_summary_fast<1, true> : D == 2 ? k_summary_fast<2, true> : k_summary_fast<3, true>)
                     : (D == 1 ? k_summary_fast<1, false> : D == 2 ? k_summary_fast<2, false> : k_summary_fast<3, false>);
-  kf<<<(unsigned)(p1 - p0), kSumFastThreads, 0, s>>>(static_cast<const float2*>(w32), is32, exps, (int)N,
+  kf<<<(unsigned)so.n_parts, kSumFastThreads, 0, s>>>(static_cast<const float2*>(w32), is32, exps, (int)N,
                                                       static_cast<const float*>(inblock ? chunk_q : recs), T, ih, il, B,
-                                                      D, edges, ref, so, p0);
+                                                      D, edges, ref, so);
   return cudaGetLastError();
 }
 
