@@ -15,20 +15,27 @@
 // coefficients are the walker's c_k / 2pi contracted with the event's chunk
 // matrices, and the delay enters as exp(2 pi i f_c tau_d) exp(2 pi i j df tau_d).
 //
-// Mapping: a block of 8 warps owns 8 walkers (one per warp) and one slice of
-// the grid (blockIdx.y), which it walks in segments of 32 chunks (1024
-// points); the number of slices is picked so the grid fills whole waves.  Per
-// segment the block stages the chunk matrices and the FP32 data copy times
-// f^-7/6 in shared memory, the data transposed (read once for the 8 walkers;
-// the event's data stay in L2).  Lane c of a warp forms its walker's Taylor
-// coefficients and chunk factors exp(2 pi i f_c tau_d) for chunk c, keeps them
-// in registers and walks the chunk's 32 points; the offset factors
-// exp(2 pi i (j - 16) df tau_d), the same for all lanes at a given offset j,
-// come from a per-warp table (broadcast loads), and the chunk factor is
-// applied once to the chunk's sum.  Per point: the phase polynomial, one
-// sin/cos, and per detector the offset factor times the phasor times the
-// data.  Per-lane sums are FP32 per chunk, accumulated in float pairs; the
-// warp sum and the final combination are FP64.
+// Mapping: a block of 8 warps takes 8 walkers (one per warp) and a group of
+// segments of 64 chunks (2048 points) at a time; the (walkers, group) pairs are
+// dealt to one wave of blocks in equal contiguous shares.  Per segment the block stages the chunk matrices and the FP32 data
+// copy times f^-7/6 in shared memory, the data transposed (read once for the 8
+// walkers; the event's data stay in L2).  Lane l of a warp forms its walker's
+// Taylor coefficients for chunks l and l + 32 and walks their 32 points side by
+// side, the two chunks as the halves of paired FP32 values; the offset factors
+// exp(2 pi i (j - 16) df tau_d), the same for all chunks at a given offset j,
+// come from a per-warp table (broadcast loads), and the chunk factors
+// exp(2 pi i f_c tau_d) are applied once to the chunk's sums.  Per point: the
+// phase polynomial, one sin/cos, and per detector the offset factor times the
+// phasor times the data.  Per-lane sums are FP32 per chunk, accumulated in float
+// pairs over a group of segments, at whose end the warp's lanes are added (a
+// fixed tree of float pairs); the groups are added in FP64.  The groups depend
+// on the grid alone, so a walker's result does not depend on the batch.
+//
+// Bound: the FP32 pipe (71 % busy, 51 % of the issue slots; ~80 operations per
+// point and walker with 3 detectors, and the chunk coefficients).  One chunk per lane in scalar FP32
+// (detectors 0 and 1 paired), in waves of slices, issued 119 warp instructions
+// per 32 points (71 % of the slots, pipe 63 %) against 72 now.  512 walkers, 260
+// k points, 3 detectors: call 588 -> 513 us; 7 walkers 83 -> 36 us.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -42,247 +49,291 @@ namespace rb {
 
 constexpr int kFullWarps = 8;
 constexpr int kFullThreads = kFullWarps * 32;
-constexpr int kSegC = 32;                 // chunks per segment
+constexpr int kSegC = 64;                 // chunks per segment, two per lane
 constexpr int kSegP = kSegC * kChunk;     // points per segment
-constexpr int kWtRow = kSegC + 1;       // transposed data row (padded: conflict-free stores)
-constexpr int kQPad = kQRow + 1;        // staged chunk-matrix row (padded: lane c reads row c without conflicts)
-constexpr size_t kFullSmem = sizeof(float) * (kSegC * kQPad + 4) + (sizeof(float4) + sizeof(float2)) * kChunk * kWtRow +
-                             (sizeof(float4) + sizeof(float2)) * kFullWarps * kChunk;
+constexpr int kWtRow = kSegC / 2 + 1;     // transposed data row (padded: conflict-free stores)
+constexpr int kQPad = kQRow + 4;          // staged chunk-matrix row (padded: 16-byte loads of row l by lane l without conflicts)
+constexpr int full_smem(int nd) {
+  return (int)(sizeof(float4) * (nd * kChunk * kWtRow + nd * kFullWarps * kChunk + 2 * kChunk) + sizeof(float) * kSegC * kQPad);
+}
 
-// Per slice and walker: the slice's part of Z_d (complex, 3 detectors) as
-// FP64 in zout[slice][w][6].  ND = number of detectors.
+// Segments per group: up to 64 groups.
+constexpr int kGroups = 64;
+__host__ __device__ constexpr int group_segments(int n_seg) { return (n_seg + kGroups - 1) / kGroups; }
+
+// One level of a transposed warp sum of float pairs: lanes whose bit o is clear
+// keep values [0, M) and send [M, N), the others keep [M, N) (zero beyond N)
+// and send [0, M); each adds what its partner sent (two-sum of the high parts).
+template <int N, int M>
+__device__ __forceinline__ void ff_level(const f2x (&in)[N], f2x (&out)[M], int lane, int o) {
+  const bool up = (lane & o) != 0;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const f2x lo = in[i], hi = (M + i < N) ? in[M + i] : f2x{0.f, 0.f};
+    const f2x keep = up ? hi : lo, send = up ? lo : hi;
+    const float bh = __shfl_xor_sync(0xffffffffu, send.hi, o), bl = __shfl_xor_sync(0xffffffffu, send.lo, o);
+    out[i] = keep;
+    f2x_add(out[i].hi, out[i].lo, bh);
+    out[i].lo = __fadd_rn(out[i].lo, bl);
+  }
+}
+
+// Per group of segments and walker: the group's part of Z_d (complex, 3
+// detectors) as FP64 in zout[group][w][6].  ND = number of detectors.
 template <int ND>
-__global__ void __launch_bounds__(kFullThreads) k_full_z(const float2* __restrict__ w32, int N,
-                                                        const float* __restrict__ q, int n_chunks,
-                                                        const WalkerAbs* __restrict__ wabs, int64_t W,
-                                                        float invT_hi, float invT_lo, int seg_per_slice,
-                                                        double* __restrict__ zout) {
-  // dynamic shared memory: the segment's chunk matrices; its data times
-  // f^-7/6 transposed, for point c * 32 + j of the segment at [j][c] --
-  // detectors 0 and 1 as {re_0, re_1, im_0, im_1} (wp), the single detector
-  // D-1 as {re, im} (ws); and per warp the walker's offset factors
-  // exp(2 pi i (j - 16) df tau_d) in the same two forms (tp, ts)
+__global__ void __launch_bounds__(kFullThreads, 2) k_full_z(const float2* __restrict__ w32, int N,
+                                                           const float* __restrict__ q, int n_chunks,
+                                                           const WalkerAbs* __restrict__ wabs, int64_t W,
+                                                           float invT_hi, float invT_lo,
+                                                           double* __restrict__ zout) {
+  // dynamic shared memory: the segment's data times f^-7/6, transposed: for
+  // detector d and offset j, [d][j][l] holds {re, re', im, im'} of chunks l and
+  // l + 32 (wt); per warp the walker's offset factors exp(2 pi i (j - 16) df
+  // tau_d) as {re, re, im, im} (tp[warp][j][d]); the offsets' powers {j, j, j^2,
+  // j^2}, {j^3, j^3, 0, 0} of j - 16 (jt); the segment's chunk matrices (qs)
   extern __shared__ __align__(16) unsigned char smem_full[];
-  float* qs = reinterpret_cast<float*>(smem_full);
-  float4 (*wp)[kWtRow] = reinterpret_cast<float4 (*)[kWtRow]>(qs + kSegC * kQPad + 4 - (kSegC * kQPad) % 4);
-  float2 (*ws)[kWtRow] = reinterpret_cast<float2 (*)[kWtRow]>(wp + kChunk);
-  float4 (*tp)[kChunk] = reinterpret_cast<float4 (*)[kChunk]>(ws + kChunk);
-  float2 (*ts)[kChunk] = reinterpret_cast<float2 (*)[kChunk]>(tp + kFullWarps);
-  constexpr bool kPair = ND >= 2;
-  constexpr int kSingle = (ND & 1) ? ND - 1 : -1;
-  constexpr int D = ND;
+  float4 (*wt)[kChunk][kWtRow] = reinterpret_cast<float4 (*)[kChunk][kWtRow]>(smem_full);
+  float4 (*tp)[kChunk][ND] = reinterpret_cast<float4 (*)[kChunk][ND]>(wt + ND);
+  float4 (*jt)[2] = reinterpret_cast<float4 (*)[2]>(tp + kFullWarps);
+  float* qs = reinterpret_cast<float*>(jt + kChunk);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t w = (int64_t)blockIdx.x * kFullWarps + warp;
-  const bool live = w < W;
-  // the walker's absolute values (float pairs)
-  float ch[kNBasis][2], p0[2], tt[kMaxDet][2];
-  int valid = 0;
-  if (live) {
-    const WalkerAbs& a = wabs[w];
-    for (int k = 0; k < kNBasis; ++k) { ch[k][0] = a.chat[k][0]; ch[k][1] = a.chat[k][1]; }
-    p0[0] = a.phi0t[0];
-    p0[1] = a.phi0t[1];
-    for (int d = 0; d < kMaxDet; ++d) { tt[d][0] = a.taut[d][0]; tt[d][1] = a.taut[d][1]; }
-    valid = a.valid;
-  } else {
-    for (int k = 0; k < kNBasis; ++k) ch[k][0] = ch[k][1] = 0.f;
-    p0[0] = p0[1] = 0.f;
-    for (int d = 0; d < kMaxDet; ++d) tt[d][0] = tt[d][1] = 0.f;
-  }
-  // offset factors of the walker: lane j forms exp(2 pi i (j - 16) df tau_d)
-  {
+  const int n_seg = (n_chunks + kSegC - 1) / kSegC, gs = group_segments(n_seg), n_groups = (n_seg + gs - 1) / gs;
+  if (warp == 0) {
     const float jf = small_int_float(lane - kChunk / 2);
-    float2 t[kMaxDet];
-#pragma unroll
-    for (int d = 0; d < kMaxDet; ++d) {
-      float sh = 0.f, sl = 0.f;
-      f2x_fma_acc(tt[d][0], tt[d][1], invT_hi, invT_lo, sh, sl);  // tau_d df
-      const float p = __fmul_rn(sh, jf);
-      const float e = __fmaf_rn(sl, jf, __fmaf_rn(sh, jf, -p));
-      t[d] = cis_turns(frac_turns(p, e));
-    }
-    tp[warp][lane] = make_float4(t[0].x, t[1].x, t[0].y, t[1].y);
-    ts[warp][lane] = t[kSingle < 0 ? 0 : kSingle];
+    jt[lane][0] = make_float4(jf, jf, jf * jf, jf * jf);
+    jt[lane][1] = make_float4(jf * jf * jf, jf * jf * jf, 0.f, 0.f);
   }
-  float zh[kMaxDet][2], zl[kMaxDet][2];  // Z_d as float pairs (re, im)
-  for (int d = 0; d < kMaxDet; ++d) zh[d][0] = zh[d][1] = zl[d][0] = zl[d][1] = 0.f;
-  const int n_seg = (n_chunks + kSegC - 1) / kSegC;
-  const int sg0 = blockIdx.y * seg_per_slice, sg1 = min(n_seg, sg0 + seg_per_slice);
-  for (int sg = sg0; sg < sg1; ++sg) {
-    const int c0 = sg * kSegC, nc = min(kSegC, n_chunks - c0);
-    __syncthreads();  // the previous segment is no longer read (and tw is written)
-    {
-      const float* src = q + (size_t)c0 * kQRow;
-      for (int i = tid; i < nc * kQRow; i += kFullThreads) {
-        const int c = i / kQRow;
-        qs[c * kQPad + (i - c * kQRow)] = __ldg(src + i);
+  // the (walker octet, group) pairs, octet-major, in equal contiguous shares
+  const int64_t units = (W + kFullWarps - 1) / kFullWarps * n_groups;
+  const int64_t u0 = units * blockIdx.x / gridDim.x, u1 = units * (blockIdx.x + 1) / gridDim.x;
+  for (int64_t u = u0; u < u1; ++u) {
+    const int g = (int)(u % n_groups);
+    const int64_t w = u / n_groups * kFullWarps + warp;
+    const bool live = w < W;
+    const WalkerAbs& wa = wabs[live ? w : W - 1];
+    const bool valid = live && wa.valid;
+    if (u == u0 || g == 0) {
+      // offset factors of the warp's walker: lane j forms exp(2 pi i (j - 16) df tau_d)
+      __syncwarp();
+      const float jf = small_int_float(lane - kChunk / 2);
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+        float sh = 0.f, sl = 0.f;
+        if (valid) f2x_fma_acc(wa.taut[d][0], wa.taut[d][1], invT_hi, invT_lo, sh, sl);  // tau_d df
+        const float p = __fmul_rn(sh, jf);
+        const float e = __fmaf_rn(sl, jf, __fmaf_rn(sh, jf, -p));
+        const float2 t = cis_turns(frac_turns(p, e));
+        tp[warp][lane][d] = make_float4(t.x, t.x, t.y, t.y);
       }
     }
-    __syncthreads();
-    // data times f^-7/6 = f_c^-7/6 (1 + j u)^-7/6 (chunk series), transposed;
-    // points past the grid are zero
-    for (int p = tid; p < kSegP; p += kFullThreads) {
-      const int c = p >> 5, jj = p & (kChunk - 1);
-      const int k = c0 * kChunk + p;
-      float2 v[kMaxDet] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-      if (c < nc && k < N) {
-        const float* qa = qs + c * kQPad + kQamp;
+    f2x z[2 * ND];  // the lane's part of Z_d (re, im)
+#pragma unroll
+    for (int i = 0; i < 2 * ND; ++i) z[i] = f2x{0.f, 0.f};
+    for (int sg = g * gs; sg < min(n_seg, (g + 1) * gs); ++sg) {
+      const int c0 = sg * kSegC, nc = min(kSegC, n_chunks - c0);
+      __syncthreads();  // the previous segment is no longer read (and the tables are written)
+      {
+        const float4* src = reinterpret_cast<const float4*>(q + (size_t)c0 * kQRow);
+        float4* dst = reinterpret_cast<float4*>(qs);
+#pragma unroll 8
+        for (int i = tid; i < nc * (kQRow / 4); i += kFullThreads)
+          dst[(i / (kQRow / 4)) * (kQPad / 4) + i % (kQRow / 4)] = __ldg(src + i);
+      }
+      __syncthreads();
+      // data times f^-7/6 = f_c^-7/6 (1 + j u)^-7/6 (chunk series), transposed,
+      // chunks c and c + 32 together; points past the grid are zero
+#pragma unroll 2
+      for (int i = 0; i < kSegP / 2 / kFullThreads; ++i) {
+        const int p = tid + i * kFullThreads, c = p >> 5, jj = p & (kChunk - 1);
         const float j = small_int_float(jj - kChunk / 2);
-        const float A = qa[0] * fmaf(j, fmaf(j, fmaf(j, fmaf(j, qa[4], qa[3]), qa[2]), qa[1]), 1.f);
+        float2 v[2][ND];
 #pragma unroll
-        for (int d = 0; d < D; ++d) {
-          const float2 x = __ldg(w32 + (size_t)d * N + k);
-          v[d] = make_float2(x.x * A, x.y * A);
+        for (int h = 0; h < 2; ++h) {
+          const int ch = c + h * (kSegC / 2), k = (c0 + ch) * kChunk + jj;
+          const bool in = ch < nc && k < N;
+          const float* qa = qs + ch * kQPad + kQamp;
+          const float A = in ? qa[0] * fmaf(j, fmaf(j, fmaf(j, fmaf(j, qa[4], qa[3]), qa[2]), qa[1]), 1.f) : 0.f;
+#pragma unroll
+          for (int d = 0; d < ND; ++d) {
+            const float2 x = in ? __ldg(w32 + (size_t)d * N + k) : make_float2(0.f, 0.f);
+            v[h][d] = in ? make_float2(x.x * A, x.y * A) : make_float2(0.f, 0.f);
+          }
         }
+#pragma unroll
+        for (int d = 0; d < ND; ++d) wt[d][jj][c] = make_float4(v[0][d].x, v[1][d].x, v[0][d].y, v[1][d].y);
       }
-      if (kPair) wp[jj][c] = make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
-      if (kSingle >= 0) ws[jj][c] = v[kSingle < 0 ? 0 : kSingle];
-    }
-    // lane c: the walker's coefficients of chunk c (X0 with Phi0, whole turns
-    // dropped) and the chunk factors exp(2 pi i f_c tau_d), in registers
-    float X0h = 0.f, X0l = 0.f, X1h = 0.f, X1l = 0.f, X2h = 0.f, X2l = 0.f, xn[kOrd - 2];
-    float2 E[kMaxDet];
+      __syncthreads();  // wt complete
+      if (!valid) continue;
+      // the walker's coefficients of the lane's chunks (X0 with Phi0, whole turns
+      // dropped); a chunk past the last has zero rows and zero data
+      const bool in0 = lane < nc, in1 = lane + kSegC / 2 < nc;
+      if (!in0) continue;
+      const float* r0 = qs + lane * kQPad;
+      const float* r1 = r0 + (kSegC / 2) * kQPad;
+      // float4 i of the two rows
+      auto row4 = [&](int i, float4& a, float4& b) {
+        a = reinterpret_cast<const float4*>(r0)[i];
+        b = in1 ? reinterpret_cast<const float4*>(r1)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      };
+      float2 X0h = pv::splat<float2>(wa.phi0t[0]), X0l = pv::splat<float2>(wa.phi0t[1]);
+      float2 X1h = make_float2(0.f, 0.f), X1l = X1h, X2h = X1h, X2l = X1h, xn[kOrd - 2];
 #pragma unroll
-    for (int n = 0; n < kOrd - 2; ++n) xn[n] = 0.f;
-#pragma unroll
-    for (int d = 0; d < kMaxDet; ++d) E[d] = make_float2(1.f, 0.f);
-    const bool act = live && valid && lane < nc;
-    if (act) {
-      const float* row = qs + lane * kQPad;
-      X0h = p0[0];
-      X0l = p0[1];
+      for (int n = 0; n < kOrd - 2; ++n) xn[n] = make_float2(0.f, 0.f);
+      float4 a, b;
 #pragma unroll
       for (int k = 0; k < kNBasis; ++k) {
-        const float a = ch[k][0], b = ch[k][1];
-        f2x_fma_acc(a, b, row[kQ01 + 4 * k], row[kQ01 + 4 * k + 1], X0h, X0l);
-        f2x_fma_acc(a, b, row[kQ01 + 4 * k + 2], row[kQ01 + 4 * k + 3], X1h, X1l);
-        f2x_fma_acc(a, b, row[kQ2 + 2 * k], row[kQ2 + 2 * k + 1], X2h, X2l);
-#pragma unroll
-        for (int n = 0; n < kOrd - 2; ++n) xn[n] = fmaf(a, row[kQh + n * kNBasis + k], xn[n]);
+        const float2 ch = pv::splat<float2>(wa.chat[k][0]), cl = pv::splat<float2>(wa.chat[k][1]);
+        row4(kQ01 / 4 + k, a, b);
+        pv::fma_acc(ch, cl, make_float2(a.x, b.x), make_float2(a.y, b.y), X0h, X0l);
+        pv::fma_acc(ch, cl, make_float2(a.z, b.z), make_float2(a.w, b.w), X1h, X1l);
+        if (k % 2 == 0) {
+          const float2 ch1 = pv::splat<float2>(wa.chat[k + 1][0]), cl1 = pv::splat<float2>(wa.chat[k + 1][1]);
+          row4(kQ2 / 4 + k / 2, a, b);
+          pv::fma_acc(ch, cl, make_float2(a.x, b.x), make_float2(a.y, b.y), X2h, X2l);
+          pv::fma_acc(ch1, cl1, make_float2(a.z, b.z), make_float2(a.w, b.w), X2h, X2l);
+        }
       }
-      X0h = __fadd_rn(X0h, -round_fma_pipe(X0h));
-      const float fch = row[kQfc], fcl = row[kQfc + 1];
 #pragma unroll
-      for (int d = 0; d < D; ++d) {
-        float ah = 0.f, al = 0.f;
-        f2x_fma_acc(tt[d][0], tt[d][1], fch, fcl, ah, al);  // f_c tau_d
-        E[d] = cis_turns(frac_turns(ah, al));
+      for (int i = 0; i < (kOrd - 2) * kNBasis / 4; ++i) {  // orders 3..8, basis index fastest
+        row4(kQh / 4 + i, a, b);
+        const float2 m[4] = {make_float2(a.x, b.x), make_float2(a.y, b.y), make_float2(a.z, b.z), make_float2(a.w, b.w)};
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int n = (4 * i + v) / kNBasis, k = (4 * i + v) % kNBasis;
+          xn[n] = pv::fma(pv::splat<float2>(wa.chat[k][0]), m[v], xn[n]);
+        }
       }
-    }
-    __syncthreads();  // wt complete
-    if (!act) continue;
-    float2 apr = make_float2(0.f, 0.f), api = apr;  // detectors 0, 1
-    float asr = 0.f, asi = 0.f;                     // detector D-1
+      X0h = pv::frac1(X0h);
+      float2 ar[ND], ai[ND];  // the chunks' sums
+#pragma unroll
+      for (int d = 0; d < ND; ++d) ar[d] = ai[d] = make_float2(0.f, 0.f);
+      const float2 one = make_float2(1.f, 1.f), two = make_float2(2.f, 2.f), mtwo = make_float2(-2.f, -2.f);
 #pragma unroll 2
-    for (int jj = 0; jj < kChunk; ++jj) {
-      const float jf = small_int_float(jj - kChunk / 2);
-      // x = X0 + X1 j + X2 j^2 + j^3 (X3 + ... + X8 j^5)
-      const float t = fmaf(fmaf(fmaf(fmaf(fmaf(xn[5], jf, xn[4]), jf, xn[3]), jf, xn[2]), jf, xn[1]), jf, xn[0]);
-      const float j2 = jf * jf;
-      const float t3 = t * (j2 * jf);
-      const float p1 = __fmul_rn(X1h, jf);
-      float e1 = __fmaf_rn(X1h, jf, -p1);
-      e1 = __fmaf_rn(X1l, jf, e1);
-      const float p2 = __fmul_rn(X2h, j2);
-      float e2 = __fmaf_rn(X2h, j2, -p2);
-      e2 = __fmaf_rn(X2l, j2, e2);
-      float sh = X0h, sl = X0l;
-      f2x_add(sh, sl, p1);
-      f2x_add(sh, sl, p2);
-      sl = __fadd_rn(sl, __fadd_rn(__fadd_rn(e1, e2), t3));
-      const float2 z = cis_turns(frac_turns(sh, sl));  // exp(+2 pi i x)
-      // offset factor exp(2 pi i (j - 16) df tau_d) (the same for all lanes)
-      // times the phasor, times the data
-      if constexpr (kPair) {
-        const float4 T = tp[warp][jj];
-        const float4 v = wp[jj][lane];
-        const float2 Tr = make_float2(T.x, T.y), Ti = make_float2(T.z, T.w);
-        const float2 zx = make_float2(z.x, z.x), zy = make_float2(z.y, z.y);
-        const float2 ur = pv::fma(zx, Tr, pv::mul(pv::neg(zy), Ti)), ui = pv::fma(zx, Ti, pv::mul(zy, Tr));
-        const float2 vr = make_float2(v.x, v.y), vi = make_float2(v.z, v.w);
-        apr = pv::fma(vr, ur, pv::fma(pv::neg(vi), ui, apr));
-        api = pv::fma(vr, ui, pv::fma(vi, ur, api));
-      }
-      if constexpr (kSingle >= 0) {
-        const float2 T = ts[warp][jj];
-        const float ur = fmaf(z.x, T.x, -z.y * T.y), ui = fmaf(z.x, T.y, z.y * T.x);
-        const float2 v = ws[jj][lane];
-        asr = fmaf(v.x, ur, fmaf(-v.y, ui, asr));
-        asi = fmaf(v.x, ui, fmaf(v.y, ur, asi));
-      }
-    }
-    // the chunk factor, once per chunk, then into the lane's float pairs
-    float acc[kMaxDet][2] = {{apr.x, api.x}, {apr.y, api.y}, {0.f, 0.f}};
-    if (kSingle >= 0) {
-      acc[kSingle < 0 ? 0 : kSingle][0] = asr;
-      acc[kSingle < 0 ? 0 : kSingle][1] = asi;
-    }
+      for (int jj = 0; jj < kChunk; ++jj) {
+        const float4 ja = jt[jj][0], jb = jt[jj][1];
+        const float2 j1 = make_float2(ja.x, ja.y), j2 = make_float2(ja.z, ja.w), j3 = make_float2(jb.x, jb.y);
+        // x = X0 + X1 j + X2 j^2 + j^3 (X3 + ... + X8 j^5)
+        float2 t = pv::fma(xn[5], j1, xn[4]);
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      const float gr = fmaf(E[d].x, acc[d][0], -E[d].y * acc[d][1]);
-      const float gi = fmaf(E[d].x, acc[d][1], E[d].y * acc[d][0]);
-      f2x_add(zh[d][0], zl[d][0], gr);
-      f2x_add(zh[d][1], zl[d][1], gi);
-    }
-  }
-  if (!live) return;
-  double* zo = zout + ((size_t)blockIdx.y * W + w) * 6;
-  // warp sums in FP64 (lane order fixed by the butterfly)
+        for (int n = 3; n >= 0; --n) t = pv::fma(t, j1, xn[n]);
+        const float2 t3 = pv::mul(t, j3);
+        const float2 p1 = pv::mul(X1h, j1), p2 = pv::mul(X2h, j2);
+        const float2 e1 = pv::fma(X1l, j1, pv::fma(X1h, j1, pv::neg(p1)));
+        const float2 e2 = pv::fma(X2l, j2, pv::fma(X2h, j2, pv::neg(p2)));
+        float2 sh = X0h, sl = X0l;
+        pv::add_acc(sh, sl, p1);
+        pv::add_acc(sh, sl, p2);
+        sl = pv::add(sl, pv::add(pv::add(e1, e2), t3));
+        const float2 y = pv::frac1(pv::frac(sh, sl));
+        float2 sn, cs;
+        pv::sincos_half(y, sn, cs);
+        const float2 zx = pv::fma(pv::mul(mtwo, sn), sn, one), zy = pv::mul(pv::mul(two, sn), cs);  // exp(+2 pi i x)
+        // offset factor times the phasor, times the data
 #pragma unroll
-  for (int d = 0; d < kMaxDet; ++d) {
-    const double re = warp_sum_f64((double)zh[d][0] + (double)zl[d][0]);
-    const double im = warp_sum_f64((double)zh[d][1] + (double)zl[d][1]);
-    if (lane == 0) {
-      zo[2 * d] = valid ? re : 0.0;
-      zo[2 * d + 1] = valid ? im : 0.0;
+        for (int d = 0; d < ND; ++d) {
+          const float4 T = tp[warp][jj][d], v = wt[d][jj][lane];
+          const float2 Tr = make_float2(T.x, T.y), Ti = make_float2(T.z, T.w);
+          const float2 vr = make_float2(v.x, v.y), vi = make_float2(v.z, v.w);
+          const float2 ur = pv::fma(zx, Tr, pv::mul(pv::neg(zy), Ti)), ui = pv::fma(zx, Ti, pv::mul(zy, Tr));
+          ar[d] = pv::fma(vr, ur, pv::fma(pv::neg(vi), ui, ar[d]));
+          ai[d] = pv::fma(vr, ui, pv::fma(vi, ur, ai[d]));
+        }
+      }
+      // the chunk factors exp(2 pi i f_c tau_d), once per chunk, then into the
+      // lane's float pairs, chunk l before chunk l + 32
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (h == 1 && !in1) continue;
+          const float* r = h ? r1 : r0;
+          float ah = 0.f, al = 0.f;
+          f2x_fma_acc(wa.taut[d][0], wa.taut[d][1], r[kQfc], r[kQfc + 1], ah, al);  // f_c tau_d
+          const float2 E = cis_turns(frac_turns(ah, al));
+          const float a_r = h ? ar[d].y : ar[d].x, a_i = h ? ai[d].y : ai[d].x;
+          f2x_add(z[2 * d].hi, z[2 * d].lo, fmaf(E.x, a_r, -E.y * a_i));
+          f2x_add(z[2 * d + 1].hi, z[2 * d + 1].lo, fmaf(E.x, a_i, E.y * a_r));
+        }
+      }
     }
+    // the lanes' sums: after the five levels a lane holds one value
+    constexpr int n0 = 2 * ND, n1 = (n0 + 1) / 2, n2 = (n1 + 1) / 2, n3 = (n2 + 1) / 2;
+    static_assert(n3 == 1, "three levels reduce to one value");
+    f2x z1[n1], z2[n2], z3[1], z4[1], z5[1];
+    ff_level(z, z1, lane, 16);
+    ff_level(z1, z2, lane, 8);
+    ff_level(z2, z3, lane, 4);
+    ff_level(z3, z4, lane, 2);
+    ff_level(z4, z5, lane, 1);
+    // its index: the halves the lane kept, from the last level back (a lane whose
+    // kept half was padding holds none)
+    int idx = (lane & 4) ? n3 : 0;
+    bool ok = (lane & 3) == 0 && idx < n2;
+    idx += (lane & 8) ? n2 : 0;
+    ok = ok && idx < n1;
+    idx += (lane & 16) ? n1 : 0;
+    if (live && ok && idx < n0) zout[((size_t)g * W + w) * 6 + idx] = (double)z5[0].hi + (double)z5[0].lo;
   }
-  if (lane == 0 && !valid) zo[0] = NAN;  // marks an unphysical walker
 }
 
 // log L per walker from Z_d and K_d (FP64); H_d from the summary's B0 and
-// the reference prefactor, scales from the FP32 data copy's exponents.
-__global__ void __launch_bounds__(128) k_full_finish(const double* __restrict__ zout, int n_slices,
+// the reference prefactor, scales from the FP32 data copy's exponents.  Eight
+// lanes per walker, each adding every eighth group; one warp per detector forms
+// H_d (one warp for all detectors and one thread per walker took 31 us for 512
+// walkers, all of it load latency).
+constexpr int kFinishLanes = 8;
+constexpr int kFinishThreads = 128;
+__global__ void __launch_bounds__(kFinishThreads) k_full_finish(const double* __restrict__ zout, int n_groups,
                                                      const WalkerAbs* __restrict__ wabs,
                                                      int64_t W, int D, int B, double T, const int* __restrict__ exps,
                                                      const double* __restrict__ summ, const RefValues* __restrict__ ref,
                                                      double* __restrict__ logl) {
+  static_assert(kFinishThreads / 32 >= kMaxDet, "one warp per detector");
   __shared__ double H[kMaxDet], sc0[kMaxDet];
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    for (int d = 0; d < D; ++d) {
-      double s = 0.0;
-      for (int b = lane; b < B; b += 32) s += summ[((size_t)d * B + b) * 6 + 4];  // B0
-      s = warp_sum_f64(s);
-      if (lane == 0) {
-        const double kr = ref->K[d][0], ki = ref->K[d][1];
-        H[d] = s / (kr * kr + ki * ki);
-        const int sd = exps[2 * d], sS = exps[2 * d + 1];
-        sc0[d] = (4.0 / T) * __hiloint2double((1023 + sS - sd) << 20, 0);
-      }
-    }
-  }
-  __syncthreads();
-  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= W) return;
-  if (!wabs[w].valid) {
-    logl[w] = -INFINITY;
-    return;
-  }
+  const int part = threadIdx.x % kFinishLanes;
+  const int64_t w = ((int64_t)blockIdx.x * kFinishThreads + threadIdx.x) / kFinishLanes;
+  const int64_t wc = w < W ? w : W - 1;
+  // the walker's sums over the groups, lane by lane, then a fixed tree
   double z[2 * kMaxDet] = {0, 0, 0, 0, 0, 0};
-  for (int sl = 0; sl < n_slices; ++sl) {  // slices in order: the sum does not depend on the schedule
-    const double* zs = zout + ((size_t)sl * W + w) * 6;
+  for (int g = part; g < n_groups; g += kFinishLanes) {
+    const double* zs = zout + ((size_t)g * W + wc) * 6;
 #pragma unroll
     for (int i = 0; i < 2 * kMaxDet; ++i)
       if (i < 2 * D) z[i] += zs[i];
   }
+  const int d = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (d < D) {
+    double s[4] = {0, 0, 0, 0};
+    for (int b = lane; b < B; b += 128)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (b + 32 * u < B) s[u] += summ[((size_t)d * B + b + 32 * u) * 6 + 4];  // B0
+    const double t = warp_sum_f64((s[0] + s[1]) + (s[2] + s[3]));
+    if (lane == 0) {
+      const double kr = ref->K[d][0], ki = ref->K[d][1];
+      H[d] = t / (kr * kr + ki * ki);
+      const int sd = exps[2 * d], sS = exps[2 * d + 1];
+      sc0[d] = (4.0 / T) * __hiloint2double((1023 + sS - sd) << 20, 0);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 2 * kMaxDet; ++i)
+    if (i < 2 * D)
+#pragma unroll
+      for (int o = kFinishLanes / 2; o > 0; o >>= 1) z[i] += __shfl_xor_sync(0xffffffffu, z[i], o);
+  if (w >= W || part != 0) return;
+  if (!wabs[w].valid) {
+    logl[w] = -INFINITY;
+    return;
+  }
   double L = 0.0;
 #pragma unroll
-  for (int d = 0; d < kMaxDet; ++d) {
-    if (d >= D) break;
-    const double kr = wabs[w].K[d][0], ki = wabs[w].K[d][1];
-    const double dh = sc0[d] * (kr * z[2 * d] + ki * z[2 * d + 1]);  // Re(conj(K) Z)
-    L += dh - 0.5 * (kr * kr + ki * ki) * H[d];
+  for (int dd = 0; dd < kMaxDet; ++dd) {
+    if (dd >= D) break;
+    const double kr = wabs[w].K[dd][0], ki = wabs[w].K[dd][1];
+    const double dh = sc0[dd] * (kr * z[2 * dd] + ki * z[2 * dd + 1]);  // Re(conj(K) Z)
+    L += dh - 0.5 * (kr * kr + ki * ki) * H[dd];
   }
   logl[w] = L;
 }
@@ -321,37 +372,23 @@ extern "C" int rb_loglike_full_batch(rb_event_t ev, const double* theta_dev, int
     e.w32_resident = e.w32_current = true;
     count_launches(1);
   }
-  void (*const kz)(const float2*, int, const float*, int, const WalkerAbs*, int64_t, float, float, int, double*) =
+  void (*const kz)(const float2*, int, const float*, int, const WalkerAbs*, int64_t, float, float, double*) =
       e.n_det == 1 ? k_full_z<1> : e.n_det == 2 ? k_full_z<2> : k_full_z<3>;
+  const int smem = full_smem(e.n_det);
   static std::atomic<bool> smem_raised[kMaxDet];  // the attribute is idempotent: concurrent first calls only repeat it
   if (!smem_raised[e.n_det - 1].load(std::memory_order_acquire)) {
-    if ((err = cudaFuncSetAttribute(kz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFullSmem)) != cudaSuccess)
+    if ((err = cudaFuncSetAttribute(kz, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
       return cuda_fail(err, "rb_loglike_full_batch: shared memory attribute");
     smem_raised[e.n_det - 1].store(true, std::memory_order_release);
   }
-  // slices of the grid per group of 8 walkers: at least two waves of blocks
-  // (2 per SM), then the count in the next few that wastes the least of the last wave
+  // one wave of blocks (2 per SM), each with an equal share of the (8 walkers,
+  // group) pairs
   const int nc = (int)((e.N + kChunk - 1) / kChunk);
-  const int n_seg = (nc + kSegC - 1) / kSegC;
-  const int64_t wblocks = (W + kFullWarps - 1) / kFullWarps;
-  int n_slices = 1;
-  {
-    int dev = 0, n_sm = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t wave = 2 * (int64_t)n_sm;
-    const int64_t s_min = std::max<int64_t>(1, (2 * wave + wblocks - 1) / wblocks);
-    const int64_t s_cap = std::max<int64_t>(1, n_seg / 2);  // keep >= 2 segments per slice
-    double best = -1.0;
-    for (int64_t sl = std::min(s_min, s_cap); sl <= std::min(s_min + 8, s_cap); ++sl) {
-      const int64_t per = (n_seg + sl - 1) / sl, used = (n_seg + per - 1) / per;  // slices actually non-empty
-      const int64_t blocks = wblocks * used;
-      const double eff = (double)blocks / (double)(wave * ((blocks + wave - 1) / wave));
-      if (eff > best + 1e-9) { best = eff; n_slices = (int)used; }
-    }
-  }
-  const int seg_per_slice = (n_seg + n_slices - 1) / n_slices;
+  const int n_seg = (nc + kSegC - 1) / kSegC, gs = group_segments(n_seg), n_groups = (n_seg + gs - 1) / gs;
+  const int64_t units = (W + kFullWarps - 1) / kFullWarps * n_groups;
+  const unsigned blocks = (unsigned)std::min<int64_t>(units, 2 * (int64_t)sm_count());
   char* buf = nullptr;
-  const size_t abs_bytes = sizeof(WalkerAbs) * W, z_bytes = sizeof(double) * 6 * W * n_slices;
+  const size_t abs_bytes = sizeof(WalkerAbs) * W, z_bytes = sizeof(double) * 6 * W * n_groups;
   err = ws_alloc(reinterpret_cast<void**>(&buf), abs_bytes + z_bytes, s);
   if (err != cudaSuccess) return cuda_fail(err, "rb_loglike_full_batch: workspace allocation");
   WalkerAbs* wabs = reinterpret_cast<WalkerAbs*>(buf);
@@ -362,11 +399,11 @@ extern "C" int rb_loglike_full_batch(rb_event_t ev, const double* theta_dev, int
   if ((err = launch_setup_abs(theta_dev, W, e.ec, wabs, s)) != cudaSuccess) {
     rc = cuda_fail(err, "rb_loglike_full_batch: set-up kernel");
   } else {
-    kz<<<dim3((unsigned)wblocks, (unsigned)n_slices), kFullThreads, kFullSmem, s>>>(
-        static_cast<const float2*>(e.d_w32), (int)e.N, static_cast<const float*>(e.d_chunkq), nc, wabs, W, ih, il,
-        seg_per_slice, zout);
-    k_full_finish<<<(unsigned)((W + 127) / 128), 128, 0, s>>>(zout, n_slices, wabs, W, e.n_det, e.n_bins, e.T, e.d_wexp,
-                                                              e.d_summ, e.d_ref, logl_dev);
+    kz<<<blocks, kFullThreads, smem, s>>>(static_cast<const float2*>(e.d_w32), (int)e.N,
+                                          static_cast<const float*>(e.d_chunkq), nc, wabs, W, ih, il, zout);
+    constexpr int per_block = kFinishThreads / kFinishLanes;
+    k_full_finish<<<(unsigned)((W + per_block - 1) / per_block), kFinishThreads, 0, s>>>(
+        zout, n_groups, wabs, W, e.n_det, e.n_bins, e.T, e.d_wexp, e.d_summ, e.d_ref, logl_dev);
     if ((err = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(err, "rb_loglike_full_batch: kernels");
     else count_launches(3);
   }
