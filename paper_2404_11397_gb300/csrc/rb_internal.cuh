@@ -220,7 +220,8 @@ struct EventDev {
   // upper bounds of |g_k(f) / 2pi| (k < kNBasis) and of f over the event's
   // grid: the mixed kernel's per-walker bound on its phase terms
   float gmax[kNBasis + 1];
-  // FP64 tables: g[k][e] (10*Ep), f[e] (Ep), then per detector 6 rows of Bp
+  // FP64 tables: g[k][e] (10*Ep), f[e] (Ep), then per detector 6 rows of Bp, the
+  // coefficients gmr, gpr, gmi, gpi, h, q of the slot image
   const double* tab64;
   const RefValues* ref;
 };
@@ -293,7 +294,7 @@ __device__ __forceinline__ double event_base_logl(const EventDev& ev) { return e
 struct SummaryOut {
   double* summ;          // [D][B][6] FP64 summary: A0 re/im, A1 re/im, B0, B1
   float* bin32;          // [D][6][Bp] bin tables (float)
-  double* bin64;         // [D][6][Bp] bin tables (FP64)
+  double* bin64;         // [D][6][Bp] bin coefficients (FP64; EventDev::tab64)
   const double* inv_df;  // [B] 1 / (f_{b+1} - f_b)
   double* share;         // [D][B] per-bin share of log L(theta_ref)
   SummarySync* sync;     // counters, zero between builds
@@ -555,6 +556,51 @@ __device__ __forceinline__ void add_acc(V& hi, V& lo, V v) {
   hi = s;
 }
 }  // namespace pv
+
+// Sine and cosine of 2 pi x in FP64: x is reduced to a quarter turn, 2 pi x = theta +
+// q pi/2 with theta = 2 pi r, r in [-1/8, 1/8] (q's low two bits are returned),
+// and sin theta = sn, cos theta = 1 + w pc by their Taylor series (|theta| <= pi/4:
+// the first dropped terms are below 2^-54 of the leading ones).  19 FP64 operations (an FP64 warp
+// instruction holds its SM sub-partition's FP64 unit for ~65 clocks): the
+// quadrant is left to the caller's integer selects.
+__device__ __forceinline__ int quarter_turn64(double x, double& sn, double& pc, double& w) {
+  const double magic = 6755399441055744.0;  // 1.5 * 2^52
+  const double t = fma(x, 4.0, magic);
+  const double r = fma(t - magic, -0.25, x);
+  w = r * r;
+  double ps = -0.7181223017785006;       // -(2 pi)^15 / 15!
+  ps = fma(ps, w, 3.819952584848282);   // (2 pi)^13 / 13!
+  ps = fma(ps, w, -15.09464257682299);  // -(2 pi)^11 / 11!
+  ps = fma(ps, w, 42.058693944897655);   // (2 pi)^9 / 9!
+  ps = fma(ps, w, -76.70585975306139);   // -(2 pi)^7 / 7!
+  ps = fma(ps, w, 81.60524927607506);    // (2 pi)^5 / 5!
+  ps = fma(ps, w, -41.34170224039976);  // -(2 pi)^3 / 3!
+  ps = fma(ps, w, 6.283185307179586);
+  sn = r * ps;
+  pc = 0.28200596845579123;       // (2 pi)^16 / 16!
+  pc = fma(pc, w, -1.714390711088672);  // -(2 pi)^14 / 14!
+  pc = fma(pc, w, 7.903536371318469);    // (2 pi)^12 / 12!
+  pc = fma(pc, w, -26.4262567833744);   // -(2 pi)^10 / 10!
+  pc = fma(pc, w, 60.24464137187666);   // (2 pi)^8 / 8!
+  pc = fma(pc, w, -85.45681720669373);   // -(2 pi)^6 / 6!
+  pc = fma(pc, w, 64.9393940226683);    // (2 pi)^4 / 4!
+  pc = fma(pc, w, -19.739208802178716);  // -(2 pi)^2 / 2
+  return __double2loint(t) & 3;
+}
+
+// exp(-2 pi i x) - 1, relative accuracy kept next to x = 0 (0 at 0):
+//   q = 0: (c1, -sn)  1: (-sn - 1, -c1 - 1)  2: (-c1 - 2, sn)  3: (sn - 1, c1 + 1),  c1 = w pc
+__device__ __forceinline__ void expm1_neg_turns64(double x, double& er, double& ei) {
+  double sn, pc, w;
+  const int q = quarter_turn64(x, sn, pc, w);
+  const double c1 = w * pc;
+  const double a = (q & 1) ? sn : c1, b = (q & 1) ? c1 : sn;
+  const int fa = (int)(((unsigned)(q + 1) & 2u) << 30), fb = (int)((~(unsigned)q & 2u) << 30);
+  const int ka = q == 0 ? 0 : (q == 2 ? (int)0xC0000000u : (int)0xBFF00000u);                   // 0, -1, -2, -1
+  const int kb = q == 1 ? (int)0xBFF00000u : (q == 3 ? 0x3FF00000 : 0);                        // 0, -1, 0, 1
+  er = __hiloint2double(__double2hiint(a) ^ fa, __double2loint(a)) + __hiloint2double(ka, 0);
+  ei = __hiloint2double(__double2hiint(b) ^ fb, __double2loint(b)) + __hiloint2double(kb, 0);
+}
 
 // Device-scope release/acquire fence.  The summary builds publish per-part
 // and per-bin results and then take a ticket with a relaxed atomic; the

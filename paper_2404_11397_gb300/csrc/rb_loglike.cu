@@ -159,14 +159,14 @@ __device__ __forceinline__ void warp_sum_ff(float& h, float& l) {
 // One level of a transposed warp sum: lanes whose bit o is clear keep values
 // [0, M) of `in` and send [M, N), lanes whose bit is set keep [M, N) (zero
 // beyond N) and send [0, M); each adds what its partner sent.
-template <int N, int M>
-__device__ __forceinline__ void tsum_level(const float (&in)[N], float (&out)[M], int lane, int o) {
+template <class T, int N, int M>
+__device__ __forceinline__ void tsum_level(const T (&in)[N], T (&out)[M], int lane, int o) {
   const bool up = (lane & o) != 0;
 #pragma unroll
   for (int i = 0; i < M; ++i) {
-    const float lo = in[i], hi = (M + i < N) ? in[M + i] : 0.f;
-    const float keep = up ? hi : lo, send = up ? lo : hi;
-    out[i] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, o));
+    const T lo = in[i], hi = (M + i < N) ? in[M + i] : T(0);
+    const T keep = up ? hi : lo, send = up ? lo : hi;
+    out[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
   }
 }
 
@@ -174,17 +174,17 @@ __device__ __forceinline__ void tsum_level(const float (&in)[N], float (&out)[M]
 // after five halving levels every lane holds the total of one value, which
 // it writes to out[index] (shared memory); 31 shuffles for 32 values against
 // 5 NV for NV separate butterflies.
-template <int NV>
-__device__ __forceinline__ void warp_transposed_sums(const float (&v)[NV], int lane, float* out) {
+template <class T, int NV>
+__device__ __forceinline__ void warp_transposed_sums(const T (&v)[NV], int lane, T* out) {
   static_assert(NV >= 1 && NV <= 32, "up to 32 values");
   constexpr int m1 = (NV + 1) / 2, m2 = (m1 + 1) / 2, m3 = (m2 + 1) / 2, m4 = (m3 + 1) / 2, m5 = (m4 + 1) / 2;
   static_assert(m5 == 1, "five levels reduce to one value");
-  float a[m1], b[m2], c[m3], d[m4], e[m5];
-  tsum_level<NV, m1>(v, a, lane, 16);
-  tsum_level<m1, m2>(a, b, lane, 8);
-  tsum_level<m2, m3>(b, c, lane, 4);
-  tsum_level<m3, m4>(c, d, lane, 2);
-  tsum_level<m4, m5>(d, e, lane, 1);
+  T a[m1], b[m2], c[m3], d[m4], e[m5];
+  tsum_level(v, a, lane, 16);
+  tsum_level(a, b, lane, 8);
+  tsum_level(b, c, lane, 4);
+  tsum_level(c, d, lane, 2);
+  tsum_level(d, e, lane, 1);
   // the value's index: the positions this lane kept, from the last level back
   // (a lane whose kept half was padding at some level holds no value)
   int idx = (lane & 1) ? m5 : 0;
@@ -267,60 +267,37 @@ __device__ __forceinline__ void mala_finish(const MalaArgs& m, int64_t w, int la
 
 // Chain rule for one walker: lane j < 13 returns d log L / d theta_j from the
 // reduced adjoints (adj_c over the basis coefficients, adj_tau per detector
-// delay, adj_rho per detector prefactor) and the set-up tangents.
-template <class T>
-__device__ __forceinline__ double chain_rule(int j, int n_det, const T* adj_c, const T* adj_tau, const T (*adj_rho)[2],
-                                             const T (*rho)[2], const WalkerTan<T>& tn) {
-  T g = T(0);
-  if (j < kNTanIntr)
-    for (int k = 0; k < kNBasis; ++k) g += adj_c[k] * tn.dc[k][j];
-  for (int d = 0; d < n_det; ++d) {
-    if (j == 7) g += adj_tau[d];                                   // t_c
-    if (j == 11 || j == 12) g += adj_tau[d] * tn.dtd[d][j - 11];  // ra, dec through the delay
-    // prefactor: d log L = Re(conj(gbar_rho) rho dln rho), dln rho = lr + i li
-    const T Gr = adj_rho[d][0] * rho[d][0] + adj_rho[d][1] * rho[d][1];
-    const T Gi = adj_rho[d][0] * rho[d][1] - adj_rho[d][1] * rho[d][0];
-    T lr = T(0), li = T(0);
-    if (j == 0) { lr = tn.lnamp_Mc; li = -tn.dphi0[0]; }
-    else if (j == 1) { li = -tn.dphi0[1]; }
-    else if (j == 6) { lr = tn.lnamp_dL; }
-    else if (j == 8) { li = T(1); }
-    else if (j >= 9) { lr = tn.dlnP[d][j - 9][0]; li = tn.dlnP[d][j - 9][1]; }
-    g += Gr * lr - Gi * li;
-  }
-  return (double)g;
-}
-
-// The same chain rule for the mixed kernel, with the tangents in shared
-// memory: every lane runs one instruction stream (the lane's tangent entries
-// picked by index and select, no divergent branches).  G_d = conj(gbar_rho_d)
-// rho_d, the prefactor's adjoint in the form d log L = Re(G_d dln rho_d).
-template <int D>
-__device__ __forceinline__ float chain_rule_lanes(int j, const float* adj_c, const float* adj_tau, const float (*G)[2],
-                                                  const WalkerTan<float>& tn) {
-  const float* t = reinterpret_cast<const float*>(&tn);
-  constexpr int oDc = offsetof(WalkerTan<float>, dc) / 4, oPhi = offsetof(WalkerTan<float>, dphi0) / 4;
-  constexpr int oDtd = offsetof(WalkerTan<float>, dtd) / 4, oLnP = offsetof(WalkerTan<float>, dlnP) / 4;
-  constexpr int oMc = offsetof(WalkerTan<float>, lnamp_Mc) / 4, oDl = offsetof(WalkerTan<float>, lnamp_dL) / 4;
+// delay, G_d = conj(gbar_rho_d) rho_d per prefactor: d log L = Re(G_d dln rho_d))
+// and the set-up tangents.  Every lane runs one instruction stream (the lane's
+// tangent entries picked by index and select, no divergent branches).
+__device__ __forceinline__ float madd(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double madd(double a, double b, double c) { return fma(a, b, c); }
+template <int D, class T>
+__device__ __forceinline__ T chain_rule_lanes(int j, const T* adj_c, const T* adj_tau, const T (*G)[2],
+                                              const WalkerTan<T>& tn) {
+  const T* t = reinterpret_cast<const T*>(&tn);
+  constexpr int oDc = offsetof(WalkerTan<T>, dc) / sizeof(T), oPhi = offsetof(WalkerTan<T>, dphi0) / sizeof(T);
+  constexpr int oDtd = offsetof(WalkerTan<T>, dtd) / sizeof(T), oLnP = offsetof(WalkerTan<T>, dlnP) / sizeof(T);
+  constexpr int oMc = offsetof(WalkerTan<T>, lnamp_Mc) / sizeof(T), oDl = offsetof(WalkerTan<T>, lnamp_dL) / sizeof(T);
   const bool intr = j < kNTanIntr, radec = j == 11 || j == 12, ext = j >= 9;
   const int ji = intr ? j : 0, jr = radec ? j - 11 : 0, je = ext ? j - 9 : 0;
-  float g = 0.f;
+  T g = T(0);
 #pragma unroll
   for (int k = 0; k < kNBasis; ++k) {
-    const float v = t[oDc + k * kNTanIntr + ji];
-    g = fmaf(adj_c[k], intr ? v : 0.f, g);
+    const T v = t[oDc + k * kNTanIntr + ji];
+    g = madd(adj_c[k], intr ? v : T(0), g);
   }
   // d ln rho_d = lr + i li: ln amplitude (Mc, dL), -dPhi0 (Mc, q), phi_c, antenna (iota, psi, ra, dec)
   const int ir = j == 0 ? oMc : (j == 6 ? oDl : oMc);
-  const float lr_own = (j == 0 || j == 6) ? t[ir] : 0.f;
+  const T lr_own = (j == 0 || j == 6) ? t[ir] : T(0);
   const int ii = j == 1 ? oPhi + 1 : oPhi;
-  const float li_own = (j == 0 || j == 1) ? -t[ii] : (j == 8 ? 1.f : 0.f);
+  const T li_own = (j == 0 || j == 1) ? -t[ii] : (j == 8 ? T(1) : T(0));
 #pragma unroll
   for (int d = 0; d < D; ++d) {
-    const float td = t[oDtd + 2 * d + jr];
-    g = fmaf(adj_tau[d], radec ? td : (j == 7 ? 1.f : 0.f), g);
-    const float pr = t[oLnP + 8 * d + 2 * je], pi = t[oLnP + 8 * d + 2 * je + 1];
-    const float lr = ext ? pr : lr_own, li = ext ? pi : li_own;
+    const T td = t[oDtd + 2 * d + jr];
+    g = madd(adj_tau[d], radec ? td : (j == 7 ? T(1) : T(0)), g);
+    const T pr = t[oLnP + 8 * d + 2 * je], pi = t[oLnP + 8 * d + 2 * je + 1];
+    const T lr = ext ? pr : lr_own, li = ext ? pi : li_own;
     g += G[d][0] * lr - G[d][1] * li;  // Re(G_d dln rho_d)
   }
   return g;
@@ -852,7 +829,7 @@ __global__ void __launch_bounds__(kThreads)
       const float two_pi = 6.28318530717958648f;
       // the walker's adjoint sums (basis coefficients, then per detector the
       // delay and the prefactor ratio re/im) by one transposed warp sum
-      warp_transposed_sums<kNV>(v, lane, work->red);
+      warp_transposed_sums(v, lane, work->red);
       __syncwarp();
       float ac[kNBasis], at[kMaxDet], ar[kMaxDet][2];
 #pragma unroll
@@ -889,18 +866,31 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // ---------------------------------------------------------------------------
-// Plain FP64 comparison path: same mapping, everything in FP64, tables read
-// through the cache from global memory.
+// Plain FP64 comparison path: lane l of chunk c at edge 31 c + l, everything in
+// FP64, tables read through the cache from global memory.
+//
+// Bound: the FP64 pipe (one warp instruction per ~65 clocks per SM
+// sub-partition, whatever the lanes), so what counts is FP64 instructions per
+// edge: with three detectors 170 -- the bin term in the coefficients of its edge
+// values (as det_edge_slot; the beta1 term, zero for a ratio of constant
+// modulus, left out), e^{-2 pi i x} - 1 from one quarter-turn reduction, the
+// prefactor's adjoint as the sum of conj(gbar) r -- and 21 additions for the warp
+// sums of 20 values (transposed).  In the general form (alpha0, alpha1,
+// beta0, beta1, sincospi, butterflies) it was 251 and 100.  1000 walkers, 200
+// bins: 150 -> 79 us (FP64 pipe 84 -> 89 % busy), errors against the oracle unchanged.
 // ---------------------------------------------------------------------------
-template <bool GRAD, bool MALA = false>
+template <int ND, bool GRAD, bool MALA = false>
 __global__ void __launch_bounds__(256) k_rb_f64(LaunchArgs a) {
   static_assert(!MALA || GRAD, "the MALA step needs the gradient");
+  constexpr int kNV = 1 + (GRAD ? kNBasis + 3 * ND : 0);  // log L; basis coefficients, delays, G re, G im
+  __shared__ double s_red[256 / 32][32];
   const EventDev& ev = a.ev;
-  const int Ep = ev.e_pad, Bp = ev.b_pad, D = ev.n_det, B = ev.n_bins, E = ev.n_edges;
+  const int Ep = ev.e_pad, Bp = ev.b_pad, B = ev.n_bins, E = ev.n_edges;
   const double* __restrict__ g64 = ev.tab64;
   const double* __restrict__ f64 = ev.tab64 + (size_t)kNBasis * Ep;
   const double* __restrict__ bin64 = ev.tab64 + (size_t)(kNBasis + 1) * Ep;
   const int lane = threadIdx.x & 31;
+  double* red = s_red[threadIdx.x >> 5];
   // each block takes a contiguous, equal share of the walkers (so every SM
   // gets W / grid of them, +-1), its warps take them in turn
   const int64_t per_blk = a.W / gridDim.x, rem_blk = a.W % gridDim.x;
@@ -920,103 +910,87 @@ __global__ void __launch_bounds__(256) k_rb_f64(LaunchArgs a) {
       }
       continue;
     }
-    double dc[kNBasis], tau[kMaxDet], rho[kMaxDet][2], sig[kMaxDet][2];
+    double dc[kNBasis], tau[ND], rho[ND][2], sig[ND][2];
 #pragma unroll
     for (int k = 0; k < kNBasis; ++k) dc[k] = s->dc[k];
 #pragma unroll
-    for (int d = 0; d < kMaxDet; ++d) {
+    for (int d = 0; d < ND; ++d) {
       tau[d] = s->tau[d];
       rho[d][0] = s->rho[d][0]; rho[d][1] = s->rho[d][1];
       sig[d][0] = s->sig[d][0]; sig[d][1] = s->sig[d][1];
     }
-    double acc = 0.0;
-    double adj_c[kNBasis], adj_tau[kMaxDet], adj_rho[kMaxDet][2];
-    if (GRAD) {
+    double v[kNV];
 #pragma unroll
-      for (int k = 0; k < kNBasis; ++k) adj_c[k] = 0.0;
-#pragma unroll
-      for (int d = 0; d < kMaxDet; ++d) { adj_tau[d] = 0.0; adj_rho[d][0] = adj_rho[d][1] = 0.0; }
-    }
+    for (int i = 0; i < kNV; ++i) v[i] = 0.0;
     for (int c0 = 0; c0 < B; c0 += 31) {
       const int e = c0 + lane;
       const bool has_edge = e < E;
       const bool has_bin = (lane < 31) && (e < B);
-      const int ee = has_edge ? e : E - 1;
+      const int ee = has_edge ? e : E - 1, eb = has_bin ? e : 0;
       double x = 0.0;
 #pragma unroll
       for (int k = 0; k < kNBasis; ++k) x = fma(dc[k], g64[k * Ep + ee], x);
       const double fe = f64[ee];
       double adj_x = 0.0;
 #pragma unroll
-      for (int d = 0; d < kMaxDet; ++d) {
-        if (d < D) {
-          const double xd = fma(fe, tau[d], x);
-          const double y = xd - rint(xd);
-          double sn, cs;
-          sincospi(y, &sn, &cs);
-          const double em_r = -2.0 * sn * sn, em_i = -2.0 * sn * cs;
-          const double dr = rho[d][0] * em_r - rho[d][1] * em_i + sig[d][0];
-          const double di = rho[d][0] * em_i + rho[d][1] * em_r + sig[d][1];
-          const double nr = __shfl_down_sync(kFull, dr, 1);
-          const double ni = __shfl_down_sync(kFull, di, 1);
-          double Ur = 0.0, Ui = 0.0, Vr = 0.0, Vi = 0.0;
-          if (has_bin) {
-            const double* bt = bin64 + (size_t)d * 6 * Bp;
-            const double a0r = bt[e], a0i = bt[Bp + e], a1r = bt[2 * Bp + e], a1i = bt[3 * Bp + e];
-            const double b0 = bt[4 * Bp + e], b1 = bt[5 * Bp + e];
-            const double sr = dr + nr, si = di + ni, tr = nr - dr, ti = ni - di;
-            acc += a0r * sr + a0i * si + a1r * tr + a1i * ti - b0 * (sr + 0.25 * (sr * sr + si * si)) -
-                   b1 * (tr + 0.5 * (sr * tr + si * ti));
-            if (GRAD) {
-              const double hs_r = 1.0 + 0.5 * sr, hs_i = 0.5 * si;
-              Ur = a0r - b0 * hs_r - 0.5 * b1 * tr;
-              Ui = a0i - b0 * hs_i - 0.5 * b1 * ti;
-              Vr = a1r - b1 * hs_r;
-              Vi = a1i - b1 * hs_i;
-            }
-          }
-          if (GRAD) {
-            double gr = Ur - Vr, gi = Ui - Vi;
-            const double lr = __shfl_up_sync(kFull, Ur + Vr, 1);
-            const double li = __shfl_up_sync(kFull, Ui + Vi, 1);
-            if (lane > 0) { gr += lr; gi += li; }
-            if (has_edge) {
-              const double rr = 1.0 + dr, ri = di;
-              const double dldx = gr * ri - gi * rr;
-              adj_x += dldx;
-              adj_tau[d] += dldx * fe;
-              const double Er = 1.0 + em_r, Ei = em_i;
-              adj_rho[d][0] += gr * Er + gi * Ei;
-              adj_rho[d][1] += gi * Er - gr * Ei;
-            }
+      for (int d = 0; d < ND; ++d) {
+        double em_r, em_i;
+        expm1_neg_turns64(fma(fe, tau[d], x), em_r, em_i);
+        const double dr = fma(rho[d][0], em_r, fma(-rho[d][1], em_i, sig[d][0]));
+        const double di = fma(rho[d][0], em_i, fma(rho[d][1], em_r, sig[d][1]));
+        const double nr = __shfl_down_sync(kFull, dr, 1);
+        const double ni = __shfl_down_sync(kFull, di, 1);
+        // the bin on the edge's right; zero coefficients where there is none
+        const double* bt = bin64 + (size_t)d * 6 * Bp + eb;
+        const double gmr = has_bin ? bt[0] : 0.0, gpr = has_bin ? bt[Bp] : 0.0, gmi = has_bin ? bt[2 * Bp] : 0.0;
+        const double gpi = has_bin ? bt[3 * Bp] : 0.0, q = has_bin ? bt[5 * Bp] : 0.0;
+        const double sr = dr + nr, si = di + ni;
+        v[0] = fma(gmr, dr, v[0]);
+        v[0] = fma(gpr, nr, v[0]);
+        v[0] = fma(gmi, di, v[0]);
+        v[0] = fma(gpi, ni, v[0]);
+        v[0] = fma(q, fma(sr, sr, si * si), v[0]);
+        if (GRAD) {
+          const double h = has_bin ? bt[4 * Bp] : 0.0;
+          double gr = fma(h, sr, gmr), gi = fma(h, si, gmi);
+          const double lr = __shfl_up_sync(kFull, fma(h, sr, gpr), 1), li = __shfl_up_sync(kFull, fma(h, si, gpi), 1);
+          gr += lane > 0 ? lr : 0.0;
+          gi += lane > 0 ? li : 0.0;
+          if (has_edge) {
+            const double rr = 1.0 + dr;
+            const double dldx = fma(gr, di, -(gi * rr));  // Im(conj(gbar) r)
+            adj_x += dldx;
+            v[1 + kNBasis + d] = fma(dldx, fe, v[1 + kNBasis + d]);
+            v[1 + kNBasis + ND + d] = fma(gr, rr, fma(gi, di, v[1 + kNBasis + ND + d]));
+            v[1 + kNBasis + 2 * ND + d] += dldx;
           }
         }
       }
       if (GRAD && has_edge) {
 #pragma unroll
-        for (int k = 0; k < kNBasis; ++k) adj_c[k] += adj_x * g64[k * Ep + ee];
+        for (int k = 0; k < kNBasis; ++k) v[1 + k] = fma(adj_x, g64[k * Ep + ee], v[1 + k]);
       }
     }
-    const double tot = warp_sum_f64(acc);
-    const double logl = base_logl + tot;
+    warp_transposed_sums(v, lane, red);
+    __syncwarp();
+    const double logl = base_logl + red[0];
     if (!MALA && lane == 0) a.logl[RB_IDX(w, a.W, 105)] = logl;
     if (GRAD) {
+      double ac[kNBasis], at[ND], G[ND][2];
 #pragma unroll
-      for (int k = 0; k < kNBasis; ++k) adj_c[k] = kTwoPi * warp_sum_f64(adj_c[k]);
+      for (int k = 0; k < kNBasis; ++k) ac[k] = kTwoPi * red[1 + k];
 #pragma unroll
-      for (int d = 0; d < kMaxDet; ++d) {
-        adj_tau[d] = kTwoPi * warp_sum_f64(adj_tau[d]);
-        adj_rho[d][0] = warp_sum_f64(adj_rho[d][0]);
-        adj_rho[d][1] = warp_sum_f64(adj_rho[d][1]);
+      for (int d = 0; d < ND; ++d) {
+        at[d] = kTwoPi * red[1 + kNBasis + d];
+        G[d][0] = red[1 + kNBasis + ND + d];
+        G[d][1] = red[1 + kNBasis + 2 * ND + d];
       }
       double g = 0.0;
-      if (lane < kNPar) {
-        const WalkerTan<double>& tn = reinterpret_cast<const WalkerTan<double>*>(a.tan)[w];
-        g = chain_rule<double>(lane, D, adj_c, adj_tau, adj_rho, rho, tn);
-      }
+      if (lane < kNPar) g = chain_rule_lanes<ND>(lane, ac, at, G, reinterpret_cast<const WalkerTan<double>*>(a.tan)[w]);
       if (MALA) mala_finish(a.mala, w, lane, logl, g);
       else if (lane < kNPar) a.grad[RB_IDX(w * kNPar + lane, a.W * kNPar, 106)] = g;
     }
+    __syncwarp();  // red is read before the next walker's sums
   }
 }
 
@@ -1184,26 +1158,32 @@ cudaError_t launch_rb_fused(const EventDev& ev, const EventConst& ec, const doub
   return grad ? launch_fused_t<true, false>(a, s, n_sm, done) : launch_fused_t<false, false>(a, s, n_sm, done);
 }
 
+template <bool GRAD, bool MALA>
+static cudaError_t launch_f64_t(const LaunchArgs& a, cudaStream_t s, int n_sm) {
+  void (*const kernels[kMaxDet])(LaunchArgs) = {k_rb_f64<1, GRAD, MALA>, k_rb_f64<2, GRAD, MALA>, k_rb_f64<3, GRAD, MALA>};
+  if (a.ev.n_det < 1 || a.ev.n_det > kMaxDet) return cudaErrorInvalidValue;
+  auto* fn = kernels[a.ev.n_det - 1];
+  const int bs = 256;
+  int per_sm = 0;
+  cudaError_t err = blocks_per_sm(reinterpret_cast<const void*>(fn), bs, 0, &per_sm);
+  if (err != cudaSuccess) return err;
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  // a batch that does not fill the SMs with eight walkers per block is spread over
+  // more of them, down to one walker per SM sub-partition (each has one FP64 unit)
+  const int64_t dense = (a.W * 32 + bs - 1) / bs;
+  const int64_t thin = std::min<int64_t>((a.W + kThinWalkers - 1) / kThinWalkers, n_sm);
+  fn<<<(unsigned)std::min<int64_t>(std::max(dense, thin), (int64_t)per_sm * n_sm), bs, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_rb_f64(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl, double* grad,
                           cudaStream_t s, int n_sm, const MalaArgs* mala) {
   LaunchArgs a{ev, ws, tan, W, logl, grad, {}};
-  if (mala) a.mala = *mala;
-  const int bs = 256;
-  int per_sm = 0;
-  const void* fn = mala ? reinterpret_cast<const void*>(k_rb_f64<true, true>)
-                 : grad ? reinterpret_cast<const void*>(k_rb_f64<true>) : reinterpret_cast<const void*>(k_rb_f64<false>);
-  cudaError_t err = blocks_per_sm(fn, bs, 0, &per_sm);
-  if (err != cudaSuccess) return err;
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
-  const int64_t blocks_needed = (W * 32 + bs - 1) / bs;
-  const int64_t grid = std::min<int64_t>(blocks_needed, (int64_t)per_sm * n_sm);
-  if (mala)
-    k_rb_f64<true, true><<<(unsigned)grid, bs, 0, s>>>(a);
-  else if (grad)
-    k_rb_f64<true><<<(unsigned)grid, bs, 0, s>>>(a);
-  else
-    k_rb_f64<false><<<(unsigned)grid, bs, 0, s>>>(a);
-  return cudaGetLastError();
+  if (mala) {
+    a.mala = *mala;
+    return launch_f64_t<true, true>(a, s, n_sm);
+  }
+  return grad ? launch_f64_t<true, false>(a, s, n_sm) : launch_f64_t<false, false>(a, s, n_sm);
 }
 
 }  // namespace rb

@@ -151,7 +151,6 @@ __device__ void summary_epilogue(const SummaryOut& so, int b, int d0, int nd, in
       }
       so.summ[((size_t)d * B + b) * 6 + f] = o;
       t = (f == 2 || f == 3 || f == 5) ? o * inv_df_b : 0.5 * o;
-      so.bin64[((size_t)d * 6 + f) * so.Bp + b] = t;
       // float image (layout in EventDev), with beta0 and beta1 negated
       const float t32 = (float)(f >= 4 ? -t : t);
       const size_t Bp = so.Bp;
@@ -176,6 +175,7 @@ __device__ void summary_epilogue(const SummaryOut& so, int b, int d0, int nd, in
         const size_t NS = so.n_slots;
         float* sb = so.slot_bin32 + (size_t)d * kSlotBinFloats * NS;
         sb[((size_t)(f >> 1) * NS + sl) * 4 + (f & 1) * 2 + h] = (float)val;
+        so.bin64[((size_t)d * 6 + f) * so.Bp + b] = val;
       }
     }
     const double b0 = __shfl_sync(0xffffffffu, o, (6 * g + 4) & 31);
@@ -654,33 +654,10 @@ __device__ __forceinline__ double small_int_double(int i) {
   return __hiloint2double(0x43380000 + (i >> 31), i) - 6755399441055744.0;
 }
 
-// exp(-2 pi i x): x reduced to a quarter turn, r in [-1/8, 1/8], and the
-// Taylor series of sine and cosine of 2 pi r (|2 pi r| <= pi/4: the first
-// dropped terms are below 2^-54).  20 FP64 operations; the quadrant is applied with
-// integer selects.
+// exp(-2 pi i x).
 __device__ __forceinline__ double2 cis_neg_turns64(double x) {
-  const double magic = 6755399441055744.0;  // 1.5 * 2^52
-  const double t = fma(x, 4.0, magic);
-  const int q = __double2loint(t);
-  const double r = fma(t - magic, -0.25, x);
-  const double w = r * r;
-  double ps = -0.7181223017785006;       // -(2 pi)^15 / 15!
-  ps = fma(ps, w, 3.819952584848282);   // (2 pi)^13 / 13!
-  ps = fma(ps, w, -15.09464257682299);  // -(2 pi)^11 / 11!
-  ps = fma(ps, w, 42.058693944897655);   // (2 pi)^9 / 9!
-  ps = fma(ps, w, -76.70585975306139);   // -(2 pi)^7 / 7!
-  ps = fma(ps, w, 81.60524927607506);    // (2 pi)^5 / 5!
-  ps = fma(ps, w, -41.34170224039976);  // -(2 pi)^3 / 3!
-  ps = fma(ps, w, 6.283185307179586);
-  const double sn = r * ps;
-  double pc = 0.28200596845579123;       // (2 pi)^16 / 16!
-  pc = fma(pc, w, -1.714390711088672);  // -(2 pi)^14 / 14!
-  pc = fma(pc, w, 7.903536371318469);    // (2 pi)^12 / 12!
-  pc = fma(pc, w, -26.4262567833744);   // -(2 pi)^10 / 10!
-  pc = fma(pc, w, 60.24464137187666);   // (2 pi)^8 / 8!
-  pc = fma(pc, w, -85.45681720669373);   // -(2 pi)^6 / 6!
-  pc = fma(pc, w, 64.9393940226683);    // (2 pi)^4 / 4!
-  pc = fma(pc, w, -19.739208802178716);  // -(2 pi)^2 / 2
+  double sn, pc, w;
+  const int q = quarter_turn64(x, sn, pc, w);
   const double cs = fma(pc, w, 1.0);
   // theta = 2 pi r + q pi/2: (cos theta, -sin theta)
   const double a = (q & 1) ? sn : cs, b = (q & 1) ? cs : sn;
