@@ -27,7 +27,8 @@
 //                    since F+ = D:(XX - YY) cancels)
 //            warp 4: delay differences
 //   phase 3  warps 1-3: prefactor ratio rho_d and rho_d - 1
-//   (gradient) warps 5, 6: tangents in FP32 (mixed) or FP64 dual numbers.
+//   (gradient) the warps after these: tangents, FP32 dual numbers (mixed modes)
+//            or written out in FP64 from the phase-1 results.
 // Every role is a noinline function, so a walker at theta_ref reproduces the
 // fiducial values bit for bit (the reference kernel runs the same roles).
 #include <type_traits>
@@ -168,10 +169,170 @@ struct SetupSmem {
   int valid[kSetupWalkers];
 };
 
+// ---------------------------------------------------------------------------
+// FP64 tangents, written out (the FP64 set-up's warps 5-9): from the phase-1
+// results in shared memory, without the structurally zero terms that dual
+// numbers carry.  An FP64 warp instruction costs ~65 clocks, and the dual-number
+// form took ~1750 of them per detector and ~575 per pair of intrinsic
+// parameters; here ~130 per detector, ~130 for q and ~90 for the others.  1000
+// walkers, 3 detectors: set-up with the gradient 40.3 -> 19.4 us.
+// ---------------------------------------------------------------------------
+constexpr int kTan64Warps = 2 + kMaxDet;
+constexpr int kTan64Threads = kRoleThreads + kTan64Warps * 32;
+__device__ __forceinline__ void tangents_go() { asm volatile("bar.arrive 2, %0;" ::"n"(kTan64Threads) : "memory"); }
+__device__ __forceinline__ void tangents_wait() { asm volatile("bar.sync 2, %0;" ::"n"(kTan64Threads) : "memory"); }
+
+// Powers of a = (pi M)^1/3 times N0, ln(pi M), and the parts of c_5.
+struct Pow64 {
+  double N2, N3, N4, N5, N6, N7, N10, N12, u;
+};
+__device__ __forceinline__ Pow64 pow64(const SetupSmem& S, int l) {
+  Pow64 p;
+  const double a = S.a1[l] * S.a2[l], a2 = a * a, a4 = a2 * a2, N0 = S.N0[l];
+  p.N2 = N0 * a2;
+  p.N3 = p.N2 * a;
+  p.N4 = N0 * a4;
+  p.N5 = p.N4 * a;
+  p.N6 = p.N4 * a2;
+  p.N7 = p.N6 * a;
+  p.N10 = p.N6 * a4;
+  p.N12 = p.N10 * a2;
+  p.u = S.lnMc[l] - 0.6 * S.lneta[l];
+  return p;
+}
+constexpr double kC5 = -6848.0 / 21.0, kC6 = -6848.0 / 63.0, kLn4 = 1.3862943611198906;
+constexpr double kPhi0Const = 1.0 + 1.5 * 1.791759469228055;  // 1 + 3/2 ln 6
+
+// d / d(Mc, chi1, chi2, Lambda1, Lambda2): c_k goes as Mc^(m/3 - 5/3) (m the power of a),
+// and linearly with the spin and tidal terms.
+__device__ void tangents64_mass(const SetupSmem& S, int l, WalkerTan<double>& o) {
+  const Pow64 p = pow64(S, l);
+  const double Mc = S.th[0][l], q = S.th[1][l], chi1 = S.th[2][l], chi2 = S.th[3][l], eta = S.eta[l];
+  const double iM = 1.0 / Mc, iM3 = iM * (1.0 / 3.0);
+  const double c5 = p.N6 * fma(kC5, fma(p.u, 1.0 / 3.0, kLn4), S.phi[4][l]), c6 = p.N6 * kC6;
+  o.dc[0][0] = S.N0[l] * (-5.0 * iM3);
+  o.dc[1][0] = p.N2 * S.phi[0][l] * (-3.0 * iM3);
+  o.dc[2][0] = p.N3 * S.phi[1][l] * (-2.0 * iM3);
+  o.dc[3][0] = p.N4 * S.phi[2][l] * -iM3;
+  o.dc[4][0] = 0.0;
+  o.dc[5][0] = (c5 + 3.0 * c6) * iM3;
+  o.dc[6][0] = c6 * iM3;
+  o.dc[7][0] = p.N7 * S.phi[5][l] * (2.0 * iM3);
+  o.dc[8][0] = p.N10 * S.phi[6][l] * (5.0 * iM3);
+  o.dc[9][0] = p.N12 * S.phi[7][l] * (7.0 * iM3);
+  o.dphi0[0] = p.N5 * S.phi[3][l] * iM;
+  o.lnamp_Mc = (5.0 / 6.0) * iM;
+  o.lnamp_dL = -1.0 / S.th[6][l];
+  const double X1 = 1.0 / (1.0 + q), X2 = q * X1;
+  const double X1_2 = X1 * X1, X2_2 = X2 * X2, e75 = 75.0 * eta, es = eta * (474.0 / 48.0);
+#pragma unroll
+  for (int k = 0; k < kNBasis; ++k)
+#pragma unroll
+    for (int j = 2; j < kNTanIntr; ++j)
+      if (!((k == 2 || k == 3) && j < 4) && !(k >= 8 && j >= 4)) o.dc[k][j] = 0.0;
+  // phi3 = -16 pi + 4 beta, phi4 = ... - 10 sigma
+  o.dc[2][2] = p.N3 * ((1.0 / 3.0) * fma(113.0, X1_2, e75));
+  o.dc[2][3] = p.N3 * ((1.0 / 3.0) * fma(113.0, X2_2, e75));
+  o.dc[3][2] = p.N4 * (-10.0 * fma(es, chi2, (486.0 / 48.0) * X1_2 * chi1));
+  o.dc[3][3] = p.N4 * (-10.0 * fma(es, chi1, (486.0 / 48.0) * X2_2 * chi2));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double X = i ? X2 : X1, Xs = i ? X2_2 : X1_2, X4 = Xs * Xs;
+    o.dc[8][4 + i] = p.N10 * (fma(264.0, X, -288.0) * X4);
+    o.dc[9][4 + i] = p.N12 * (X4 * fma(fma(fma(-325.0 / 7.0, X, 5715.0 / 14.0), X, 4595.0 / 28.0), X, -15895.0 / 28.0));
+  }
+}
+
+// d / dq: eta' = (1 - q) / (1 + q)^3, (ln eta)' = (1 - q) / (q (1 + q)), X1' = -X1^2 = -X2',
+// (ln a)' = -(ln eta)' / 5, u' = -3/5 (ln eta)'.
+__device__ void tangents64_q(const SetupSmem& S, int l, WalkerTan<double>& o) {
+  const Pow64 p = pow64(S, l);
+  const double q = S.th[1][l], chi1 = S.th[2][l], chi2 = S.th[3][l], L1 = S.th[4][l], L2 = S.th[5][l], eta = S.eta[l];
+  const double X1 = 1.0 / (1.0 + q), X2 = q * X1, X1_2 = X1 * X1;
+  const double dle = (1.0 - q) * X1 / q, de = eta * dle, dla = -0.2 * dle, du = -0.6 * dle;
+  const double dX1 = -X1_2, dX2 = X1_2;
+  const double d2 = (55.0 / 9.0) * de;
+  const double d3 = (1.0 / 3.0) * fma(chi1, fma(226.0 * X1, dX1, 75.0 * de), chi2 * fma(226.0 * X2, dX2, 75.0 * de));
+  const double ds = fma(de * (474.0 / 48.0), chi1 * chi2, (486.0 / 48.0) * fma(X1 * dX1, chi1 * chi1, X2 * dX2 * (chi2 * chi2)));
+  const double d4 = fma(fma(3085.0 / 36.0, eta, 27145.0 / 504.0), de, -10.0 * ds);
+  const double d5 = (-kPi * 65.0 / 9.0) * de;
+  const double d6 = fma(fma(-127825.0 / 432.0, eta, 76055.0 / 864.0), eta,
+                        -15737765635.0 / 3048192.0 + (2255.0 / 12.0) * kPi * kPi) * de;
+  const double d7 = fma(-kPi * 74045.0 / 378.0, eta, kPi * 378515.0 / 1512.0) * de;
+  double d10 = 0.0, d12 = 0.0;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double X = i ? X2 : X1, LX = (i ? L2 * dX2 : L1 * dX1) * (X * X * X);
+    d10 = fma(fma(1320.0, X, -1152.0), LX, d10);
+    d12 = fma(fma(fma(fma(-7.0 * 325.0 / 7.0, X, 6.0 * 5715.0 / 14.0), X, 5.0 * 4595.0 / 28.0), X, -4.0 * 15895.0 / 28.0), LX, d12);
+  }
+  const double c5 = fma(kC5, fma(p.u, 1.0 / 3.0, kLn4), S.phi[4][l]);  // c_5 / N6
+  o.dc[0][1] = 0.0;
+  o.dc[1][1] = p.N2 * fma(2.0 * dla, S.phi[0][l], d2);
+  o.dc[2][1] = p.N3 * fma(3.0 * dla, S.phi[1][l], d3);
+  o.dc[3][1] = p.N4 * fma(4.0 * dla, S.phi[2][l], d4);
+  const double t5 = fma(5.0 * dla, S.phi[3][l], d5);
+  o.dc[4][1] = p.N5 * t5;
+  o.dc[5][1] = p.N6 * fma(6.0 * dla, c5, fma(kC6, du, d6));
+  o.dc[6][1] = p.N6 * (6.0 * kC6 * dla);
+  o.dc[7][1] = p.N7 * fma(7.0 * dla, S.phi[5][l], d7);
+  o.dc[8][1] = p.N10 * fma(10.0 * dla, S.phi[6][l], d10);
+  o.dc[9][1] = p.N12 * fma(12.0 * dla, S.phi[7][l], d12);
+  o.dphi0[1] = p.N5 * fma(t5, kPhi0Const + p.u, S.phi[3][l] * du);
+}
+
+// One detector's ln P and delay with respect to (iota, psi, ra, dec).  With
+// F+ = X.DX - Y.DY, Fx = 2 X.DY and the polarisation frame's derivatives
+//   d(X, Y)/dpsi = (Y, -X),  d(X, Y)/dra = (z x X, z x Y),  d(X, Y)/ddec = (-sin psi n, -cos psi n):
+//   dF+/dpsi = 2 Fx, dFx/dpsi = -2 F+,  dF+ = 2 (DX.dX - DY.dY),  dFx = 2 (DY.dX + DX.dY).
+__device__ void tangents64_det(const DetGeom& g, const SetupSmem& S, int l, double si, int d, WalkerTan<double>& o) {
+  const double sd = S.sky[0][l], cd = S.sky[1][l], sg = -S.sky[2][l], cg = S.sky[3][l];  // g = gmst - ra
+  const double sp = S.ori[0][l], cp = S.ori[1][l], ci = S.ori[2][l];
+  const double X[3] = {-cp * sg - sp * cg * sd, -cp * cg + sp * sg * sd, sp * cd};
+  const double Y[3] = {sp * sg - cp * cg * sd, sp * cg + cp * sg * sd, cp * cd};
+  const double n[3] = {cd * cg, -cd * sg, sd};
+  double DX[3], DY[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    DX[i] = g.D[i][0] * X[0] + g.D[i][1] * X[1] + g.D[i][2] * X[2];
+    DY[i] = g.D[i][0] * Y[0] + g.D[i][1] * Y[1] + g.D[i][2] * Y[2];
+  }
+  const double fp = (X[0] * DX[0] + X[1] * DX[1] + X[2] * DX[2]) - (Y[0] * DY[0] + Y[1] * DY[1] + Y[2] * DY[2]);
+  const double fx = 2.0 * (X[0] * DY[0] + X[1] * DY[1] + X[2] * DY[2]);
+  const double nX = n[0] * DX[0] + n[1] * DX[1] + n[2] * DX[2], nY = n[0] * DY[0] + n[1] * DY[1] + n[2] * DY[2];
+  // dra: z x X = (-X1, X0, 0)
+  const double fp_r = 2.0 * ((DX[1] * X[0] - DX[0] * X[1]) - (DY[1] * Y[0] - DY[0] * Y[1]));
+  const double fx_r = 2.0 * ((DY[1] * X[0] - DY[0] * X[1]) + (DX[1] * Y[0] - DX[0] * Y[1]));
+  const double fp_d = 2.0 * (cp * nY - sp * nX), fx_d = -2.0 * (sp * nY + cp * nX);
+  const double ip = 0.5 * fma(ci, ci, 1.0);  // (1 + cos^2 iota) / 2
+  const double Pr = fp * ip, Pi = -fx * ci;
+  const double iden = 1.0 / (Pr * Pr + Pi * Pi);
+  const double dPr[4] = {-fp * ci * si, 2.0 * fx * ip, fp_r * ip, fp_d * ip};
+  const double dPi[4] = {fx * si, 2.0 * fp * ci, -fx_r * ci, -fx_d * ci};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {  // d ln P = dP conj(P) / |P|^2
+    o.dlnP[d][j][0] = (dPr[j] * Pr + dPi[j] * Pi) * iden;
+    o.dlnP[d][j][1] = (dPi[j] * Pr - dPr[j] * Pi) * iden;
+  }
+  o.dtd[d][0] = (cd * sg * g.r[0] + cd * cg * g.r[1]) * (-1.0 / kClight);
+  o.dtd[d][1] = (-sd * cg * g.r[0] + sd * sg * g.r[1] + cd * g.r[2]) * (-1.0 / kClight);
+}
+
+__device__ void tangent64_warp(const SetupSmem& S, const EventConst& ec, double iota, WalkerTan<double>& o, int which) {
+  const int l = threadIdx.x & 31;
+  const int d = which - 2;
+  const double si = d >= 0 && d < ec.n_det ? sin(iota) : 0.0;  // alongside phase 1
+  tangents_wait();
+  if (which == 0) tangents64_mass(S, l, o);
+  else if (which == 1) tangents64_q(S, l, o);
+  else if (d < ec.n_det) tangents64_det(ec.det[d], S, l, si, d, o);  // entries of detectors beyond n_det are never read
+}
+
 // Runs phases 1 and 2 for the walkers of this block and leaves the absolute
 // values in shared memory.  Warps 0-4 (and only they) must call it.
+// signal: warps waiting in tangents_wait() are let go after phase 1.
 __device__ void setup_absolute(const double* __restrict__ theta, int64_t w0, int64_t W, const EventConst& ec,
-                               SetupSmem& S) {
+                               SetupSmem& S, bool signal = false) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < kNPar * kSetupWalkers; i += kRoleThreads) {
     const int l = i / kNPar, j = i % kNPar;
@@ -202,6 +363,7 @@ __device__ void setup_absolute(const double* __restrict__ theta, int64_t w0, int
     for (int k = 0; k < 3; ++k) S.ori[k][l] = o[k];
   }
   roles_sync();
+  if (signal) tangents_go();
   if (warp == 0) {
     double phi[8], c[kNBasis], phi0;
     for (int k = 0; k < 8; ++k) phi[k] = S.phi[k][l];
@@ -250,24 +412,32 @@ __global__ void __launch_bounds__(7 * 32) k_ref_values(const double* theta, Even
 // Batch set-up in FP64 for the FP64 paths: RB_FP64 writes WalkerF64 (+
 // double tangents), RB_MIXED_F64PHASE writes WalkerF64 (+ float tangents).
 // (RB_MIXED uses the float-float set-up, k_setup_dd.)
+template <int MODE>
+constexpr int setup_threads(bool grad) {
+  return !grad ? kRoleThreads : MODE == RB_FP64 ? kTan64Threads : kRoleThreads + kTanWarps * 32;
+}
 template <int MODE, bool GRAD>
-__global__ void __launch_bounds__((5 + kTanWarps) * 32) k_setup(const double* __restrict__ theta, int64_t W, EventConst ec,
+__global__ void __launch_bounds__(setup_threads<MODE>(GRAD)) k_setup(const double* __restrict__ theta, int64_t W, EventConst ec,
                                                   const RefValues* __restrict__ ref, void* __restrict__ ws_out,
                                                   void* __restrict__ tan_out) {
   static_assert(MODE == RB_FP64 || MODE == RB_MIXED_F64PHASE, "RB_MIXED uses the float-float set-up");
-  using TanT = typename std::conditional<MODE == RB_FP64, double, float>::type;
   __shared__ SetupSmem S;
   const int64_t w0 = (int64_t)blockIdx.x * kSetupWalkers;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t w = w0 + lane;
   const bool mine = w < W;
   if (warp >= 5) {
-    // tangents (gradient only) do not depend on the FP64 phases: these warps
-    // run them alongside and take no part in the role barriers
-    if (GRAD) tangent_warp<TanT>(theta, W, w0, ec, static_cast<WalkerTan<TanT>*>(tan_out) + w0, warp - 5);
+    // tangents (gradient only): these warps take no part in the role barriers
+    // (the FP64 ones start from the phase-1 results)
+    if constexpr (GRAD && MODE == RB_FP64) {
+      const int64_t wc = mine ? w : W - 1;  // pad lanes repeat the last walker's record
+      tangent64_warp(S, ec, theta[wc * kNPar + 9], static_cast<WalkerTan<double>*>(tan_out)[wc], warp - 5);
+    } else if constexpr (GRAD) {
+      tangent_warp<float>(theta, W, w0, ec, static_cast<WalkerTan<float>*>(tan_out) + w0, warp - 5);
+    }
     return;
   }
-  setup_absolute(theta, w0, W, ec, S);
+  setup_absolute(theta, w0, W, ec, S, GRAD && MODE == RB_FP64);
   const Values& r = ref->v;
   const int l = lane;
   if (warp == 0) {
@@ -408,7 +578,7 @@ static cudaError_t launch_setup_t(const double* theta, int64_t W, const EventCon
                                   void* tan, bool grad, cudaStream_t s) {
   const unsigned grid = (unsigned)((W + kSetupWalkers - 1) / kSetupWalkers);
   if (grad)
-    k_setup<MODE, true><<<grid, (5 + kTanWarps) * 32, 0, s>>>(theta, W, ec, ref, ws, tan);
+    k_setup<MODE, true><<<grid, setup_threads<MODE>(true), 0, s>>>(theta, W, ec, ref, ws, tan);
   else
     k_setup<MODE, false><<<grid, 5 * 32, 0, s>>>(theta, W, ec, ref, ws, tan);
   return cudaGetLastError();
