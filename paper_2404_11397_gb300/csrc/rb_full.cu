@@ -31,15 +31,26 @@
 // fixed tree of float pairs); the groups are added in FP64.  The groups depend
 // on the grid alone, so a walker's result does not depend on the batch.
 //
-// Bound: the FP32 pipe (71 % busy, 51 % of the issue slots; ~80 operations per
-// point and walker with 3 detectors, and the chunk coefficients).  One chunk per lane in scalar FP32
-// (detectors 0 and 1 paired), in waves of slices, issued 119 warp instructions
-// per 32 points (71 % of the slots, pipe 63 %) against 72 now.  512 walkers, 260
-// k points, 3 detectors: call 588 -> 513 us; 7 walkers 83 -> 36 us.
+// Phase: the first three Taylor terms X0 + X1 j + X2 j^2 run in integers, in units
+// of 2^-32 turns: they wrap at whole turns by themselves, a point costs two integer
+// additions (first and second differences, on a pipe that is idle otherwise), and
+// what the units drop goes into the FP32 polynomial of the remaining terms.  In float
+// pairs (products, two-sums, reductions) these terms were 31 of a point's 79 FP32
+// operations; 3 are left.  Segments whose orders beyond 4 stay below 2^-36 turns (and
+// the terms from order 3 below 2^-10, so that the sum needs no reduction) leave those
+// orders out: nearly all above ~80 Hz; the walkers of a block decide for themselves.
+//
+// Bound: the FP32 pipe (~50 operations per point and walker with 3 detectors, 24 of
+// them the detectors' products, 18 the sine and cosine, and ~12 for the chunk
+// coefficients).  512 walkers, 260 k points, 3 detectors: call 512 -> 416 us; with one
+// chunk per lane in scalar FP32, in waves of slices, it was 588.  The phases agree with
+// the float-pair form to its last bit at nearly every point: results differ by
+// 1e-12 to 2e-10, errors against FP64 sums unchanged.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "rb.h"
 #include "rb_api_internal.h"
@@ -54,7 +65,7 @@ constexpr int kSegP = kSegC * kChunk;     // points per segment
 constexpr int kWtRow = kSegC / 2 + 1;     // transposed data row (padded: conflict-free stores)
 constexpr int kQPad = kQRow + 4;          // staged chunk-matrix row (padded: 16-byte loads of row l by lane l without conflicts)
 constexpr int full_smem(int nd) {
-  return (int)(sizeof(float4) * (nd * kChunk * kWtRow + nd * kFullWarps * kChunk + 2 * kChunk) + sizeof(float) * kSegC * kQPad);
+  return (int)(sizeof(float4) * (nd * kChunk * kWtRow + nd * kFullWarps * kChunk) + sizeof(float2) * kChunk + sizeof(float) * kSegC * kQPad);
 }
 
 // Segments per group: up to 64 groups.
@@ -78,6 +89,18 @@ __device__ __forceinline__ void ff_level(const f2x (&in)[N], f2x (&out)[M], int 
   }
 }
 
+// hi + lo turns, mod 1, as an integer i in units of 2^-32 turns and the rest, e
+// turns (|e| <= 2^-32): both parts' fractions times 2^32 are integers or below
+// 2^24, so that i's conversions back are exact.
+__device__ __forceinline__ void turns_fixed(float hi, float lo, unsigned& i, float& e) {
+  float a = 0x1p32f * pv::frac1(hi), b = 0x1p32f * pv::frac1(lo);
+  a = a == 0x1p31f ? -0x1p31f : a;  // +1/2 turn is out of the integers' range (a NaN stays one)
+  b = b == 0x1p31f ? -0x1p31f : b;
+  const int ia = __float2int_rn(a), ib = __float2int_rn(b);
+  e = 0x1p-32f * ((a - (float)ia) + (b - (float)ib));
+  i = (unsigned)ia + (unsigned)ib;
+}
+
 // Per group of segments and walker: the group's part of Z_d (complex, 3
 // detectors) as FP64 in zout[group][w][6].  ND = number of detectors.
 template <int ND>
@@ -89,19 +112,18 @@ __global__ void __launch_bounds__(kFullThreads, 2) k_full_z(const float2* __rest
   // dynamic shared memory: the segment's data times f^-7/6, transposed: for
   // detector d and offset j, [d][j][l] holds {re, re', im, im'} of chunks l and
   // l + 32 (wt); per warp the walker's offset factors exp(2 pi i (j - 16) df
-  // tau_d) as {re, re, im, im} (tp[warp][j][d]); the offsets' powers {j, j, j^2,
-  // j^2}, {j^3, j^3, 0, 0} of j - 16 (jt); the segment's chunk matrices (qs)
+  // tau_d) as {re, re, im, im} (tp[warp][j][d]); the offsets {j - 16, j - 16}
+  // (jt); the segment's chunk matrices (qs)
   extern __shared__ __align__(16) unsigned char smem_full[];
   float4 (*wt)[kChunk][kWtRow] = reinterpret_cast<float4 (*)[kChunk][kWtRow]>(smem_full);
   float4 (*tp)[kChunk][ND] = reinterpret_cast<float4 (*)[kChunk][ND]>(wt + ND);
-  float4 (*jt)[2] = reinterpret_cast<float4 (*)[2]>(tp + kFullWarps);
+  float2* jt = reinterpret_cast<float2*>(tp + kFullWarps);
   float* qs = reinterpret_cast<float*>(jt + kChunk);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n_seg = (n_chunks + kSegC - 1) / kSegC, gs = group_segments(n_seg), n_groups = (n_seg + gs - 1) / gs;
   if (warp == 0) {
     const float jf = small_int_float(lane - kChunk / 2);
-    jt[lane][0] = make_float4(jf, jf, jf * jf, jf * jf);
-    jt[lane][1] = make_float4(jf * jf * jf, jf * jf * jf, 0.f, 0.f);
+    jt[lane] = make_float2(jf, jf);
   }
   // the (walker octet, group) pairs, octet-major, in equal contiguous shares
   const int64_t units = (W + kFullWarps - 1) / kFullWarps * n_groups;
@@ -163,29 +185,33 @@ __global__ void __launch_bounds__(kFullThreads, 2) k_full_z(const float2* __rest
         for (int d = 0; d < ND; ++d) wt[d][jj][c] = make_float4(v[0][d].x, v[1][d].x, v[0][d].y, v[1][d].y);
       }
       __syncthreads();  // wt complete
-      if (!valid) continue;
-      // the walker's coefficients of the lane's chunks (X0 with Phi0, whole turns
-      // dropped); a chunk past the last has zero rows and zero data
+      if (!valid) continue;  // the whole warp
+      // the walker's coefficients of the lane's chunks (X0 with Phi0); a chunk past
+      // the last has zero data and the first chunk's row (chunk l) or zeros (chunk l + 32)
       const bool in0 = lane < nc, in1 = lane + kSegC / 2 < nc;
-      if (!in0) continue;
-      const float* r0 = qs + lane * kQPad;
-      const float* r1 = r0 + (kSegC / 2) * kQPad;
+      const float* r0 = qs + (in0 ? lane : 0) * kQPad;
+      const float* r1 = qs + (lane + kSegC / 2) * kQPad;
       // float4 i of the two rows
       auto row4 = [&](int i, float4& a, float4& b) {
         a = reinterpret_cast<const float4*>(r0)[i];
         b = in1 ? reinterpret_cast<const float4*>(r1)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
       };
       float2 X0h = pv::splat<float2>(wa.phi0t[0]), X0l = pv::splat<float2>(wa.phi0t[1]);
-      float2 X1h = make_float2(0.f, 0.f), X1l = X1h, X2h = X1h, X2l = X1h, xn[kOrd - 2];
-#pragma unroll
-      for (int n = 0; n < kOrd - 2; ++n) xn[n] = make_float2(0.f, 0.f);
+      float2 X1h = make_float2(0.f, 0.f), X1l = X1h, X2h = X1h, X2l = X1h;
+      float2 s_abs = X1h, g_lf = X1h, g_cf = X1h;  // the terms' moduli; ln f_c, f_c^1/3
       float4 a, b;
 #pragma unroll
       for (int k = 0; k < kNBasis; ++k) {
         const float2 ch = pv::splat<float2>(wa.chat[k][0]), cl = pv::splat<float2>(wa.chat[k][1]);
         row4(kQ01 / 4 + k, a, b);
-        pv::fma_acc(ch, cl, make_float2(a.x, b.x), make_float2(a.y, b.y), X0h, X0l);
+        const float2 g = make_float2(a.x, b.x);
+        pv::fma_acc(ch, cl, g, make_float2(a.y, b.y), X0h, X0l);
         pv::fma_acc(ch, cl, make_float2(a.z, b.z), make_float2(a.w, b.w), X1h, X1l);
+        if (k == 4) g_lf = make_float2(fabsf(g.x), fabsf(g.y));
+        if (k == 5) g_cf = g;
+        const float2 cabs = pv::splat<float2>(fabsf(wa.chat[k][0]));
+        if (k == 4) s_abs = pv::add(s_abs, cabs);
+        s_abs = pv::fma(cabs, k == 6 ? pv::fma(g_lf, g_cf, g_cf) : make_float2(fabsf(g.x), fabsf(g.y)), s_abs);
         if (k % 2 == 0) {
           const float2 ch1 = pv::splat<float2>(wa.chat[k + 1][0]), cl1 = pv::splat<float2>(wa.chat[k + 1][1]);
           row4(kQ2 / 4 + k / 2, a, b);
@@ -193,52 +219,88 @@ __global__ void __launch_bounds__(kFullThreads, 2) k_full_z(const float2* __rest
           pv::fma_acc(ch1, cl1, make_float2(a.z, b.z), make_float2(a.w, b.w), X2h, X2l);
         }
       }
+      // X0, X1, X2 mod 1 as integers in units of 2^-32 turns and the rest: x0 + x1 j
+      // + x2 j^2 then wraps at whole turns by itself, exactly
+      unsigned x[2], d1[2], d2[2];
+      float2 e0, e1, e2;
+      {
+        unsigned i0[2], i1[2], i2[2];
+        turns_fixed(X0h.x, X0l.x, i0[0], e0.x);
+        turns_fixed(X0h.y, X0l.y, i0[1], e0.y);
+        turns_fixed(X1h.x, X1l.x, i1[0], e1.x);
+        turns_fixed(X1h.y, X1l.y, i1[1], e1.y);
+        turns_fixed(X2h.x, X2l.x, i2[0], e2.x);
+        turns_fixed(X2h.y, X2l.y, i2[1], e2.y);
 #pragma unroll
-      for (int i = 0; i < (kOrd - 2) * kNBasis / 4; ++i) {  // orders 3..8, basis index fastest
-        row4(kQh / 4 + i, a, b);
-        const float2 m[4] = {make_float2(a.x, b.x), make_float2(a.y, b.y), make_float2(a.z, b.z), make_float2(a.w, b.w)};
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const int n = (4 * i + v) / kNBasis, k = (4 * i + v) % kNBasis;
-          xn[n] = pv::fma(pv::splat<float2>(wa.chat[k][0]), m[v], xn[n]);
+        for (int h = 0; h < 2; ++h) {  // value (biased by half a turn), first and second difference at j = -16
+          x[h] = i0[h] - 16u * i1[h] + 256u * i2[h] + 0x80000000u;
+          d1[h] = i1[h] - 31u * i2[h];
+          d2[h] = 2u * i2[h];
         }
       }
-      X0h = pv::frac1(X0h);
       float2 ar[ND], ai[ND];  // the chunks' sums
 #pragma unroll
       for (int d = 0; d < ND; ++d) ar[d] = ai[d] = make_float2(0.f, 0.f);
-      const float2 one = make_float2(1.f, 1.f), two = make_float2(2.f, 2.f), mtwo = make_float2(-2.f, -2.f);
-#pragma unroll 2
-      for (int jj = 0; jj < kChunk; ++jj) {
-        const float4 ja = jt[jj][0], jb = jt[jj][1];
-        const float2 j1 = make_float2(ja.x, ja.y), j2 = make_float2(ja.z, ja.w), j3 = make_float2(jb.x, jb.y);
-        // x = X0 + X1 j + X2 j^2 + j^3 (X3 + ... + X8 j^5)
-        float2 t = pv::fma(xn[5], j1, xn[4]);
+      auto points = [&](auto short_c) {
+        constexpr bool SHORT = decltype(short_c)::value;
+        constexpr int NT = SHORT ? 2 : kOrd - 2;  // orders from 3 up
+        float2 xn[NT];
 #pragma unroll
-        for (int n = 3; n >= 0; --n) t = pv::fma(t, j1, xn[n]);
-        const float2 t3 = pv::mul(t, j3);
-        const float2 p1 = pv::mul(X1h, j1), p2 = pv::mul(X2h, j2);
-        const float2 e1 = pv::fma(X1l, j1, pv::fma(X1h, j1, pv::neg(p1)));
-        const float2 e2 = pv::fma(X2l, j2, pv::fma(X2h, j2, pv::neg(p2)));
-        float2 sh = X0h, sl = X0l;
-        pv::add_acc(sh, sl, p1);
-        pv::add_acc(sh, sl, p2);
-        sl = pv::add(sl, pv::add(pv::add(e1, e2), t3));
-        const float2 y = pv::frac1(pv::frac(sh, sl));
-        float2 sn, cs;
-        pv::sincos_half(y, sn, cs);
-        const float2 zx = pv::fma(pv::mul(mtwo, sn), sn, one), zy = pv::mul(pv::mul(two, sn), cs);  // exp(+2 pi i x)
-        // offset factor times the phasor, times the data
+        for (int n = 0; n < NT; ++n) xn[n] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int d = 0; d < ND; ++d) {
-          const float4 T = tp[warp][jj][d], v = wt[d][jj][lane];
-          const float2 Tr = make_float2(T.x, T.y), Ti = make_float2(T.z, T.w);
-          const float2 vr = make_float2(v.x, v.y), vi = make_float2(v.z, v.w);
-          const float2 ur = pv::fma(zx, Tr, pv::mul(pv::neg(zy), Ti)), ui = pv::fma(zx, Ti, pv::mul(zy, Tr));
-          ar[d] = pv::fma(vr, ur, pv::fma(pv::neg(vi), ui, ar[d]));
-          ai[d] = pv::fma(vr, ui, pv::fma(vi, ur, ai[d]));
+        for (int i = 0; i < NT * kNBasis / 4; ++i) {  // basis index fastest
+          row4(kQh / 4 + i, a, b);
+          const float2 m[4] = {make_float2(a.x, b.x), make_float2(a.y, b.y), make_float2(a.z, b.z), make_float2(a.w, b.w)};
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const int n = (4 * i + v) / kNBasis, k = (4 * i + v) % kNBasis;
+            xn[n] = pv::fma(pv::splat<float2>(wa.chat[k][0]), m[v], xn[n]);
+          }
         }
-      }
+        const float2 one = make_float2(1.f, 1.f), two = make_float2(2.f, 2.f);
+#pragma unroll 2
+        for (int jj = 0; jj < kChunk; ++jj) {
+          const float2 j = jt[jj];
+          // the high 16 bits of x as floats 2^23 + h (a byte permutation), the low 16 converted
+          const float2 hb = make_float2(__uint_as_float(__byte_perm(x[0], 0x4B000000u, 0x7432)),
+                                        __uint_as_float(__byte_perm(x[1], 0x4B000000u, 0x7432)));
+          const float2 lb = make_float2(__uint2float_rn(x[0] & 0xffffu), __uint2float_rn(x[1] & 0xffffu));
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            x[h] += d1[h];
+            d1[h] += d2[h];
+          }
+          // e0 + e1 j + e2 j^2 + X3 j^3 + ...
+          float2 t = xn[NT - 1];
+#pragma unroll
+          for (int n = NT - 2; n >= 0; --n) t = pv::fma(t, j, xn[n]);
+          t = pv::fma(pv::fma(pv::fma(t, j, e2), j, e1), j, e0);
+          t = pv::fma(lb, pv::splat<float2>(0x1p-32f), t);
+          float2 y = pv::fma(pv::sub(hb, pv::splat<float2>(8421376.f)), pv::splat<float2>(0x1p-16f), t);
+          if constexpr (!SHORT) y = pv::frac1(y);
+          float2 sn, cs;
+          pv::sincos_half(y, sn, cs);
+          const float2 s2 = pv::mul(two, sn);
+          const float2 zx = pv::fma(pv::neg(s2), sn, one), zy = pv::mul(s2, cs);  // exp(+2 pi i x)
+          // offset factor times the phasor, times the data
+#pragma unroll
+          for (int d = 0; d < ND; ++d) {
+            const float4 T = tp[warp][jj][d], v = wt[d][jj][lane];
+            const float2 Tr = make_float2(T.x, T.y), Ti = make_float2(T.z, T.w);
+            const float2 vr = make_float2(v.x, v.y), vi = make_float2(v.z, v.w);
+            const float2 ur = pv::fma(zx, Tr, pv::mul(pv::neg(zy), Ti)), ui = pv::fma(zx, Ti, pv::mul(zy, Tr));
+            ar[d] = pv::fma(vr, ur, pv::fma(pv::neg(vi), ui, ar[d]));
+            ai[d] = pv::fma(vr, ui, pv::fma(vi, ur, ai[d]));
+          }
+        }
+      };
+      // |X_n j^n| <= 6 s_abs (16 u)^n (every |alpha_kn|, |beta_n| <= 5.2); 16 u from
+      // the amplitude series' first coefficient, -7/6 u
+      const float u16 = 13.8f * fabsf(r0[kQamp + 1]);
+      const float b3 = 6.f * fmaxf(s_abs.x, s_abs.y) * (u16 * u16 * u16);
+      const bool small = b3 < 0x1p-10f && b3 * (u16 * u16) < 0x1p-36f;
+      if (__all_sync(0xffffffffu, small)) points(std::true_type{});
+      else points(std::false_type{});
       // the chunk factors exp(2 pi i f_c tau_d), once per chunk, then into the
       // lane's float pairs, chunk l before chunk l + 32
 #pragma unroll
