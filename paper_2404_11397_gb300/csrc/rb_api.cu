@@ -755,8 +755,6 @@ struct HostOut {
   bool direct = false;
 };
 
-bool trace_events_set();
-
 // The host-buffer batch's launches as a graph: captured (not run) for the
 // walkers' and outputs' mapped addresses, W and mode on the event's capture
 // stream, with a workspace of its own; replaced when the call changes.
@@ -1213,9 +1211,9 @@ int run_batch(const EventEntry* e, const double* theta, int64_t W, double* logl,
   // set-up and likelihood in one launch where the batch allows it (not with
   // trace events, which bracket the likelihood kernel alone, nor for launches
   // that share the GPU with others)
-  if (mode == RB_MIXED && spread && !trace_events_set()) {
+  if (mode == RB_MIXED && spread && !mala && !trace_events_set()) {
     bool done = false;
-    const cudaError_t ferr = launch_rb_fused(e->dev, e->ec, theta, W, logl, grad, s, sm_count(), mala, &done);
+    const cudaError_t ferr = launch_rb_fused(e->dev, e->ec, theta, W, logl, grad, s, sm_count(), nullptr, &done);
     if (ferr != cudaSuccess) return cuda_fail(ferr, "likelihood kernel");
     if (done) {
       count_launches(1);

@@ -155,5 +155,6 @@ cudaError_t launch_batch_main(const EventEntry* e, void* ws, void* tan, int64_t 
 // Events recorded on the launch stream right before / after the main
 // likelihood kernel of every batch (NULL disables).
 void set_trace_events(void* before, void* after);
+bool trace_events_set();
 
 }  // namespace rb

@@ -99,6 +99,9 @@ struct MalaArgs {
   int* accepted;        // [W] output
   double eps[kNPar];    // step sizes
   int init;             // 1: adopt the proposal (= the state) unconditionally
+  // for the kernel that forms the proposals itself (zp, lu, jac, inside unused)
+  const double* u;      // [W] uniform draws
+  double lo[kNPar], hi[kNPar];  // prior box
 };
 
 // Fiducial values of the mixed path, float pairs (hi, lo) from the

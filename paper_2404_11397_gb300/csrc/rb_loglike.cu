@@ -107,6 +107,7 @@ struct __align__(16) FusedRecords {
 constexpr size_t kFusedWork = sizeof(DdSmem) > (kThreads / 32) * sizeof(WarpWork) ? (sizeof(DdSmem) + 15) / 16 * 16
                                                                                : (kThreads / 32) * sizeof(WarpWork);
 constexpr size_t kFusedBytes = sizeof(FusedRecords) + kFusedWork;
+static_assert(kFusedBytes % 16 == 0, "the MALA chains start on a 16-byte boundary");
 static_assert(sizeof(FusedRecords) % 16 == 0, "the set-up's values start on a 16-byte boundary");
 static_assert(kThreads >= kDdRoleThreads + kTanWarps * 32, "a FUSED block has a warp for every set-up role");
 static_assert(sizeof(WalkerMixed) % 16 == 0, "record copied in 16-byte pieces");
@@ -219,7 +220,7 @@ struct LaunchArgs {
   double* grad;
   MalaArgs mala;     // MALA kernels only
 };
-// the FUSED kernels form the records themselves
+// the FUSED kernels form the records themselves (a MALA step's from its proposals, theta NULL)
 struct FusedArgs : LaunchArgs {
   const double* theta;  // [W][13]
   EventConst ec;
@@ -231,38 +232,99 @@ struct FusedArgs : LaunchArgs {
 // (Sec. II.D, MALA; the sum over j is a warp reduction), accept when
 // log u < log alpha, and the chain state updated in place.  The whole warp
 // calls it (logl and inside are warp-uniform).
-__device__ __forceinline__ void mala_finish(const MalaArgs& m, int64_t w, int lane, double logl, double gth) {
-  const bool inside = m.inside[w] != 0;
+struct MalaWalker {
+  bool inside;
+  double lu, jac9, jac12;  // log u, the Jacobian factors of cos iota and sin dec
+  double zp;               // the lane's component of the proposal
+};
+__device__ __forceinline__ MalaWalker mala_walker(const MalaArgs& m, int64_t w, int lane) {
+  return {m.inside[w] != 0, m.lu[w], m.jac[2 * w], m.jac[2 * w + 1], lane < kNPar ? m.zp[w * kNPar + lane] : 0.0};
+}
+__device__ __forceinline__ void mala_finish(const MalaArgs& m, int64_t w, int lane, double logl, double gth,
+                                            const MalaWalker& mw) {
+  const bool inside = mw.inside;
   const double logpp = inside ? logl : -INFINITY;
   double gz = 0.0, term = 0.0;
   if (lane < kNPar) {
     gz = gth;
-    if (lane == 9) gz = gth * m.jac[2 * w];
-    else if (lane == 12) gz = gth * m.jac[2 * w + 1];
+    if (lane == 9) gz = gth * mw.jac9;
+    else if (lane == 12) gz = gth * mw.jac12;
     if (!inside) gz = 0.0;
+  }
+  if (m.init) {
+    if (lane < kNPar) m.gz[w * kNPar + lane] = gz;
+    if (lane == 0) {
+      m.logp[w] = logpp;
+      if (m.accepted) m.accepted[w] = inside ? 1 : 0;
+    }
+    return;
+  }
+  if (lane < kNPar) {
     const double xi = m.xi[w * kNPar + lane];
     const double t = xi + 0.5 * m.eps[lane] * (m.gz[w * kNPar + lane] + gz);
     term = t * t - xi * xi;
   }
   term = warp_sum_f64(term);
-  if (m.init) {
-    if (lane < kNPar) m.gz[w * kNPar + lane] = gz;
-    if (lane == 0) {
-      m.logp[w] = logpp;
-      m.accepted[w] = inside ? 1 : 0;
-    }
-    return;
-  }
   const double la = (logpp == -INFINITY) ? -INFINITY : logpp - m.logp[w] - 0.5 * term;
-  const bool acc = m.lu[w] < la;
+  const bool acc = mw.lu < la;
   if (acc) {
     if (lane < kNPar) {
-      m.z[w * kNPar + lane] = m.zp[w * kNPar + lane];
+      m.z[w * kNPar + lane] = mw.zp;
       m.gz[w * kNPar + lane] = gz;
     }
     if (lane == 0) m.logp[w] = logpp;
   }
-  if (lane == 0) m.accepted[w] = acc ? 1 : 0;
+  if (lane == 0 && m.accepted) m.accepted[w] = acc ? 1 : 0;
+}
+
+// The proposals of a FUSED block's chains, in its shared memory (as
+// k_mala_propose forms them, expression for expression).
+struct __align__(16) MalaBlock {
+  double theta[kSetupWalkers][kNPar];  // theta(z'), or theta(z) outside the box
+  double zp9[kSetupWalkers], zp12[kSetupWalkers];  // cos iota and sin dec of the proposal (its other components are theta's)
+  double lu[kSetupWalkers], jac9[kSetupWalkers], jac12[kSetupWalkers];
+  int inside[kSetupWalkers];
+};
+// The whole block calls it; n chains from w0.  The block is synchronised at its end.
+__device__ __forceinline__ void mala_propose_block(const MalaArgs& m, int64_t w0, int n, MalaBlock& S) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid < kSetupWalkers) S.inside[tid] = 1;
+  __syncthreads();
+  for (int i = tid; i < n * kNPar; i += kThreads) {
+    const int l = i / kNPar, j = i - l * kNPar;
+    const int64_t g = w0 * kNPar + i;
+    const double c = m.z[g];
+    const double p = m.init ? c : c + 0.5 * m.eps[j] * m.eps[j] * m.gz[g] + m.eps[j] * m.xi[g];
+    S.theta[l][j] = p;
+    if (j == 9) S.zp9[l] = p;
+    if (j == 12) S.zp12[l] = p;
+    if (!(p > m.lo[j] && p < m.hi[j])) S.inside[l] = 0;
+  }
+  __syncthreads();
+  // a chain outside the box is evaluated at its current state (and rejected)
+  for (int i = tid; i < n * kNPar; i += kThreads) {
+    const int l = i / kNPar, j = i - l * kNPar;
+    if (S.inside[l] == 0 && j != 9 && j != 12) S.theta[l][j] = m.z[w0 * kNPar + i];
+  }
+  // the FP64 functions of a chain on four warps side by side, one per SM sub-partition
+  if (warp < 4 && lane < n) {
+    const bool in = S.inside[lane] != 0;
+    const double* zw = m.z + (w0 + lane) * kNPar;
+    const double p9 = S.zp9[lane], p12 = S.zp12[lane];
+    if (warp == 0) {
+      S.theta[lane][9] = acos(in ? p9 : zw[9]);
+    } else if (warp == 1) {
+      S.theta[lane][12] = asin(in ? p12 : zw[12]);
+    } else if (warp == 2) {
+      // d iota / d cos iota = -1 / sin iota, d dec / d sin dec = 1 / cos dec
+      // (1 - z^2 as (1 - z)(1 + z): no cancellation next to the box edges)
+      S.jac9[lane] = in ? -1.0 / sqrt((1.0 - p9) * (1.0 + p9)) : 0.0;
+      S.jac12[lane] = in ? 1.0 / sqrt((1.0 - p12) * (1.0 + p12)) : 0.0;
+    } else {
+      S.lu[lane] = m.init ? 0.0 : log(m.u[w0 + lane]);
+    }
+  }
+  __syncthreads();
 }
 
 // Chain rule for one walker: lane j < 13 returns d log L / d theta_j from the
@@ -525,14 +587,26 @@ __global__ void __launch_bounds__(kThreads)
   const int64_t nwarps = blockDim.x >> 5;
   const unsigned char* rec_g = static_cast<const unsigned char*>(a.ws);
   const unsigned char* tan_g = static_cast<const unsigned char*>(a.tan);
+  const MalaBlock* chains = nullptr;  // FUSED MALA: the block's chains
   if constexpr (FUSED) {
     DdSmem& S = *reinterpret_cast<DdSmem*>(fused + 1);
     const int warp = threadIdx.x >> 5;
+    // theta of the block's walkers, the first and the end of its rows
+    const double* theta = a.theta;
+    int64_t t_begin = w_begin, t_end = w_end;
+    if constexpr (MALA) {
+      MalaBlock* mb = reinterpret_cast<MalaBlock*>(reinterpret_cast<unsigned char*>(fused) + kFusedBytes);
+      mala_propose_block(a.mala, w_begin, (int)(w_end - w_begin), *mb);
+      chains = mb;
+      theta = &mb->theta[0][0];
+      t_begin = 0;
+      t_end = w_end - w_begin;
+    }
     if (warp < kDdRoleWarps) {
-      setup_absolute_dd(a.theta, w_begin, w_end, a.ec, S);
+      setup_absolute_dd(theta, t_begin, t_end, a.ec, S);
       setup_record_dd(ev.ref->dd, a.ec, S, &fused->rec[lane], w_begin + lane < w_end);
     } else if (GRAD && warp < kDdRoleWarps + 3 + D) {
-      tangent_warp<float>(a.theta, w_end, w_begin, a.ec, fused->tan, warp - kDdRoleWarps);
+      tangent_warp<float>(theta, t_end, t_begin, a.ec, fused->tan, warp - kDdRoleWarps);
     }
   }
   // the first walker's record and tangents travel with the tables
@@ -553,6 +627,17 @@ __global__ void __launch_bounds__(kThreads)
     work->lane_gmax[lane] = gk >= 0 ? ev.gmax[gk] : 0.f;
   }
 
+  // the MALA step of walker w, its log L and gradient (lane j: component j) at hand
+  auto mala_step = [&](int64_t w, double logl, double gth) {
+    if constexpr (FUSED) {
+      const int l = (int)(w - w_begin);
+      const MalaWalker mw{chains->inside[l] != 0, chains->lu[l], chains->jac9[l], chains->jac12[l],
+                          lane == 9 ? chains->zp9[l] : lane == 12 ? chains->zp12[l] : lane < kNPar ? chains->theta[l][lane] : 0.0};
+      mala_finish(a.mala, w, lane, logl, gth, mw);
+    } else {
+      mala_finish(a.mala, w, lane, logl, gth, mala_walker(a.mala, w, lane));
+    }
+  };
   int buf = 0;
   for (int64_t w = warp0; w < w_end; w += nwarps, buf ^= 1) {
     if (!FUSED) cp_async_wait_all();  // this walker's record and tangents
@@ -641,8 +726,8 @@ __global__ void __launch_bounds__(kThreads)
                                        GRAD ? tan_g + sizeof(WalkerTan<float>) * RB_IDX(wn, a.W, 107) : nullptr, lane);
     }
     if (!valid) {
-      if (MALA) {
-        mala_finish(a.mala, w, lane, -INFINITY, 0.0);
+      if constexpr (MALA) {
+        mala_step(w, -INFINITY, 0.0);
       } else {
         if (lane == 0) a.logl[w] = -INFINITY;
         if (GRAD && lane < kNPar) a.grad[w * kNPar + lane] = 0.0;
@@ -653,8 +738,8 @@ __global__ void __launch_bounds__(kThreads)
       // a phase term beyond 2^18 turns (~1.6e6 rad): past the range of the
       // float-pair phase sums' whole-turn reductions; not evaluated (NaN,
       // rejected by the MALA step)
-      if (MALA) {
-        mala_finish(a.mala, w, lane, -INFINITY, 0.0);
+      if constexpr (MALA) {
+        mala_step(w, -INFINITY, 0.0);
       } else {
         if (lane == 0) a.logl[w] = __longlong_as_double(0x7ff8000000000000ll);
         if (GRAD && lane < kNPar) a.grad[w * kNPar + lane] = __longlong_as_double(0x7ff8000000000000ll);
@@ -859,7 +944,7 @@ __global__ void __launch_bounds__(kThreads)
         const WalkerTan<float>& tn = FUSED ? fused->tan[wl] : *reinterpret_cast<const WalkerTan<float>*>(slot->tan[buf]);
         g = f2d_int(chain_rule_lanes<D>(lane, ac, at, ar, tn));
       }
-      if (MALA) mala_finish(a.mala, w, lane, logl, g);
+      if constexpr (MALA) mala_step(w, logl, g);
       else if (lane < kNPar) a.grad[RB_IDX(w * kNPar + lane, a.W * kNPar, 106)] = g;
     }
   }
@@ -903,7 +988,7 @@ __global__ void __launch_bounds__(256) k_rb_f64(LaunchArgs a) {
     const WalkerF64* s = reinterpret_cast<const WalkerF64*>(a.ws) + w;
     if (!s->valid) {
       if (MALA) {
-        mala_finish(a.mala, w, lane, -INFINITY, 0.0);
+        mala_finish(a.mala, w, lane, -INFINITY, 0.0, mala_walker(a.mala, w, lane));
       } else {
         if (lane == 0) a.logl[w] = -INFINITY;
         if (GRAD && lane < kNPar) a.grad[w * kNPar + lane] = 0.0;
@@ -987,7 +1072,7 @@ __global__ void __launch_bounds__(256) k_rb_f64(LaunchArgs a) {
       }
       double g = 0.0;
       if (lane < kNPar) g = chain_rule_lanes<ND>(lane, ac, at, G, reinterpret_cast<const WalkerTan<double>*>(a.tan)[w]);
-      if (MALA) mala_finish(a.mala, w, lane, logl, g);
+      if (MALA) mala_finish(a.mala, w, lane, logl, g, mala_walker(a.mala, w, lane));
       else if (lane < kNPar) a.grad[RB_IDX(w * kNPar + lane, a.W * kNPar, 106)] = g;
     }
     __syncwarp();  // red is read before the next walker's sums
@@ -1117,11 +1202,12 @@ cudaError_t launch_rb_mixed(const EventDev& ev, const void* ws, const void* tan,
 
 // Set-up and likelihood in one launch, where it applies (*done): every block
 // gets at most kSetupWalkers walkers, and the tables leave room for their
-// records beside them.
+// records beside them.  With mala the kernel forms the proposals too (theta is not
+// read).
 template <int ND, bool GRAD, bool MALA>
 static cudaError_t launch_fused_nd(const FusedArgs& a, cudaStream_t s, int n_sm, bool* done) {
   auto* fn = k_rb_mixed<ND, GRAD, false, MALA, true>;
-  const size_t smem = a.ev.slot32_floats * sizeof(float) + kFusedBytes;
+  const size_t smem = a.ev.slot32_floats * sizeof(float) + kFusedBytes + (MALA ? sizeof(MalaBlock) : 0);
   *done = false;
   if (smem > smem_optin_max()) return cudaSuccess;
   int per_sm = 0;

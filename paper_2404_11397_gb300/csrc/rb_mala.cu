@@ -10,6 +10,7 @@
 //   log L(theta(z')) and d log L / d theta                         (set-up + batch kernel)
 //   log alpha = log pi(z') - log pi(z) - 1/2 sum_j [(xi_j + eps_j (g_j + g'_j)/2)^2 - xi_j^2]
 //   accept if log u < log alpha, state updated in place            (batch kernel epilogue)
+// (mixed batches of up to 32 chains per SM: all of it in the batch kernel).
 // The draws are inputs, so the step is reproducible.
 #include <cmath>
 #include <cstdint>
@@ -19,6 +20,9 @@
 #include "rb_internal.cuh"
 
 namespace rb {
+
+cudaError_t launch_rb_fused(const EventDev& ev, const EventConst& ec, const double* theta, int64_t W, double* logl,
+                            double* grad, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done);
 
 struct MalaBox {
   double eps[kNPar], lo[kNPar], hi[kNPar];
@@ -85,7 +89,7 @@ __global__ void __launch_bounds__(kProposeThreads) k_mala_propose(const double* 
 }
 
 // Per-chain workspace of a MALA call (bytes per chain, without the batch's).
-static size_t mala_ws_bytes() { return sizeof(double) * (2 * kNPar + 1 + 2) + 2 * sizeof(int); }
+static size_t mala_ws_bytes() { return sizeof(double) * (2 * kNPar + 1 + 2) + sizeof(int); }
 
 static int mala_run(rb_event_t ev, double* z, double* logp, double* gz, int64_t W, const double* eps_host,
                     const double* lo_host, const double* hi_host, const double* xi, const double* u, int* accepted,
@@ -108,16 +112,41 @@ static int mala_run(rb_event_t ev, double* z, double* logp, double* gz, int64_t 
     return set_error(RB_EINVAL, "%s: cos iota and sin dec bounds must lie in [-1, 1]", who);
   const EventEntry* e = event_entry(ev);
   cudaStream_t s = (cudaStream_t)stream;
+  MalaArgs m{};
+  m.z = z;
+  m.logp = logp;
+  m.gz = gz;
+  m.xi = xi;
+  m.u = u;
+  m.accepted = accepted;
+  m.init = init ? 1 : 0;
+  for (int j = 0; j < kNPar; ++j) {
+    m.eps[j] = box.eps[j];
+    m.lo[j] = box.lo[j];
+    m.hi[j] = box.hi[j];
+  }
+  cudaError_t err;
+  // Mixed batches that take the set-up and likelihood in one launch (rb_loglike.cu)
+  // take the proposals there too: one kernel, no workspace.  1000 chains, 3 detectors,
+  // 200 bins: a step with its copies 53 -> 47 us.  Not with trace events, which bracket the likelihood kernel.
+  if (mode == RB_MIXED && !trace_events_set()) {
+    bool done = false;
+    if ((err = launch_rb_fused(e->dev, e->ec, nullptr, W, nullptr, nullptr, s, sm_count(), &m, &done)) != cudaSuccess)
+      return cuda_fail(err, "MALA step kernel");
+    if (done) {
+      count_launches(1);
+      return RB_OK;
+    }
+  }
   char* buf = nullptr;
   const size_t per = mala_ws_bytes();
-  cudaError_t err = ws_alloc(reinterpret_cast<void**>(&buf), per * W, s);
+  err = ws_alloc(reinterpret_cast<void**>(&buf), per * W, s);
   if (err != cudaSuccess) return cuda_fail(err, "MALA workspace allocation");
   double* zp = reinterpret_cast<double*>(buf);
   double* theta = zp + kNPar * W;
   double* lu = theta + kNPar * W;
   double* jac = lu + W;
   int* inside = reinterpret_cast<int*>(jac + 2 * W);
-  int* acc_scratch = inside + W;
   k_mala_propose<<<(unsigned)((W + 31) / 32), kProposeThreads, 0, s>>>(z, gz, xi, u, box, W, init ? 1 : 0, zp, theta,
                                                                        lu, jac, inside);
   err = cudaGetLastError();
@@ -126,18 +155,10 @@ static int mala_run(rb_event_t ev, double* z, double* logp, double* gz, int64_t 
     rc = cuda_fail(err, "MALA proposal kernel");
   } else {
     count_launches(1);
-    MalaArgs m{};
-    m.z = z;
     m.zp = zp;
-    m.logp = logp;
-    m.gz = gz;
-    m.xi = init ? zp : xi;  // unused terms when init (eps = 0)
     m.lu = lu;
     m.jac = jac;
     m.inside = inside;
-    m.accepted = accepted ? accepted : acc_scratch;
-    for (int j = 0; j < kNPar; ++j) m.eps[j] = box.eps[j];
-    m.init = init ? 1 : 0;
     rc = run_batch(e, theta, W, nullptr, nullptr, mode, s, nullptr, &m);
   }
   cudaFreeAsync(buf, s);
