@@ -624,4 +624,48 @@ __device__ __forceinline__ float warp_sum_f32(float v) {
   return v;
 }
 
+// One level of a transposed warp sum: lanes whose bit o is clear keep values
+// [0, M) of `in` and send [M, N), lanes whose bit is set keep [M, N) (zero
+// beyond N) and send [0, M); each adds what its partner sent.
+template <class T, int N, int M>
+__device__ __forceinline__ void tsum_level(const T (&in)[N], T (&out)[M], int lane, int o) {
+  const bool up = (lane & o) != 0;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const T lo = in[i], hi = (M + i < N) ? in[M + i] : T(0);
+    const T keep = up ? hi : lo, send = up ? lo : hi;
+    out[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+  }
+}
+
+// Warp sums of NV <= 32 values per lane, each a fixed-order five-level tree:
+// after five halving levels every lane holds the total of one value, which
+// it writes to out[index] (shared memory); 31 shuffles for 32 values against
+// 5 NV for NV separate butterflies.
+template <class T, int NV>
+__device__ __forceinline__ void warp_transposed_sums(const T (&v)[NV], int lane, T* out) {
+  static_assert(NV >= 1 && NV <= 32, "up to 32 values");
+  constexpr int m1 = (NV + 1) / 2, m2 = (m1 + 1) / 2, m3 = (m2 + 1) / 2, m4 = (m3 + 1) / 2, m5 = (m4 + 1) / 2;
+  static_assert(m5 == 1, "five levels reduce to one value");
+  T a[m1], b[m2], c[m3], d[m4], e[m5];
+  tsum_level(v, a, lane, 16);
+  tsum_level(a, b, lane, 8);
+  tsum_level(b, c, lane, 4);
+  tsum_level(c, d, lane, 2);
+  tsum_level(d, e, lane, 1);
+  // the value's index: the positions this lane kept, from the last level back
+  // (a lane whose kept half was padding at some level holds no value)
+  int idx = (lane & 1) ? m5 : 0;
+  bool ok = idx < m4;
+  idx += (lane & 2) ? m4 : 0;
+  ok = ok && idx < m3;
+  idx += (lane & 4) ? m3 : 0;
+  ok = ok && idx < m2;
+  idx += (lane & 8) ? m2 : 0;
+  ok = ok && idx < m1;
+  idx += (lane & 16) ? m1 : 0;
+  ok = ok && idx < NV;
+  if (ok) out[idx] = e[0];
+}
+
 }  // namespace rb

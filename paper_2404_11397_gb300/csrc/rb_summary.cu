@@ -395,20 +395,19 @@ cudaError_t launch_summary(const DataPtrs& in, int64_t kmin, int64_t N, double T
 // k_summary for the current theta_ref): the build then streams the strain,
 // the PSD and h0, 40 B per (point, detector), with no waveform arithmetic.
 // One block of kStoredThreads per part of a bin (the fast build's parts), all
-// detectors; the per-point terms are k_summary's, with f = (kmin + k) (1/T)
-// and 1/S from rcp_newton in place of the two FP64 divisions (the FP64 pipe
-// is the bound); block sums in a fixed order, the parts of a bin added in index order by the
+// detectors; the per-point terms are k_summary's, with the moments about a bin's middle
+// in whole half grid steps and 1/S from rcp_newton in place of the two FP64 divisions
+// (the FP64 pipe is the bound: 16 FP64 operations per point and detector); block sums in a fixed order, the parts of a bin added in index order by the
 // last of them to finish, which runs the FP64 epilogue (base log L by the
 // fixed-point sum).  Several warps per part keep enough FP64 work in flight
 // to cover the FP64 pipe's latency.
 constexpr int kStoredThreads = 128;
 
-// 1/S for a positive normal double by Newton-Raphson iteration for the
-// reciprocal, r <- r + r (1 - S r), which doubles the correct bits per step:
-// the seed is the FP32 reciprocal of S scaled to [1, 2) (built and moved back
-// to FP64 with integer operations, ~23 correct bits), two steps give FP64
-// accuracy (within 1 ulp).  Four FP64 FMAs in all; inputs outside
-// [2^-1022, 2^1021) take the division.
+// 1/S for a positive normal double by iteration on the reciprocal's residual: the
+// seed is the FP32 reciprocal of S scaled to [1, 2) (built and moved back to FP64 with
+// integer operations, e = 1 - S r ~ 2^-22), one third-order step r + r (e + e^2) gives
+// FP64 accuracy (the next term is below 2^-66; within 1 ulp).  Three FP64 FMAs in all
+// (two second-order steps: four); inputs outside [2^-1022, 2^1021) take the division.
 __device__ __forceinline__ double rcp_newton(double S) {
   const unsigned hi = (unsigned)__double2hiint(S), lo = (unsigned)__double2loint(S);
   const int ef = (int)((hi >> 20) & 0x7FFu);
@@ -420,43 +419,58 @@ __device__ __forceinline__ double rcp_newton(double S) {
   const int er = (int)((rb >> 23) & 0xFFu) - 127;
   const unsigned m = rb & 0x7FFFFFu;
   double r = __hiloint2double((int)(((unsigned)(er + 1023 - (ef - 1023)) << 20) | (m >> 3)), (int)((m & 7u) << 29));
-  r = fma(r, fma(-S, r, 1.0), r);
-  r = fma(r, fma(-S, r, 1.0), r);
-  return r;
+  const double e = fma(-S, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Integer -> double, exactly, by one FP64 addition (the conversion instruction
+// issues on the FP64 pipe too, and the 64-bit one more than once): 1.5 2^52 + i
+// put together with integer operations.
+__device__ __forceinline__ double small_int_double(int i) {
+  return __hiloint2double(0x43380000 + (i >> 31), i) - 6755399441055744.0;
+}
+
+// A point's terms, weight w = 1/S, offset n: x = d conj(h) and |h|^2 (hh) into the
+// sums and the moments (nine operations for x, three for |h|^2).
+__device__ __forceinline__ void add_terms(double* acc, double w, double n, double2 dv, double hr, double hi, double hh) {
+  const double xr = fma(dv.x, hr, dv.y * hi), xi = fma(dv.y, hr, -(dv.x * hi)), wn = w * n;
+  acc[0] = fma(w, xr, acc[0]);
+  acc[1] = fma(w, xi, acc[1]);
+  acc[2] = fma(wn, xr, acc[2]);
+  acc[3] = fma(wn, xi, acc[3]);
+  acc[4] = fma(w, hh, acc[4]);
+  acc[5] = fma(wn, hh, acc[5]);
 }
 
 // Blocks take the parts from the last one down: the bins widen with frequency,
 // so the full parts start first and the short ones fill the gaps at the end
-// (519,169 points, 3 detectors, 1000 bins: FP64 build from the stored waveform 118.6 ->
-// 110.7 us, mixed rebuild 24.3 -> 23.2 us, the chunk-expanded FP64 build's kernel 174 ->
-// 161 us; results do not depend on the order).
+// (519,169 points, 3 detectors, 1000 bins, when this came: FP64 build from the stored
+// waveform 118.6 -> 110.7 us, mixed rebuild 24.3 -> 23.2 us, the chunk-expanded FP64 build's
+// kernel 174 -> 161 us; results do not depend on the order).
 __device__ __forceinline__ int part_of_block(int n_parts) { return n_parts - 1 - (int)blockIdx.x; }
 
 // The end of the FP64 builds that take one block per part of a bin: the block's
 // sums of the per-thread sums acc (six per detector, terms over S without the
-// factor 4 df), the parts of a bin added in index order by the last of them to
+// factor 4 df, moments in units of half a grid step), the parts of a bin added in index order by the last of them to
 // finish, which runs the FP64 epilogue (base log L by the fixed-point sum).
 template <int ND>
-__device__ __forceinline__ void stored_part_sums(const double (&acc)[ND][6], double inv_T, int pid, const PartDesc& pd, int b, int B, const SummaryOut& so,
-                                                 double (*red)[kStoredThreads], double* qsum, double* sblock) {
+__device__ __forceinline__ void stored_part_sums(const double (&acc)[6 * ND], double inv_T, int pid, const PartDesc& pd, int b, int B, const SummaryOut& so,
+                                                 double (*wsum)[6 * kMaxDet], double* sblock) {
   __shared__ bool s_last;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  // block sums in a fixed order: warp w takes quantities w, w + 4, ...; each
-  // lane adds the 4 threads l, l + 32, l + 64, l + 96, then a shuffle tree
-#pragma unroll
-  for (int d = 0; d < ND; ++d)
-#pragma unroll
-    for (int j = 0; j < 6; ++j) red[6 * d + j][tid] = acc[d][j];
+  // block sums in a fixed order: transposed warp sums (20 additions per warp for 18
+  // values; rows of 128 in shared memory, a warp per value, took 36), then the warps
+  warp_transposed_sums(acc, lane, wsum[wid]);
   __syncthreads();
-  for (int q = wid; q < 6 * ND; q += kStoredThreads / 32) {
-    double v = red[q][lane];
+  double mine = 0.0;
+  if (tid < 6 * ND) {
+    double v = wsum[0][tid];
 #pragma unroll
-    for (int i = 1; i < kStoredThreads / 32; ++i) v += red[q][lane + 32 * i];
-    v = warp_sum_f64(v);
-    if (lane == 0) qsum[q] = 4.0 * inv_T * v;
+    for (int i = 1; i < kStoredThreads / 32; ++i) v += wsum[i][tid];
+    const int j = tid % 6;
+    mine = 4.0 * inv_T * v;
+    if (j == 2 || j == 3 || j == 5) mine *= 0.5 * inv_T;
   }
-  __syncthreads();
-  double mine = tid < 6 * ND ? qsum[tid] : 0.0;
   if (pd.n_parts > 1) {
     double* ps = reinterpret_cast<double*>(so.part_sums);  // [n_parts][kPartSlots] doubles
     if (tid < 6 * ND) ps[(size_t)pid * kPartSlots + tid] = mine;
@@ -486,39 +500,28 @@ template <int ND>
 __global__ void __launch_bounds__(kStoredThreads) k_summary_stored(DataPtrs in, const double* __restrict__ h0,
                                                                    int64_t kmin, int64_t N, double T, int B,
                                                                    const int64_t* __restrict__ edges, SummaryOut so) {
-  __shared__ double red[6 * ND][kStoredThreads];  // per-thread sums, one row per quantity
-  __shared__ double qsum[6 * kMaxDet];
+  __shared__ double wsum[kStoredThreads / 32][6 * kMaxDet];
   __shared__ double sblock[6 * kMaxDet];
   const int pid = part_of_block(so.n_parts), tid = threadIdx.x;
   const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
   const int b = pd.bin;
-  const double fm = 0.5 * (grid_f(kmin, edges[b], T) + grid_f(kmin, edges[b + 1], T));
   const double inv_T = 1.0 / T;
-  double acc[ND][6];
+  double acc[6 * ND];
 #pragma unroll
-  for (int d = 0; d < ND; ++d)
-#pragma unroll
-    for (int j = 0; j < 6; ++j) acc[d][j] = 0.0;
-  // sums of the terms over S; the factor 4 df = 4 / T is applied to the sums
-  for (int64_t k = pd.start + tid; k < pd.end; k += kStoredThreads) {
-    const double f = (double)(kmin + k) * inv_T;
-    const double df = f - fm;
+  for (int i = 0; i < 6 * ND; ++i) acc[i] = 0.0;
+  // sums of the terms over S; the factor 4 df = 4 / T is applied to the sums.
+  // n = 2 (f - f_m) T, an integer: the moments' unit is applied to the sums too
+  double n = (double)(2 * ((int64_t)pd.start + tid) - edges[b] - edges[b + 1]);
+  for (int64_t k = pd.start + tid; k < pd.end; k += kStoredThreads, n += 2.0 * kStoredThreads) {
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
       const double2 dv = __ldcs(reinterpret_cast<const double2*>(in.data[d]) + RB_IDX(k, N, 222));
       const double2 hv = __ldcs(reinterpret_cast<const double2*>(h0) + (size_t)d * N + RB_IDX(k, N, 222));
       const double w = rcp_newton(__ldcs(in.psd[d] + k));
-      const double hr = hv.x, hi = hv.y, dr = dv.x, di = dv.y;
-      const double xr = dr * hr + di * hi, xi = di * hr - dr * hi, hh = hr * hr + hi * hi;
-      acc[d][0] += w * xr;
-      acc[d][1] += w * xi;
-      acc[d][2] += w * xr * df;
-      acc[d][3] += w * xi * df;
-      acc[d][4] += w * hh;
-      acc[d][5] += w * hh * df;
+      add_terms(&acc[6 * d], w, n, dv, hv.x, hv.y, hv.x * hv.x + hv.y * hv.y);
     }
   }
-  stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, red, qsum, sblock);
+  stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, wsum, sblock);
 }
 
 cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t kmin, int64_t N, double T, int D, int B,
@@ -540,10 +543,16 @@ cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t 
 //   h_d(f) = K_d f^-7/6 exp(-2 pi i [x(f) + f tau_d]),  f = f_c (1 + j u),
 //   exp(-2 pi i f tau_d) = exp(-2 pi i f_c tau_d) exp(-2 pi i j df tau_d),
 // the first factor (times K_d f_c^-7/6) from the chunk's record, the second from
-// a 32-entry table.  ~115 FP64 operations per point: 519,169 points, 3 detectors,
-// 1000 bins: k_summary 605 us, this kernel 161 us (FP64 pipe 84 % busy) and the
-// records 19 us; the whole rebuild call 615 -> 194 us.  Errors against 80-bit
-// sums (2-norm): A0 8.2e-13 (k_summary 8.3e-13), A1 5.5e-13 (5.5e-13), B0, B1 below 2.5e-15.  A record keeps the orders
+// a 32-entry table; detector 0's delay goes into the phase (linear in j) instead, and
+// the others' are taken from it.  ~100 FP64 operations per point with three detectors
+// (an FP64 warp instruction holds its SM sub-partition's FP64 unit for ~65 clocks, so
+// operations are what counts): 519,169 points, 3 detectors, 1000 bins: k_summary 605 us,
+// this kernel 134 us (FP64 pipe 84 % busy) and the records 18 us; the whole rebuild call
+// 640 -> 181 us.  Before detector 0's delay went into the phase, the moments into whole
+// steps and the block sums into transposed warp sums it was ~115 operations, 161 us.
+// Errors against FP64 torch sums (2-norm) on four events: A0 1.5e-13 to 2.2e-12 (k_summary
+// 1.4e-13 to 2.2e-12), A1 1.4e-13 to 8.6e-13 (1.5e-13 to 8.6e-13).
+// A record keeps the orders
 // that reach 2^-48 turns at the chunk's ends (up to 9 of them); X_0, up to
 // thousands of turns, is reduced to [-1/2, 1/2] before it is rounded, so the phase's
 // error stays that of the basis functions, as in k_summary.
@@ -553,8 +562,8 @@ cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t 
 constexpr int kOrd64 = 9;
 constexpr int kAmp64 = 9;  // binomial orders of (1 + j u)^-7/6: (1/64)^10 < 2^-53
 struct __align__(16) ChunkRec64 {
-  double X[kOrd64 + 1];  // phase in turns, X[0] reduced, zero beyond the orders kept
-  double G[kMaxDet][2];  // K_d f_c^-7/6 exp(-2 pi i f_c tau_d)
+  double X[kOrd64 + 1];  // phase in turns with f tau_0, X[0] reduced, zero beyond the orders kept
+  double G[kMaxDet][2];  // K_d f_c^-7/6 exp(-2 pi i f_c (tau_d - tau_0))
 };
 
 struct TaylorTables64 {
@@ -572,15 +581,17 @@ __device__ __forceinline__ void two_sum64(double a, double b, double& s, double&
 }
 
 // One thread per chunk; the last block forms the offset table
-// etab[d][j] = exp(-2 pi i (j - 16) df tau_d).
-__global__ void __launch_bounds__(64) k_chunk64(const RefValues* __restrict__ ref, int64_t kmin, double T, int n_chunks, int D,
+// etab[d][j] = exp(-2 pi i (j - 16) df (tau_d - tau_0)).  Blocks of four warps, one
+// per SM sub-partition: in blocks of two, half of an SM's FP64 units had no work.
+constexpr int kChunk64Threads = 128;
+__global__ void __launch_bounds__(kChunk64Threads) k_chunk64(const RefValues* __restrict__ ref, int64_t kmin, double T, int n_chunks, int D,
                                                 TaylorTables64 tt, ChunkRec64* __restrict__ recs,
                                                 double2* __restrict__ etab) {
   const Values& v = ref->v;
   if (blockIdx.x == gridDim.x - 1) {
     for (int i = threadIdx.x; i < D * kChunk; i += blockDim.x) {
       double s, c;
-      sincospi(2.0 * (((double)(i % kChunk - kChunk / 2) / T) * v.tau[i / kChunk]), &s, &c);
+      sincospi(2.0 * (((double)(i % kChunk - kChunk / 2) / T) * (v.tau[i / kChunk] - v.tau[0])), &s, &c);
       etab[i] = make_double2(c, -s);
     }
     return;
@@ -610,7 +621,8 @@ __global__ void __launch_bounds__(64) k_chunk64(const RefValues* __restrict__ re
   const double inv2pi = 1.0 / kTwoPi;
   constexpr double inv2pi_lo = -9.839338337591243e-18;  // 1/2pi - fl(1/2pi)
   const double xh = sh * inv2pi, xl = fma(sh, inv2pi, -xh) + (sh * inv2pi_lo + sl * inv2pi);
-  r.X[0] = (xh - rint(xh)) + xl;
+  const double y0 = fc * v.tau[0];
+  r.X[0] = (xh - rint(xh)) + ((y0 - rint(y0)) + (xl + fma(fc, v.tau[0], -y0)));
   // orders kept: |X_n j^n| <= 6 sum_k |c_k P_k| (1 + |ln f_c|) / 2 pi (16 u)^n
   // (every |alpha_kn|, |beta_n| <= 5.2 up to order 10), below 2^-48 turns beyond n_ord
   double bound = 0.0;
@@ -628,7 +640,7 @@ __global__ void __launch_bounds__(64) k_chunk64(const RefValues* __restrict__ re
     double x = 0.0;
 #pragma unroll
     for (int k = 0; k < kNBasis; ++k) x = fma(cp[k], k == 6 ? fma(tt.beta6[n], lf, tt.alpha[k][n]) : tt.alpha[k][n], x);
-    r.X[n] = x * un;
+    r.X[n] = n == 1 ? fma(x, un, v.tau[0] / T) : x * un;
     un *= u;
   }
   const double kamp = 8.035028173395984e-06 / kMpcS;
@@ -638,20 +650,15 @@ __global__ void __launch_bounds__(64) k_chunk64(const RefValues* __restrict__ re
       r.G[d][0] = r.G[d][1] = 0.0;
       continue;
     }
-    double s, co;
-    const double y = fc * v.tau[d];
-    sincospi(2.0 * (y - rint(y)), &s, &co);
+    double s = 0.0, co = 1.0;
+    if (d > 0) {
+      const double y = fc * (v.tau[d] - v.tau[0]);
+      sincospi(2.0 * (y - rint(y)), &s, &co);
+    }
     const double a = kamp * v.amp * (sqrt(icf) / fc), Kr = a * v.P64[d][0], Ki = a * v.P64[d][1];
     r.G[d][0] = Kr * co + Ki * s;  // K exp(-2 pi i y)
     r.G[d][1] = Ki * co - Kr * s;
   }
-}
-
-// Integer -> double, exactly, by one FP64 addition (the conversion instruction
-// issues on the FP64 pipe too, and the 64-bit one more than once): 1.5 2^52 + i
-// put together with integer operations.
-__device__ __forceinline__ double small_int_double(int i) {
-  return __hiloint2double(0x43380000 + (i >> 31), i) - 6755399441055744.0;
 }
 
 // exp(-2 pi i x).
@@ -677,13 +684,13 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in,
                                                                     SummaryOut so) {
   constexpr int kRecDoubles = sizeof(ChunkRec64) / sizeof(double);
   constexpr int kRecs = kPartPoints / kChunk + 1;  // chunk records a part can touch
-  __shared__ double red[6 * ND][kStoredThreads];
-  __shared__ double qsum[6 * kMaxDet];
+  __shared__ double wsum[kStoredThreads / 32][6 * kMaxDet];
   __shared__ double sblock[6 * kMaxDet];
   __shared__ ChunkRec64 srec[kRecs];
   __shared__ double su[kRecs], sg2[ND][kRecs];  // u and |G_d|^2 of the part's chunks
   __shared__ int sord[kRecs], samp[kRecs];      // orders of the phase and of the amplitude series
   __shared__ double2 se[ND * kChunk];
+  __shared__ double s_amp[kAmp64 + 1];  // (indexed at run time: a parameter array would be copied to local memory)
   const int pid = part_of_block(so.n_parts), tid = threadIdx.x;
   const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
   const int b = pd.bin, c0 = pd.start / kChunk, nrec = (pd.end - 1) / kChunk - c0 + 1;
@@ -692,14 +699,15 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in,
     double* dst = reinterpret_cast<double*>(srec);
     for (int i = tid; i < nrec * kRecDoubles; i += kStoredThreads) dst[RB_IDX(i, kRecs * kRecDoubles, 204)] = __ldg(src + i);
     for (int i = tid; i < ND * kChunk; i += kStoredThreads) se[i] = etab[i];
+    if (tid == 0)
+#pragma unroll
+      for (int i = 0; i <= kAmp64; ++i) s_amp[i] = as.c[i];
   }
   const int64_t e0 = edges[b], e1 = edges[b + 1];
-  const double inv_T = 1.0 / T, half_df = 0.5 * inv_T;
-  double acc[ND][6];
+  const double inv_T = 1.0 / T;
+  double acc[6 * ND];
 #pragma unroll
-  for (int d = 0; d < ND; ++d)
-#pragma unroll
-    for (int j = 0; j < 6; ++j) acc[d][j] = 0.0;
+  for (int i = 0; i < 6 * ND; ++i) acc[i] = 0.0;
   __syncthreads();
   if (tid < nrec) {
     const int nc = (int)kmin + (c0 + tid) * kChunk + kChunk / 2;
@@ -720,7 +728,15 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in,
     }
   }
   __syncthreads();
-  for (int64_t k = pd.start + tid; k < pd.end; k += kStoredThreads) {
+  // a thread keeps its place in the chunks
+  static_assert(kStoredThreads % kChunk == 0, "a thread's points have the same offset");
+  const int jj = (pd.start + tid) % kChunk;
+  const double j = small_int_double(jj - kChunk / 2);
+  double2 ed[ND];
+#pragma unroll
+  for (int d = 1; d < ND; ++d) ed[d] = se[d * kChunk + jj];
+  double n = small_int_double((int)(2 * ((int64_t)pd.start + tid) - e0 - e1));  // 2 (f - f_m) T
+  for (int64_t k = pd.start + tid; k < pd.end; k += kStoredThreads, n += 2.0 * kStoredThreads) {
     double2 dv[ND];
     double S[ND];
 #pragma unroll
@@ -728,34 +744,28 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in,
       dv[d] = __ldcs(reinterpret_cast<const double2*>(in.data[d]) + RB_IDX(k, N, 222));
       S[d] = __ldcs(in.psd[d] + k);
     }
-    const int ci = RB_IDX((int)(k / kChunk) - c0, kRecs, 203), jj = (int)(k % kChunk);
+    const int ci = RB_IDX((int)(k / kChunk) - c0, kRecs, 203);
     const ChunkRec64& r = srec[ci];
-    const double j = small_int_double(jj - kChunk / 2);
     double x = 0.0;
-    for (int n = sord[ci]; n >= 0; --n) x = fma(x, j, r.X[n]);
+    for (int i = sord[ci]; i >= 0; --i) x = fma(x, j, r.X[i]);
     const double2 z = cis_neg_turns64(x);
     const double ju = j * su[ci];
-    double a = as.c[samp[ci]];
-    for (int n = samp[ci] - 1; n >= 0; --n) a = fma(a, ju, as.c[n]);  // (1 + j u)^-7/6
+    double a = s_amp[samp[ci]];
+    for (int i = samp[ci] - 1; i >= 0; --i) a = fma(a, ju, s_amp[i]);  // (1 + j u)^-7/6
     const double zr = a * z.x, zi = a * z.y, a2 = a * a;
-    const double df = small_int_double((int)(2 * k - e0 - e1)) * half_df;  // f - f_m
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
-      const double2 e = se[d * kChunk + jj];
-      const double Fr = r.G[d][0] * e.x - r.G[d][1] * e.y, Fi = r.G[d][0] * e.y + r.G[d][1] * e.x;
+      double Fr = r.G[d][0], Fi = r.G[d][1];
+      if (d > 0) {
+        Fr = r.G[d][0] * ed[d].x - r.G[d][1] * ed[d].y;
+        Fi = r.G[d][0] * ed[d].y + r.G[d][1] * ed[d].x;
+      }
       const double hr = zr * Fr - zi * Fi, hi = zr * Fi + zi * Fr;
       __stcs(reinterpret_cast<double2*>(h0_out) + (size_t)d * N + k, make_double2(hr, hi));
-      const double w = rcp_newton(S[d]);
-      const double xr = w * (dv[d].x * hr + dv[d].y * hi), xi = w * (dv[d].y * hr - dv[d].x * hi), hh = w * (a2 * sg2[d][ci]);
-      acc[d][0] += xr;
-      acc[d][1] += xi;
-      acc[d][2] += xr * df;
-      acc[d][3] += xi * df;
-      acc[d][4] += hh;
-      acc[d][5] += hh * df;
+      add_terms(&acc[6 * d], rcp_newton(S[d]), n, dv[d], hr, hi, a2 * sg2[d][ci]);
     }
   }
-  stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, red, qsum, sblock);
+  stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, wsum, sblock);
 }
 
 cudaError_t launch_summary_chunk64(const DataPtrs& in, double* h0_out, void* scratch, int64_t kmin, int64_t N, double T, int D,
@@ -794,7 +804,7 @@ cudaError_t launch_summary_chunk64(const DataPtrs& in, double* h0_out, void* scr
   const int nc = (int)((N + kChunk - 1) / kChunk);
   ChunkRec64* recs = static_cast<ChunkRec64*>(scratch);
   double2* etab = reinterpret_cast<double2*>(recs + nc);
-  k_chunk64<<<(unsigned)((nc + 63) / 64 + 1), 64, 0, s>>>(ref, kmin, T, nc, D, t.tt, recs, etab);
+  k_chunk64<<<(unsigned)((nc + kChunk64Threads - 1) / kChunk64Threads + 1), kChunk64Threads, 0, s>>>(ref, kmin, T, nc, D, t.tt, recs, etab);
   auto kf = D == 1 ? k_summary_chunk64<1> : D == 2 ? k_summary_chunk64<2> : k_summary_chunk64<3>;
   kf<<<(unsigned)n_parts, kStoredThreads, 0, s>>>(in, h0_out, kmin, N, T, B, edges, recs, etab, t.as, so);
   return cudaGetLastError();
