@@ -40,7 +40,7 @@ cudaError_t launch_bin_edges_agnostic(const double* theta_ref_dev, double T, int
 cudaError_t launch_summary(const DataPtrs& in, int64_t kmin, int64_t N, double T, int D, int B,
                            const int64_t* edges, const RefValues* ref, const SummaryOut& so, double* h0_out,
                            cudaStream_t s);
-cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t kmin, int64_t N, double T, int D, int B,
+cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t N, double T, int D, int B,
                                   const int64_t* edges, const SummaryOut& so, int n_parts, cudaStream_t s);
 cudaError_t launch_summary_chunk64(const DataPtrs& in, double* h0_out, void* scratch, int64_t kmin, int64_t N, double T, int D,
                                    int B, const int64_t* edges, const RefValues* ref, const SummaryOut& so, int n_parts,
@@ -1165,7 +1165,7 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
       e.h0_valid = err == cudaSuccess;
       ++launches;
     } else {
-      err = launch_summary_stored(in, e.d_h0, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.out(), e.n_parts, s);
+      err = launch_summary_stored(in, e.d_h0, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.out(), e.n_parts, s);
     }
     e.w32_current = !in_opt && e.w32_resident;
   } else {

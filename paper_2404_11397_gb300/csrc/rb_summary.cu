@@ -498,14 +498,13 @@ __device__ __forceinline__ void stored_part_sums(const double (&acc)[6 * ND], do
 
 template <int ND>
 __global__ void __launch_bounds__(kStoredThreads) k_summary_stored(DataPtrs in, const double* __restrict__ h0,
-                                                                   int64_t kmin, int64_t N, double T, int B,
+                                                                   int64_t N, double inv_T, int B,
                                                                    const int64_t* __restrict__ edges, SummaryOut so) {
   __shared__ double wsum[kStoredThreads / 32][6 * kMaxDet];
   __shared__ double sblock[6 * kMaxDet];
   const int pid = part_of_block(so.n_parts), tid = threadIdx.x;
   const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
   const int b = pd.bin;
-  const double inv_T = 1.0 / T;
   double acc[6 * ND];
 #pragma unroll
   for (int i = 0; i < 6 * ND; ++i) acc[i] = 0.0;
@@ -524,10 +523,10 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_stored(DataPtrs in, 
   stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, wsum, sblock);
 }
 
-cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t kmin, int64_t N, double T, int D, int B,
+cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t N, double T, int D, int B,
                                   const int64_t* edges, const SummaryOut& so, int n_parts, cudaStream_t s) {
   auto kf = D == 1 ? k_summary_stored<1> : D == 2 ? k_summary_stored<2> : k_summary_stored<3>;
-  kf<<<(unsigned)n_parts, kStoredThreads, 0, s>>>(in, h0, kmin, N, T, B, edges, so);
+  kf<<<(unsigned)n_parts, kStoredThreads, 0, s>>>(in, h0, N, 1.0 / T, B, edges, so);  // 1/T: a division by every thread is ~12 FP64 operations
   return cudaGetLastError();
 }
 
@@ -547,8 +546,8 @@ cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t 
 // the others' are taken from it.  ~100 FP64 operations per point with three detectors
 // (an FP64 warp instruction holds its SM sub-partition's FP64 unit for ~65 clocks, so
 // operations are what counts): 519,169 points, 3 detectors, 1000 bins: k_summary 605 us,
-// this kernel 134 us (FP64 pipe 84 % busy) and the records 18 us; the whole rebuild call
-// 640 -> 181 us.  Before detector 0's delay went into the phase, the moments into whole
+// this kernel 131 us (FP64 pipe 84 % busy) and the records 16 us; the whole rebuild call
+// 640 -> 176 us.  Before detector 0's delay went into the phase, the moments into whole
 // steps and the block sums into transposed warp sums it was ~115 operations, 161 us.
 // Errors against FP64 torch sums (2-norm) on four events: A0 1.5e-13 to 2.2e-12 (k_summary
 // 1.4e-13 to 2.2e-12), A1 1.4e-13 to 8.6e-13 (1.5e-13 to 8.6e-13).
@@ -580,9 +579,20 @@ __device__ __forceinline__ void two_sum64(double a, double b, double& s, double&
   e = (a - (s - bb)) + (b - bb);
 }
 
+// exp(-2 pi i x).
+__device__ __forceinline__ double2 cis_neg_turns64(double x) {
+  double sn, pc, w;
+  const int q = quarter_turn64(x, sn, pc, w);
+  const double cs = fma(pc, w, 1.0);
+  // theta = 2 pi r + q pi/2: (cos theta, -sin theta)
+  const double a = (q & 1) ? sn : cs, b = (q & 1) ? cs : sn;
+  const unsigned fa = ((unsigned)(q + 1) & 2u) << 30, fb = ((unsigned)~q & 2u) << 30;  // signs: - for q = 1, 2; - for q = 0, 1
+  return make_double2(__hiloint2double(__double2hiint(a) ^ (int)fa, __double2loint(a)),
+                      __hiloint2double(__double2hiint(b) ^ (int)fb, __double2loint(b)));
+}
+
 // One thread per chunk; the last block forms the offset table
-// etab[d][j] = exp(-2 pi i (j - 16) df (tau_d - tau_0)).  Blocks of four warps, one
-// per SM sub-partition: in blocks of two, half of an SM's FP64 units had no work.
+// etab[d][j] = exp(-2 pi i (j - 16) df (tau_d - tau_0)).
 constexpr int kChunk64Threads = 128;
 __global__ void __launch_bounds__(kChunk64Threads) k_chunk64(const RefValues* __restrict__ ref, int64_t kmin, double T, int n_chunks, int D,
                                                 TaylorTables64 tt, ChunkRec64* __restrict__ recs,
@@ -640,44 +650,28 @@ __global__ void __launch_bounds__(kChunk64Threads) k_chunk64(const RefValues* __
     double x = 0.0;
 #pragma unroll
     for (int k = 0; k < kNBasis; ++k) x = fma(cp[k], k == 6 ? fma(tt.beta6[n], lf, tt.alpha[k][n]) : tt.alpha[k][n], x);
-    r.X[n] = n == 1 ? fma(x, un, v.tau[0] / T) : x * un;
+    r.X[n] = n == 1 ? fma(x, un, v.tau[0] * (fc * u)) : x * un;
     un *= u;
   }
-  const double kamp = 8.035028173395984e-06 / kMpcS;
+  const double a = 8.035028173395984e-06 / kMpcS * v.amp * (sqrt(icf) * P[1]);  // |K| f_c^-7/6 without |P|
 #pragma unroll
   for (int d = 0; d < kMaxDet; ++d) {
     if (d >= D) {
       r.G[d][0] = r.G[d][1] = 0.0;
       continue;
     }
-    double s = 0.0, co = 1.0;
-    if (d > 0) {
-      const double y = fc * (v.tau[d] - v.tau[0]);
-      sincospi(2.0 * (y - rint(y)), &s, &co);
-    }
-    const double a = kamp * v.amp * (sqrt(icf) / fc), Kr = a * v.P64[d][0], Ki = a * v.P64[d][1];
-    r.G[d][0] = Kr * co + Ki * s;  // K exp(-2 pi i y)
-    r.G[d][1] = Ki * co - Kr * s;
+    const double Kr = a * v.P64[d][0], Ki = a * v.P64[d][1];
+    const double2 z = d > 0 ? cis_neg_turns64(fc * (v.tau[d] - v.tau[0])) : make_double2(1.0, 0.0);
+    r.G[d][0] = Kr * z.x - Ki * z.y;
+    r.G[d][1] = Kr * z.y + Ki * z.x;
   }
-}
-
-// exp(-2 pi i x).
-__device__ __forceinline__ double2 cis_neg_turns64(double x) {
-  double sn, pc, w;
-  const int q = quarter_turn64(x, sn, pc, w);
-  const double cs = fma(pc, w, 1.0);
-  // theta = 2 pi r + q pi/2: (cos theta, -sin theta)
-  const double a = (q & 1) ? sn : cs, b = (q & 1) ? cs : sn;
-  const unsigned fa = ((unsigned)(q + 1) & 2u) << 30, fb = ((unsigned)~q & 2u) << 30;  // signs: - for q = 1, 2; - for q = 0, 1
-  return make_double2(__hiloint2double(__double2hiint(a) ^ (int)fa, __double2loint(a)),
-                      __hiloint2double(__double2hiint(b) ^ (int)fb, __double2loint(b)));
 }
 
 // One block per part of a bin, all detectors, as k_summary_stored; h0 goes to
 // h0_out for the builds that follow.
 template <int ND>
 __global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in, double* __restrict__ h0_out, int64_t kmin,
-                                                                    int64_t N, double T, int B,
+                                                                    int64_t N, double inv_T, int B,
                                                                     const int64_t* __restrict__ edges,
                                                                     const ChunkRec64* __restrict__ recs,
                                                                     const double2* __restrict__ etab, AmpSeries64 as,
@@ -704,14 +698,13 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in,
       for (int i = 0; i <= kAmp64; ++i) s_amp[i] = as.c[i];
   }
   const int64_t e0 = edges[b], e1 = edges[b + 1];
-  const double inv_T = 1.0 / T;
   double acc[6 * ND];
 #pragma unroll
   for (int i = 0; i < 6 * ND; ++i) acc[i] = 0.0;
   __syncthreads();
   if (tid < nrec) {
     const int nc = (int)kmin + (c0 + tid) * kChunk + kChunk / 2;
-    su[tid] = 1.0 / (double)nc;
+    su[tid] = rcp_newton(small_int_double(nc));
     int n = kOrd64;
     while (n > 1 && __double_as_longlong(srec[tid].X[n]) == 0) --n;
     sord[tid] = n;
@@ -806,7 +799,7 @@ cudaError_t launch_summary_chunk64(const DataPtrs& in, double* h0_out, void* scr
   double2* etab = reinterpret_cast<double2*>(recs + nc);
   k_chunk64<<<(unsigned)((nc + kChunk64Threads - 1) / kChunk64Threads + 1), kChunk64Threads, 0, s>>>(ref, kmin, T, nc, D, t.tt, recs, etab);
   auto kf = D == 1 ? k_summary_chunk64<1> : D == 2 ? k_summary_chunk64<2> : k_summary_chunk64<3>;
-  kf<<<(unsigned)n_parts, kStoredThreads, 0, s>>>(in, h0_out, kmin, N, T, B, edges, recs, etab, t.as, so);
+  kf<<<(unsigned)n_parts, kStoredThreads, 0, s>>>(in, h0_out, kmin, N, 1.0 / T, B, edges, recs, etab, t.as, so);
   return cudaGetLastError();
 }
 
