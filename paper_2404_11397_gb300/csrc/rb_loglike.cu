@@ -103,13 +103,36 @@ struct __align__(16) WarpSlot {
 struct __align__(16) FusedRecords {
   WalkerMixed rec[kSetupWalkers];
   WalkerTan<float> tan[kSetupWalkers];
+  unsigned long long tan_done;  // mbarrier: the tangent warps, once each
 };
+
+// One-shot mbarrier in shared memory: count arrivals complete its phase 0.
+__device__ __forceinline__ void mbar_init(unsigned long long* b, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long* b) {
+  asm volatile("{.reg .b64 t;\n\tmbarrier.arrive.shared::cta.b64 t, [%0];}" ::"r"((unsigned)__cvta_generic_to_shared(b)) : "memory");
+}
+// Waits for phase 0, at most kMbarTries attempts (a fraction of a second; the
+// arrivals are unconditional, so the limit is not met): false if it gave up.
+constexpr int kMbarTries = 1 << 16;
+__device__ __forceinline__ bool mbar_wait(unsigned long long* b) {
+  for (int i = 0; i < kMbarTries; ++i) {
+    unsigned ok;
+    asm volatile("{.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;}"
+                 : "=r"(ok)
+                 : "r"((unsigned)__cvta_generic_to_shared(b))
+                 : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
 constexpr size_t kFusedWork = sizeof(DdSmem) > (kThreads / 32) * sizeof(WarpWork) ? (sizeof(DdSmem) + 15) / 16 * 16
                                                                                : (kThreads / 32) * sizeof(WarpWork);
 constexpr size_t kFusedBytes = sizeof(FusedRecords) + kFusedWork;
 static_assert(kFusedBytes % 16 == 0, "the MALA chains start on a 16-byte boundary");
 static_assert(sizeof(FusedRecords) % 16 == 0, "the set-up's values start on a 16-byte boundary");
-static_assert(kThreads >= kDdRoleThreads + kTanWarps * 32, "a FUSED block has a warp for every set-up role");
+static_assert(kThreads > kDdRoleThreads && kThreads >= kTanWarps * 32, "a FUSED block has a warp for every set-up role");
 static_assert(sizeof(WalkerMixed) % 16 == 0, "record copied in 16-byte pieces");
 static_assert(sizeof(WalkerTan<float>) <= kTanBytes && sizeof(WalkerTan<float>) % 8 == 0, "tangent buffer");
 
@@ -451,14 +474,18 @@ __device__ __forceinline__ void det_edge_slot(float2 y, float4 rho, float4 sig, 
 // detector pair and the single detector interleave in one instruction stream.
 // ---------------------------------------------------------------------------
 //
-// FUSED: a block of at most kSetupWalkers walkers runs their set-up itself
-// (roles on its first warps, tangents on the next), into shared memory, while
-// the tables are on their way: one launch, no workspace, no records through
+// FUSED: a block of at most kSetupWalkers walkers runs their set-up itself, into
+// shared memory, on its first warps, while the others stage the tables; the tangents,
+// which only a walker's epilogue reads, follow on the last warps (those with the
+// fewest walkers) beside the other warps' slot loops.  Beside the set-up they took its
+// instruction fetches: its first phase 7.5 k clocks instead of 2.5 k, the whole set-up
+// 18 k (2 detectors, 777 walkers) of a launch's 25 k.  One launch, no workspace, no records through
 // memory, and no gap between two kernels.  Small batches are bound by the
 // host's launches and by the set-up's latency: 48 walkers, 1 detector, 100 bins, log L
-// 9.6 -> 8.4 us on the GPU and 15.0 -> 11.4 us per eager call; 3 detectors, 500 bins,
-// with the gradient, on the GPU: 64 walkers 16.2 -> 13.1 us, 4096 walkers 34.9 ->
-// 33.8 us.  More walkers per block than lanes (kSetupWalkers) would run the
+// 9.6 -> 8.1 us on the GPU and 15.0 -> 11.4 us per eager call; 3 detectors, 500 bins,
+// with the gradient, on the GPU: 48 walkers 13.0 -> 12.3 us, 4096 walkers 33.7 -> 33.3 us by
+// the tangents' place and the staging by the other warps alone (1 detector, 100 bins,
+// 4096 walkers 16.9 -> 15.7 us).  More walkers per block than lanes (kSetupWalkers) would run the
 // set-up in turns while the FP32 pipe idles: those batches keep the set-up
 // kernel, whose blocks overlap one another.
 template <int ND, bool GRAD, bool PHASE64, bool MALA, bool FUSED>
@@ -484,13 +511,15 @@ __global__ void __launch_bounds__(kThreads)
   const float4* g4 = nullptr;  // slot image: [kNBasis + 1][NS] basis values and f_e of the slots' edge pairs
   const double* g64 = nullptr;
   const double* f64 = nullptr;
+  constexpr int kStageFrom = FUSED ? kDdRoleThreads : 0;  // a FUSED block's role warps leave it to the others
   {
-    const int tid = threadIdx.x;
+    const int tid = (int)threadIdx.x - kStageFrom, nth = kThreads - kStageFrom;
     if (!PHASE64) {
       const float4* src = reinterpret_cast<const float4*>(ev.slot32);
       float4* dst = reinterpret_cast<float4*>(smem_raw);
       const size_t n4 = ev.slot32_floats / 4;
-      for (size_t i = tid; i < n4; i += blockDim.x) cp_async16(&dst[RB_IDX(i, smem16, 104)], &src[i]);
+      if (tid >= 0)
+        for (size_t i = tid; i < n4; i += nth) cp_async16(&dst[RB_IDX(i, smem16, 104)], &src[i]);
       const float* s = reinterpret_cast<const float*>(smem_raw);
       g4 = reinterpret_cast<const float4*>(s);
       sbin = s + (size_t)4 * (kNBasis + 1) * ev.n_slots;
@@ -498,11 +527,11 @@ __global__ void __launch_bounds__(kThreads)
       const size_t n_e64 = (size_t)(kNBasis + 1) * Ep;  // g[10][Ep], f[Ep]
       const double2* src = reinterpret_cast<const double2*>(ev.tab64);
       double2* dst = reinterpret_cast<double2*>(smem_raw);
-      for (size_t i = tid; i < n_e64 / 2; i += blockDim.x) cp_async16(&dst[RB_IDX(i, smem16, 104)], &src[i]);
+      for (size_t i = tid; i < n_e64 / 2; i += nth) cp_async16(&dst[RB_IDX(i, smem16, 104)], &src[i]);
       const size_t nb = ev.tab32_floats - ev.edge32_floats;
       const float4* bsrc = reinterpret_cast<const float4*>(ev.tab32 + ev.edge32_floats);
       float4* bdst = reinterpret_cast<float4*>(smem_raw + n_e64 * sizeof(double));
-      for (size_t i = tid; i < nb / 4; i += blockDim.x) cp_async16(&bdst[RB_IDX(i, smem16 - n_e64 / 2, 104)], &bsrc[i]);
+      for (size_t i = tid; i < nb / 4; i += nth) cp_async16(&bdst[RB_IDX(i, smem16 - n_e64 / 2, 104)], &bsrc[i]);
       g64 = reinterpret_cast<const double*>(smem_raw);
       f64 = g64 + (size_t)kNBasis * Ep;
       sbin = reinterpret_cast<const float*>(smem_raw + n_e64 * sizeof(double));
@@ -544,12 +573,13 @@ __global__ void __launch_bounds__(kThreads)
   const unsigned char* rec_g = static_cast<const unsigned char*>(a.ws);
   const unsigned char* tan_g = static_cast<const unsigned char*>(a.tan);
   const MalaBlock* chains = nullptr;  // FUSED MALA: the block's chains
+  constexpr int kFusedTanWarps = 3 + D;
+  // FUSED: theta of the block's walkers, the first and the end of its rows
+  const double* theta = nullptr;
+  int64_t t_begin = w_begin, t_end = w_end;
   if constexpr (FUSED) {
+    theta = a.theta;
     DdSmem& S = *reinterpret_cast<DdSmem*>(fused + 1);
-    const int warp = threadIdx.x >> 5;
-    // theta of the block's walkers, the first and the end of its rows
-    const double* theta = a.theta;
-    int64_t t_begin = w_begin, t_end = w_end;
     if constexpr (MALA) {
       MalaBlock* mb = reinterpret_cast<MalaBlock*>(reinterpret_cast<unsigned char*>(fused) + kFusedBytes);
       mala_propose_block(a.mala, w_begin, (int)(w_end - w_begin), *mb);
@@ -558,11 +588,10 @@ __global__ void __launch_bounds__(kThreads)
       t_begin = 0;
       t_end = w_end - w_begin;
     }
-    if (warp < kDdRoleWarps) {
+    if (GRAD && threadIdx.x == kDdRoleThreads) mbar_init(&fused->tan_done, kFusedTanWarps);
+    if (threadIdx.x < kDdRoleThreads) {
       setup_absolute_dd(theta, t_begin, t_end, a.ec, S);
       setup_record_dd(ev.ref->dd, a.ec, S, &fused->rec[lane], w_begin + lane < w_end);
-    } else if (GRAD && warp < kDdRoleWarps + 3 + D) {
-      tangent_warp<float>(theta, t_end, t_begin, a.ec, fused->tan, warp - kDdRoleWarps);
     }
   }
   // the first walker's record and tangents travel with the tables
@@ -571,6 +600,14 @@ __global__ void __launch_bounds__(kThreads)
                                    GRAD ? tan_g + sizeof(WalkerTan<float>) * RB_IDX(warp0, a.W, 107) : nullptr, lane);
   cp_async_wait_all();
   __syncthreads();
+  if constexpr (FUSED && GRAD) {
+    const int which = (int)(threadIdx.x >> 5) - (kThreads / 32 - kFusedTanWarps);
+    if (which >= 0) {
+      tangent_warp<float>(theta, t_end, t_begin, a.ec, fused->tan, which);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&fused->tan_done);
+    }
+  }
   const double base_logl = event_base_value(ev, base_read);
 
   // the bound on |g_k| or f that this lane's phase term takes (the record
@@ -896,9 +933,11 @@ __global__ void __launch_bounds__(kThreads)
         }
       }
       double g = 0.0;
+      bool tan_ok = true;
+      if constexpr (FUSED) tan_ok = mbar_wait(&fused->tan_done);
       if (lane < kNPar) {
         const WalkerTan<float>& tn = FUSED ? fused->tan[wl] : *reinterpret_cast<const WalkerTan<float>*>(slot->tan[buf]);
-        g = f2d_int(chain_rule_lanes<D>(lane, ac, at, ar, tn));
+        g = tan_ok ? f2d_int(chain_rule_lanes<D>(lane, ac, at, ar, tn)) : __longlong_as_double(0x7ff8000000000000ll);
       }
       if constexpr (MALA) mala_step(w, logl, g);
       else if (lane < kNPar) a.grad[RB_IDX(w * kNPar + lane, a.W * kNPar, 106)] = g;
