@@ -24,6 +24,8 @@
 #pragma once
 
 #include <cmath>
+#include <cstdint>
+#include <cstring>
 
 #if defined(__CUDACC__)
 #define RB_DD __host__ __device__ __forceinline__
@@ -98,11 +100,48 @@ RB_DD dd two_prod(float a, float b) {
 
 // --- construction -------------------------------------------------------------
 RB_DD dd from_float(float a) { return {a, 0.f}; }
+// Bit views of doubles and floats.
+RB_DD uint64_t bits_of(double x) {
+#if defined(__CUDA_ARCH__)
+  return (uint64_t)__double_as_longlong(x);
+#else
+  uint64_t u;
+  std::memcpy(&u, &x, sizeof(u));
+  return u;
+#endif
+}
+RB_DD float float_of(uint32_t u) {
+#if defined(__CUDA_ARCH__)
+  return __uint_as_float(u);
+#else
+  float x;
+  std::memcpy(&x, &u, sizeof(x));
+  return x;
+#endif
+}
 // Exact split of a double into h + l (a double has 53 bits, a dd 48: the
 // remainder below the 48th bit is rounded).
 RB_DD dd from_double(double x) {
   const float h = (float)x;
   return {h, (float)(x - (double)h)};
+}
+// The same bits on the integer pipe: the conversion instructions and the subtraction
+// issue on the FP64 pipe, ~65 clocks each.
+// r: the magnitude rounded to nearest even in its top 24 bits, the dropped 29 bits
+// zero (the encoding carries into the exponent by itself).
+RB_DD dd from_double_int(double x) {
+  const uint64_t u = bits_of(x), mag = u & 0x7FFFFFFFFFFFFFFFull;
+  const uint32_t sign = (uint32_t)(u >> 32) & 0x80000000u;
+  if (mag - (963ull << 52) < ((1150ull - 963ull) << 52)) {  // 2^-60 <= |x| < 2^127: no float here is subnormal or rounds to infinity
+    const uint64_t r = (mag + 0x0FFFFFFFull + ((mag >> 29) & 1ull)) & ~0x1FFFFFFFull;
+    // what rounding left, in units of x's last place (also where r is the next power of two)
+    const int rem = (int)(uint32_t)(mag - r);
+    const float unit = float_of(((uint32_t)(mag >> 52) - 948u) << 23);  // 2^(e - 52)
+    // exponent rebiased by 1023 - 127, mod 2^32
+    return {float_of(((uint32_t)(r >> 29) - 0xC0000000u) | sign), mul((float)(sign ? -rem : rem), unit)};
+  }
+  if (mag == 0) return {float_of(sign), 0.f};
+  return from_double(x);
 }
 RB_DD double to_double(dd a) { return (double)a.h + (double)a.l; }
 

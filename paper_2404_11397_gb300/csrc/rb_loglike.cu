@@ -16,8 +16,8 @@
 // With the Newtonian amplitude the ratio has the same modulus |rho_d| at every
 // edge, so Re(r0 r1*) = (|r_{b+1}|^2 - |r_b|^2) / (2 df_b) = 0: the beta1 term
 // (Re t + Re(s t*)/2 = (|1 + delta_{b+1}|^2 - |1 + delta_b|^2) / 2) and its
-// derivatives vanish identically.  The mixed kernel leaves it out (in FP32 it
-// is rounding noise about zero); the plain FP64 kernel keeps the general form.
+// derivatives vanish identically.  The kernels leave it out (in FP32 it is
+// rounding noise about zero; in FP64 leaving it out changes results by 1e-14).
 // delta is formed without cancellation from the half angle:
 //   exp(-2 pi i x) - 1 = -2 sin^2(pi x) - 2 i sin(pi x) cos(pi x),
 //   delta = rho (exp(-2 pi i x) - 1) + (rho - 1).
@@ -590,7 +590,8 @@ __global__ void __launch_bounds__(kThreads)
     }
     if (GRAD && threadIdx.x == kDdRoleThreads) mbar_init(&fused->tan_done, kFusedTanWarps);
     if (threadIdx.x < kDdRoleThreads) {
-      setup_absolute_dd(theta, t_begin, t_end, a.ec, S);
+      setup_load_dd<true>(theta, t_begin, t_end, S);
+      setup_absolute_dd(a.ec, S);
       setup_record_dd(ev.ref->dd, a.ec, S, &fused->rec[lane], w_begin + lane < w_end);
     }
   }

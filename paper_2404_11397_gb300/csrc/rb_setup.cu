@@ -517,7 +517,8 @@ __global__ void __launch_bounds__(kDdRoleThreads) k_ref_dd(const double* theta, 
   // the rebuild + batch step) may start and load its own inputs now; it waits
   // for this grid's completion before it reads the reference values
   asm volatile("griddepcontrol.launch_dependents;");
-  setup_absolute_dd(theta, 0, 1, ec, S);
+  setup_load_dd<true>(theta, 0, 1, S);
+  setup_absolute_dd(ec, S);
   const int j = threadIdx.x;
   RefDD& R = out->dd;
   auto put = [](float* p, dd v) { p[0] = v.h; p[1] = v.l; };
@@ -563,7 +564,8 @@ __global__ void __launch_bounds__(kDdRoleThreads + kTanWarps * 32) k_setup_dd(co
     if (GRAD) tangent_warp<float>(theta, W, w0, ec, static_cast<WalkerTan<float>*>(tan_out) + w0, warp - kDdRoleWarps);
     return;
   }
-  setup_absolute_dd(theta, w0, W, ec, S);
+  setup_load_dd<!GRAD>(theta, w0, W, S);
+  setup_absolute_dd(ec, S);
   setup_record_dd(ref->dd, ec, S, static_cast<WalkerMixed*>(ws_out) + w0 + lane, mine);
 }
 
@@ -590,7 +592,8 @@ __global__ void __launch_bounds__(kDdRoleThreads) k_setup_abs(const double* __re
                                                              EventConst ec, WalkerAbs* __restrict__ out) {
   __shared__ DdSmem S;
   const int64_t w0 = (int64_t)blockIdx.x * kSetupWalkers;
-  setup_absolute_dd(theta, w0, W, ec, S);
+  setup_load_dd<true>(theta, w0, W, S);
+  setup_absolute_dd(ec, S);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t w = w0 + lane;
   if (w >= W) return;

@@ -11,12 +11,15 @@ namespace rb {
 
 constexpr int kSetupWalkers = 32;
 
+// All finite, Mc, q and d_L positive, q <= 1; on the integer pipe (an FP64 comparison
+// holds the FP64 unit like any other FP64 instruction).
 __device__ __forceinline__ bool theta_valid(const double* th) {
   bool ok = true;
-  for (int j = 0; j < kNPar; ++j) ok = ok && isfinite(th[j]);
-  return ok && th[0] > 0.0 && th[1] > 0.0 && th[1] <= 1.0 && th[6] > 0.0;
+#pragma unroll
+  for (int j = 0; j < kNPar; ++j) ok = ok && (__double2hiint(th[j]) & 0x7ff00000) != 0x7ff00000;
+  return ok && __double_as_longlong(th[0]) > 0 && __double_as_longlong(th[1]) > 0 &&
+         __double_as_longlong(th[1]) <= 0x3ff0000000000000ll && __double_as_longlong(th[6]) > 0;
 }
-
 
 // ---------------------------------------------------------------------------
 // Small forward-mode dual numbers for the tangents (T = float or double).
@@ -353,21 +356,29 @@ __device__ __forceinline__ void ddantenna(const DetGeom& g, const dd* t, dd* P) 
   P[1] = fx::neg(mul(fc, ci));
 }
 
-// Phases 1 and 2 of the float-float set-up for the block's walkers (the
-// kDdRoleWarps role warps only), absolute values left in shared memory.
-static __device__ __noinline__ void setup_absolute_dd(const double* __restrict__ theta, int64_t w0, int64_t W,
-                                               const EventConst& ec, DdSmem& S) {
-  using fx::add;
-  using fx::mul;
-  using fx::K;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// The walkers' theta into shared memory, as doubles and float pairs (the role
+// warps).  INT: split on the integer pipe, 0.3 to 0.4 us earlier (of 8 to 13 us of a small
+// batch's launch, 0.6 us of a large one's log L).  Beside tangent warps (k_setup_dd<true>)
+// the longer code costs more than the FP64 pipe's waits, which let those warps run:
+// 0.7 us later.
+template <bool INT>
+static __device__ __noinline__ void setup_load_dd(const double* __restrict__ theta, int64_t w0, int64_t W, DdSmem& S) {
   for (int i = threadIdx.x; i < kNPar * kSetupWalkers; i += kDdRoleThreads) {
     const int l = i / kNPar, j = i % kNPar;
     const int64_t w = (w0 + l < W) ? w0 + l : W - 1;  // pad with the last walker
     const double v = theta[w * kNPar + j];
     S.th[j][l] = v;
-    S.thd[j][l] = st2(fx::from_double(v));
+    S.thd[j][l] = st2(INT ? fx::from_double_int(v) : fx::from_double(v));
   }
+}
+
+// Phases 1 and 2 of the float-float set-up for the block's walkers, loaded by
+// setup_load_dd (the kDdRoleWarps role warps only), absolute values left in shared memory.
+static __device__ __noinline__ void setup_absolute_dd(const EventConst& ec, DdSmem& S) {
+  using fx::add;
+  using fx::mul;
+  using fx::K;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   ddroles_sync();
   const int l = lane;
   switch (warp) {
