@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "rb.h"
+#include "rb_api_internal.h"
 #include "rb_dd.cuh"
 #include "rb_internal.cuh"
 #include "rb_setup_dd.cuh"
@@ -552,10 +553,9 @@ __global__ void __launch_bounds__(kDdRoleThreads) k_ref_dd(const double* theta, 
 // Mixed batch set-up: WalkerMixed (+ float tangents on the warps after the
 // role warps).
 template <bool GRAD>
-__global__ void __launch_bounds__(kDdRoleThreads + kTanWarps * 32) k_setup_dd(const double* __restrict__ theta, int64_t W,
-                                                                 EventConst ec, const RefValues* __restrict__ ref,
-                                                                 void* __restrict__ ws_out,
-                                                                 void* __restrict__ tan_out) {
+__device__ __forceinline__ void setup_dd_block(const double* __restrict__ theta, int64_t W, const EventConst& ec,
+                                               const RefValues* __restrict__ ref, void* __restrict__ ws_out,
+                                               void* __restrict__ tan_out) {
   __shared__ DdSmem S;
   const int64_t w0 = (int64_t)blockIdx.x * kSetupWalkers;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -567,6 +567,22 @@ __global__ void __launch_bounds__(kDdRoleThreads + kTanWarps * 32) k_setup_dd(co
   setup_load_dd<!GRAD>(theta, w0, W, S);
   setup_absolute_dd(ec, S);
   setup_record_dd(ref->dd, ec, S, static_cast<WalkerMixed*>(ws_out) + w0 + lane, mine);
+}
+template <bool GRAD>
+__global__ void __launch_bounds__(kDdRoleThreads + kTanWarps * 32) k_setup_dd(const double* __restrict__ theta, int64_t W,
+                                                                 EventConst ec, const RefValues* __restrict__ ref,
+                                                                 void* __restrict__ ws_out,
+                                                                 void* __restrict__ tan_out) {
+  setup_dd_block<GRAD>(theta, W, ec, ref, ws_out, tan_out);
+}
+// With the gradient, held to the registers of three blocks per SM instead of two (40
+// instead of 72, with spills: a full wave takes about a quarter longer), for
+// batches it spares a wave.
+__global__ void __launch_bounds__(kDdRoleThreads + kTanWarps * 32, 3) k_setup_dd_dense(const double* __restrict__ theta, int64_t W,
+                                                                 EventConst ec, const RefValues* __restrict__ ref,
+                                                                 void* __restrict__ ws_out,
+                                                                 void* __restrict__ tan_out) {
+  setup_dd_block<true>(theta, W, ec, ref, ws_out, tan_out);
 }
 
 // Host-side launchers.
@@ -665,7 +681,13 @@ cudaError_t launch_setup(int mode, const double* theta, int64_t W, const EventCo
                          void* ws, void* tan, bool grad, cudaStream_t s) {
   if (mode == RB_MIXED) {
     const unsigned grid = (unsigned)((W + kSetupWalkers - 1) / kSetupWalkers);
-    if (grad)
+    // the denser form where it takes fewer waves: 12000 walkers are 375 blocks, two
+    // waves of 304 or one of 456 (152 SMs); call with 1 detector, 100 bins 38.4 -> 34.1 us, with 3
+    // detectors, 500 bins 85.4 -> 80.6; at 16384, two waves in either form, it loses 2.7
+    const unsigned n_sm = (unsigned)sm_count(), sparse = (grid + 2 * n_sm - 1) / (2 * n_sm), dense = (grid + 3 * n_sm - 1) / (3 * n_sm);
+    if (grad && dense < sparse)
+      k_setup_dd_dense<<<grid, kDdRoleThreads + kTanWarps * 32, 0, s>>>(theta, W, ec, ref, ws, tan);
+    else if (grad)
       k_setup_dd<true><<<grid, kDdRoleThreads + kTanWarps * 32, 0, s>>>(theta, W, ec, ref, ws, tan);
     else
       k_setup_dd<false><<<grid, kDdRoleThreads, 0, s>>>(theta, W, ec, ref, ws, tan);

@@ -546,7 +546,7 @@ cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t 
 // the others' are taken from it.  ~100 FP64 operations per point with three detectors
 // (an FP64 warp instruction holds its SM sub-partition's FP64 unit for ~65 clocks, so
 // operations are what counts): 519,169 points, 3 detectors, 1000 bins: k_summary 605 us,
-// this kernel 131 us (FP64 pipe 84 % busy) and the records 16 us; the whole rebuild call
+// this kernel 133 us (FP64 pipe 84 % busy) and the records 17 us; the whole rebuild call
 // 640 -> 176 us.  Before detector 0's delay went into the phase, the moments into whole
 // steps and the block sums into transposed warp sums it was ~115 operations, 161 us.
 // Errors against FP64 torch sums (2-norm) on four events: A0 1.5e-13 to 2.2e-12 (k_summary
