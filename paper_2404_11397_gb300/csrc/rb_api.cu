@@ -26,7 +26,7 @@ cudaError_t launch_setup(int mode, const double* theta, int64_t W, const EventCo
 cudaError_t launch_rb_mixed(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl,
                             double* grad, bool phase64, bool spread, cudaStream_t s, int n_sm, const MalaArgs* mala);
 cudaError_t launch_rb_fused(const EventDev& ev, const EventConst& ec, const double* theta, int64_t W, double* logl,
-                            double* grad, bool spread, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done);
+                            double* grad, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done);
 cudaError_t launch_rb_f64(const EventDev& ev, const void* ws, const void* tan, int64_t W, double* logl, double* grad,
                           cudaStream_t s, int n_sm, const MalaArgs* mala);
 cudaError_t launch_bin_edges(double f_low, double f_high, double T, int64_t kmin, int64_t N, int B, int64_t* edges,
@@ -1209,10 +1209,11 @@ int run_batch(const EventEntry* e, const double* theta, int64_t W, double* logl,
   if (!theta || (!logl && !mala)) return set_error(RB_EINVAL, "NULL theta or logl");
   const bool want_grad = grad != nullptr || mala != nullptr;
   // set-up and likelihood in one launch where the batch allows it (not with
-  // trace events, which bracket the likelihood kernel alone)
-  if (mode == RB_MIXED && !mala && !trace_events_set()) {
+  // trace events, which bracket the likelihood kernel alone, nor for launches
+  // that share the GPU with others)
+  if (mode == RB_MIXED && spread && !mala && !trace_events_set()) {
     bool done = false;
-    const cudaError_t ferr = launch_rb_fused(e->dev, e->ec, theta, W, logl, grad, spread, s, sm_count(), nullptr, &done);
+    const cudaError_t ferr = launch_rb_fused(e->dev, e->ec, theta, W, logl, grad, s, sm_count(), nullptr, &done);
     if (ferr != cudaSuccess) return cuda_fail(ferr, "likelihood kernel");
     if (done) {
       count_launches(1);

@@ -1201,7 +1201,7 @@ cudaError_t launch_rb_mixed(const EventDev& ev, const void* ws, const void* tan,
 // records beside them.  With mala the kernel forms the proposals too (theta is not
 // read).
 template <int ND, bool GRAD, bool MALA>
-static cudaError_t launch_fused_nd(const FusedArgs& a, bool spread, cudaStream_t s, int n_sm, bool* done) {
+static cudaError_t launch_fused_nd(const FusedArgs& a, cudaStream_t s, int n_sm, bool* done) {
   auto* fn = k_rb_mixed<ND, GRAD, false, MALA, true>;
   const size_t smem = a.ev.slot32_floats * sizeof(float) + kFusedBytes + (MALA ? sizeof(MalaBlock) : 0);
   *done = false;
@@ -1210,7 +1210,7 @@ static cudaError_t launch_fused_nd(const FusedArgs& a, bool spread, cudaStream_t
   const cudaError_t err = blocks_per_sm(reinterpret_cast<const void*>(fn), kThreads, smem, &per_sm);
   if (err != cudaSuccess) return err;
   if (per_sm < 1) return cudaSuccess;
-  const int64_t grid = mixed_grid(a.W, spread, n_sm, (int64_t)per_sm * n_sm);
+  const int64_t grid = mixed_grid(a.W, true, n_sm, (int64_t)per_sm * n_sm);
   if ((a.W + grid - 1) / grid > kSetupWalkers) return cudaSuccess;
   fn<<<(unsigned)grid, kThreads, smem, s>>>(a);
   *done = true;
@@ -1218,26 +1218,26 @@ static cudaError_t launch_fused_nd(const FusedArgs& a, bool spread, cudaStream_t
 }
 
 template <bool GRAD, bool MALA>
-static cudaError_t launch_fused_t(const FusedArgs& a, bool spread, cudaStream_t s, int n_sm, bool* done) {
+static cudaError_t launch_fused_t(const FusedArgs& a, cudaStream_t s, int n_sm, bool* done) {
   switch (a.ev.n_det) {
-    case 1: return launch_fused_nd<1, GRAD, MALA>(a, spread, s, n_sm, done);
-    case 2: return launch_fused_nd<2, GRAD, MALA>(a, spread, s, n_sm, done);
-    case 3: return launch_fused_nd<3, GRAD, MALA>(a, spread, s, n_sm, done);
+    case 1: return launch_fused_nd<1, GRAD, MALA>(a, s, n_sm, done);
+    case 2: return launch_fused_nd<2, GRAD, MALA>(a, s, n_sm, done);
+    case 3: return launch_fused_nd<3, GRAD, MALA>(a, s, n_sm, done);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_rb_fused(const EventDev& ev, const EventConst& ec, const double* theta, int64_t W, double* logl,
-                            double* grad, bool spread, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done) {
+                            double* grad, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done) {
   FusedArgs a;
   static_cast<LaunchArgs&>(a) = LaunchArgs{ev, nullptr, nullptr, W, logl, grad, {}};
   a.theta = theta;
   a.ec = ec;
   if (mala) {
     a.mala = *mala;
-    return launch_fused_t<true, true>(a, spread, s, n_sm, done);
+    return launch_fused_t<true, true>(a, s, n_sm, done);
   }
-  return grad ? launch_fused_t<true, false>(a, spread, s, n_sm, done) : launch_fused_t<false, false>(a, spread, s, n_sm, done);
+  return grad ? launch_fused_t<true, false>(a, s, n_sm, done) : launch_fused_t<false, false>(a, s, n_sm, done);
 }
 
 template <bool GRAD, bool MALA>

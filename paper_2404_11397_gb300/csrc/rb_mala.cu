@@ -22,7 +22,7 @@
 namespace rb {
 
 cudaError_t launch_rb_fused(const EventDev& ev, const EventConst& ec, const double* theta, int64_t W, double* logl,
-                            double* grad, bool spread, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done);
+                            double* grad, cudaStream_t s, int n_sm, const MalaArgs* mala, bool* done);
 
 struct MalaBox {
   double eps[kNPar], lo[kNPar], hi[kNPar];
@@ -131,7 +131,7 @@ static int mala_run(rb_event_t ev, double* z, double* logp, double* gz, int64_t 
   // 200 bins: a step with its copies 53 -> 47 us.  Not with trace events, which bracket the likelihood kernel.
   if (mode == RB_MIXED && !trace_events_set()) {
     bool done = false;
-    if ((err = launch_rb_fused(e->dev, e->ec, nullptr, W, nullptr, nullptr, true, s, sm_count(), &m, &done)) != cudaSuccess)
+    if ((err = launch_rb_fused(e->dev, e->ec, nullptr, W, nullptr, nullptr, s, sm_count(), &m, &done)) != cudaSuccess)
       return cuda_fail(err, "MALA step kernel");
     if (done) {
       count_launches(1);

@@ -10,14 +10,10 @@
 // A launch runs the packed walkers rounded up to a multiple of 256 (copies of
 // its first walker fill the rest); every walker is computed independently by
 // one warp, so each result is bit-identical to the same request evaluated
-// alone.  The kernels read the walkers from the slot's pinned host buffers and
-// write the results to them over the host link: a launch is one or two kernels
-// (set-up and likelihood in one where the batch allows it) and a completion node.
-// With graphs, each launch is captured and applied to the slot's instantiated
-// graph for its detector count, gradient flag and number of nodes with
-// cudaGraphExecUpdate; the graph is instantiated again only when the update is
-// refused.  Ten requests in flight on four slots: 447 -> 413 us
-// against copies of walkers and results around two kernels.  The
+// alone.  With graphs, each launch is captured (copy-in, set-up, likelihood
+// kernel, copy-out, completion node) and applied to the slot's instantiated
+// graph for its detector count and gradient flag with cudaGraphExecUpdate;
+// the graph is instantiated again only when the update is refused.  The
 // scheduler thread only forms the launches; each slot's own worker thread
 // stages the walkers and issues its launch, so the host work of several
 // launches proceeds in parallel.
@@ -32,7 +28,6 @@
 #include <memory>
 #include <mutex>
 #include <thread>
-#include <tuple>
 #include <unordered_map>
 #include <utility>
 #include <vector>
@@ -64,7 +59,7 @@ struct Slot {
   Server* srv = nullptr;
   cudaStream_t stream = nullptr;
   double *h_theta = nullptr, *h_logl = nullptr, *h_grad = nullptr;  // pinned
-  double *d_theta = nullptr, *d_logl = nullptr, *d_grad = nullptr;  // the same buffers' device addresses
+  double *d_theta = nullptr, *d_logl = nullptr, *d_grad = nullptr;
   void* d_ws = nullptr;
   // the launch on the slot: its requests (walkers in this order from row 0)
   std::vector<Request*> reqs;
@@ -75,7 +70,7 @@ struct Slot {
   bool gpu_done = false;    // the launch's completion node has run; results await the worker (Server::mu)
   std::condition_variable cv_work;
   std::thread worker;
-  std::map<std::tuple<int, bool, size_t>, cudaGraphExec_t> graphs;  // (n_det, grad, nodes) -> instantiated graph (worker only)
+  std::map<std::pair<int, bool>, cudaGraphExec_t> graphs;  // (n_det, grad) -> instantiated graph (worker only)
 };
 
 // What one launch did, for the statistics.
@@ -172,13 +167,21 @@ void Server::fail_slot(Slot* s, int status, const char* why) {
   cv.notify_all();
 }
 
-// Issue the set-up and likelihood kernels and the completion host node on the
-// slot's stream (captured into a graph when enabled).
+// Issue copy-in, set-up + likelihood kernels, copy-out and the completion
+// host node on the slot's stream (captured into a graph when enabled).
 static int enqueue_work(Slot* s, const EventEntry* ev, int64_t W, bool grad, int mode) {
-  const int rc = run_batch(ev, s->d_theta, W, s->d_logl, grad ? s->d_grad : nullptr, mode, s->stream, s->d_ws, nullptr, false);
+  cudaError_t err = cudaMemcpyAsync(s->d_theta, s->h_theta, sizeof(double) * kNPar * W, cudaMemcpyHostToDevice,
+                                    s->stream);
+  if (err != cudaSuccess) return cuda_fail(err, "server copy-in");
+  int rc = run_batch(ev, s->d_theta, W, s->d_logl, grad ? s->d_grad : nullptr, mode, s->stream, s->d_ws, nullptr, false);
   if (rc != RB_OK) return rc;
-  const cudaError_t err = cudaLaunchHostFunc(s->stream, slot_done, s);
-  if (err != cudaSuccess) return cuda_fail(err, "server host node");
+  if ((err = cudaMemcpyAsync(s->h_logl, s->d_logl, sizeof(double) * W, cudaMemcpyDeviceToHost, s->stream)) !=
+      cudaSuccess)
+    return cuda_fail(err, "server copy-out");
+  if (grad && (err = cudaMemcpyAsync(s->h_grad, s->d_grad, sizeof(double) * kNPar * W, cudaMemcpyDeviceToHost,
+                                     s->stream)) != cudaSuccess)
+    return cuda_fail(err, "server copy-out grad");
+  if ((err = cudaLaunchHostFunc(s->stream, slot_done, s)) != cudaSuccess) return cuda_fail(err, "server host node");
   return RB_OK;
 }
 
@@ -208,12 +211,7 @@ int Server::launch(Slot* s, LaunchOutcome* out) {
     return rc;
   }
   if (err != cudaSuccess) return cuda_fail(err, "end capture");
-  size_t n_nodes = 0;
-  if ((err = cudaGraphGetNodes(graph, nullptr, &n_nodes)) != cudaSuccess) {
-    cudaGraphDestroy(graph);
-    return cuda_fail(err, "graph nodes");
-  }
-  const auto key = std::make_tuple(ev->n_det, grad, n_nodes);
+  const auto key = std::make_pair(ev->n_det, grad);
   cudaGraphExec_t exec = nullptr;
   auto it = s->graphs.find(key);
   if (it != s->graphs.end()) {
@@ -240,7 +238,7 @@ int Server::launch(Slot* s, LaunchOutcome* out) {
   for (Request* r : s->reqs) r->t_issued = std::chrono::steady_clock::now();
   err = cudaGraphLaunch(exec, s->stream);
   if (err != cudaSuccess) return cuda_fail(err, "graph launch");
-  count_launches(n_nodes - 1);
+  count_launches(2);
   return RB_OK;
 }
 
@@ -380,7 +378,6 @@ int rb_server_create(const rb_server_opts* opts, rb_server_t* out) {
   if (!srv) return set_error(RB_ENOMEM, "rb_server_create: host allocation");
   Server& S = srv->s;
   S.opts = o;
-  // a walker's inputs and outputs (pinned host memory, mapped) and workspace
   S.bytes_per_walker = sizeof(double) * (2 * kNPar + 1) + walker_ws_bytes(o.mode, true);
   int rc = RB_OK;
   for (int i = 0; i < o.max_slots && rc == RB_OK; ++i) {
@@ -391,9 +388,9 @@ int rb_server_create(const rb_server_opts* opts, rb_server_t* out) {
     if (err == cudaSuccess) err = cudaMallocHost(&sl->h_theta, sizeof(double) * kNPar * cap);
     if (err == cudaSuccess) err = cudaMallocHost(&sl->h_logl, sizeof(double) * cap);
     if (err == cudaSuccess) err = cudaMallocHost(&sl->h_grad, sizeof(double) * kNPar * cap);
-    if (err == cudaSuccess) err = cudaHostGetDevicePointer((void**)&sl->d_theta, sl->h_theta, 0);
-    if (err == cudaSuccess) err = cudaHostGetDevicePointer((void**)&sl->d_logl, sl->h_logl, 0);
-    if (err == cudaSuccess) err = cudaHostGetDevicePointer((void**)&sl->d_grad, sl->h_grad, 0);
+    if (err == cudaSuccess) err = cudaMalloc(&sl->d_theta, sizeof(double) * kNPar * cap);
+    if (err == cudaSuccess) err = cudaMalloc(&sl->d_logl, sizeof(double) * cap);
+    if (err == cudaSuccess) err = cudaMalloc(&sl->d_grad, sizeof(double) * kNPar * cap);
     if (err == cudaSuccess) err = cudaMalloc(&sl->d_ws, walker_ws_bytes(o.mode, true) * cap);
     if (err != cudaSuccess) rc = cuda_fail(err, "rb_server_create: slot buffers");
     S.free_slots.push_back(sl.get());
@@ -436,6 +433,9 @@ int rb_server_destroy(rb_server_t srv) {
     cudaFreeHost(sl->h_theta);
     cudaFreeHost(sl->h_logl);
     cudaFreeHost(sl->h_grad);
+    cudaFree(sl->d_theta);
+    cudaFree(sl->d_logl);
+    cudaFree(sl->d_grad);
     cudaFree(sl->d_ws);
   }
   delete srv;
