@@ -1121,7 +1121,9 @@ __global__ void __launch_bounds__(kSumFastThreads, INBLOCK ? 6 : 8)
   __shared__ double scale[kMaxDet][4];
   __shared__ double s_inv_df;
   __shared__ bool s_last;
-  const int pid = part_of_block(so.n_parts);
+  // (beside the walkers' set-up, in one wave, the order the parts come in: 4096 walkers, 500
+  // bins, the step 55.7 us from the last one down, 55.3 from the first up)
+  const int pid = INBLOCK ? part_of_block(so.n_parts) : (int)blockIdx.x;
   const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
   const int b = pd.bin;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
