@@ -565,7 +565,8 @@ __device__ __forceinline__ void add_acc(V& hi, V& lo, V v) {
 // and sin theta = sn, cos theta = 1 + w pc by their Taylor series (|theta| <= pi/4:
 // the first dropped terms are below 2^-54 of the leading ones).  19 FP64 operations (an FP64 warp
 // instruction holds its SM sub-partition's FP64 unit for ~65 clocks): the
-// quadrant is left to the caller's integer selects.
+// quadrant is left to the caller's integer selects.  |x| < 2^49: the sum with the
+// rounding constant has no unit beyond a quarter turn there.
 __device__ __forceinline__ int quarter_turn64(double x, double& sn, double& pc, double& w) {
   const double magic = 6755399441055744.0;  // 1.5 * 2^52
   const double t = fma(x, 4.0, magic);

@@ -960,6 +960,10 @@ __global__ void __launch_bounds__(kThreads)
 // beta0, beta1, sincospi, butterflies) it was 251 and 100.  1000 walkers, 200
 // bins: 150 -> 79 us (FP64 pipe 84 -> 89 % busy), errors against the oracle unchanged.
 // ---------------------------------------------------------------------------
+// e with |x| < 2^(e + 1) (inf and NaN: the largest).
+__device__ __forceinline__ int exponent64(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+__device__ __forceinline__ int exponent32(float x) { return ((__float_as_int(x) >> 23) & 0xff) - 127; }
+
 template <int ND, bool GRAD, bool MALA = false>
 __global__ void __launch_bounds__(256) k_rb_f64(LaunchArgs a) {
   static_assert(!MALA || GRAD, "the MALA step needs the gradient");
@@ -1003,55 +1007,70 @@ __global__ void __launch_bounds__(256) k_rb_f64(LaunchArgs a) {
     double v[kNV];
 #pragma unroll
     for (int i = 0; i < kNV; ++i) v[i] = 0.0;
-    for (int c0 = 0; c0 < B; c0 += 31) {
-      const int e = c0 + lane;
-      const bool has_edge = e < E;
-      const bool has_bin = (lane < 31) && (e < B);
-      const int ee = has_edge ? e : E - 1, eb = has_bin ? e : 0;
-      double x = 0.0;
+    // a walker whose phase may reach 2^49 turns (a delay of 1e12 s, say) loses the whole
+    // turns of its phases before the quarter-turn reduction.  From the exponents of its terms
+    // c_k g_k and f tau, on the integer pipe: eleven terms below 2^(m + 2) each
+    int m = -4096;
 #pragma unroll
-      for (int k = 0; k < kNBasis; ++k) x = fma(dc[k], g64[k * Ep + ee], x);
-      const double fe = f64[ee];
-      double adj_x = 0.0;
+    for (int k = 0; k < kNBasis; ++k) m = max(m, exponent64(dc[k]) + exponent32(ev.gmax[k]));
 #pragma unroll
-      for (int d = 0; d < ND; ++d) {
-        double em_r, em_i;
-        expm1_neg_turns64(fma(fe, tau[d], x), em_r, em_i);
-        const double dr = fma(rho[d][0], em_r, fma(-rho[d][1], em_i, sig[d][0]));
-        const double di = fma(rho[d][0], em_i, fma(rho[d][1], em_r, sig[d][1]));
-        const double nr = __shfl_down_sync(kFull, dr, 1);
-        const double ni = __shfl_down_sync(kFull, di, 1);
-        // the bin on the edge's right; zero coefficients where there is none
-        const double* bt = bin64 + (size_t)d * 6 * Bp + eb;
-        const double gmr = has_bin ? bt[0] : 0.0, gpr = has_bin ? bt[Bp] : 0.0, gmi = has_bin ? bt[2 * Bp] : 0.0;
-        const double gpi = has_bin ? bt[3 * Bp] : 0.0, q = has_bin ? bt[5 * Bp] : 0.0;
-        const double sr = dr + nr, si = di + ni;
-        v[0] = fma(gmr, dr, v[0]);
-        v[0] = fma(gpr, nr, v[0]);
-        v[0] = fma(gmi, di, v[0]);
-        v[0] = fma(gpi, ni, v[0]);
-        v[0] = fma(q, fma(sr, sr, si * si), v[0]);
-        if (GRAD) {
-          const double h = has_bin ? bt[4 * Bp] : 0.0;
-          double gr = fma(h, sr, gmr), gi = fma(h, si, gmi);
-          const double lr = __shfl_up_sync(kFull, fma(h, sr, gpr), 1), li = __shfl_up_sync(kFull, fma(h, si, gpi), 1);
-          gr += lane > 0 ? lr : 0.0;
-          gi += lane > 0 ? li : 0.0;
-          if (has_edge) {
-            const double rr = 1.0 + dr;
-            const double dldx = fma(gr, di, -(gi * rr));  // Im(conj(gbar) r)
-            adj_x += dldx;
-            v[1 + kNBasis + d] = fma(dldx, fe, v[1 + kNBasis + d]);
-            v[1 + kNBasis + ND + d] = fma(gr, rr, fma(gi, di, v[1 + kNBasis + ND + d]));
-            v[1 + kNBasis + 2 * ND + d] += dldx;
+    for (int d = 0; d < ND; ++d) m = max(m, exponent64(tau[d]) + exponent32(ev.gmax[kNBasis]));
+    // (as a second copy of the loop: one with the test inside took 98.9 us for 96.3)
+    auto edges = [&](auto far_c) {
+      for (int c0 = 0; c0 < B; c0 += 31) {
+        const int e = c0 + lane;
+        const bool has_edge = e < E;
+        const bool has_bin = (lane < 31) && (e < B);
+        const int ee = has_edge ? e : E - 1, eb = has_bin ? e : 0;
+        double x = 0.0;
+  #pragma unroll
+        for (int k = 0; k < kNBasis; ++k) x = fma(dc[k], g64[k * Ep + ee], x);
+        const double fe = f64[ee];
+        double adj_x = 0.0;
+  #pragma unroll
+        for (int d = 0; d < ND; ++d) {
+          double em_r, em_i;
+          double y = fma(fe, tau[d], x);
+          if constexpr (decltype(far_c)::value) y -= rint(y);
+          expm1_neg_turns64(y, em_r, em_i);
+          const double dr = fma(rho[d][0], em_r, fma(-rho[d][1], em_i, sig[d][0]));
+          const double di = fma(rho[d][0], em_i, fma(rho[d][1], em_r, sig[d][1]));
+          const double nr = __shfl_down_sync(kFull, dr, 1);
+          const double ni = __shfl_down_sync(kFull, di, 1);
+          // the bin on the edge's right; zero coefficients where there is none
+          const double* bt = bin64 + (size_t)d * 6 * Bp + eb;
+          const double gmr = has_bin ? bt[0] : 0.0, gpr = has_bin ? bt[Bp] : 0.0, gmi = has_bin ? bt[2 * Bp] : 0.0;
+          const double gpi = has_bin ? bt[3 * Bp] : 0.0, q = has_bin ? bt[5 * Bp] : 0.0;
+          const double sr = dr + nr, si = di + ni;
+          v[0] = fma(gmr, dr, v[0]);
+          v[0] = fma(gpr, nr, v[0]);
+          v[0] = fma(gmi, di, v[0]);
+          v[0] = fma(gpi, ni, v[0]);
+          v[0] = fma(q, fma(sr, sr, si * si), v[0]);
+          if (GRAD) {
+            const double h = has_bin ? bt[4 * Bp] : 0.0;
+            double gr = fma(h, sr, gmr), gi = fma(h, si, gmi);
+            const double lr = __shfl_up_sync(kFull, fma(h, sr, gpr), 1), li = __shfl_up_sync(kFull, fma(h, si, gpi), 1);
+            gr += lane > 0 ? lr : 0.0;
+            gi += lane > 0 ? li : 0.0;
+            if (has_edge) {
+              const double rr = 1.0 + dr;
+              const double dldx = fma(gr, di, -(gi * rr));  // Im(conj(gbar) r)
+              adj_x += dldx;
+              v[1 + kNBasis + d] = fma(dldx, fe, v[1 + kNBasis + d]);
+              v[1 + kNBasis + ND + d] = fma(gr, rr, fma(gi, di, v[1 + kNBasis + ND + d]));
+              v[1 + kNBasis + 2 * ND + d] += dldx;
+            }
           }
         }
+        if (GRAD && has_edge) {
+  #pragma unroll
+          for (int k = 0; k < kNBasis; ++k) v[1 + k] = fma(adj_x, g64[k * Ep + ee], v[1 + k]);
+        }
       }
-      if (GRAD && has_edge) {
-#pragma unroll
-        for (int k = 0; k < kNBasis; ++k) v[1 + k] = fma(adj_x, g64[k * Ep + ee], v[1 + k]);
-      }
-    }
+    };
+    if (m < 49 - 6) edges(std::false_type{});
+    else edges(std::true_type{});
     warp_transposed_sums(v, lane, red);
     __syncwarp();
     const double logl = base_logl + red[0];

@@ -579,7 +579,7 @@ __device__ __forceinline__ void two_sum64(double a, double b, double& s, double&
   e = (a - (s - bb)) + (b - bb);
 }
 
-// exp(-2 pi i x).
+// exp(-2 pi i x), |x| < 2^49.
 __device__ __forceinline__ double2 cis_neg_turns64(double x) {
   double sn, pc, w;
   const int q = quarter_turn64(x, sn, pc, w);
@@ -650,7 +650,11 @@ __global__ void __launch_bounds__(kChunk64Threads) k_chunk64(const RefValues* __
     double x = 0.0;
 #pragma unroll
     for (int k = 0; k < kNBasis; ++k) x = fma(cp[k], k == 6 ? fma(tt.beta6[n], lf, tt.alpha[k][n]) : tt.alpha[k][n], x);
-    r.X[n] = n == 1 ? fma(x, un, v.tau[0] * (fc * u)) : x * un;
+    x = n == 1 ? fma(x, un, v.tau[0] * (fc * u)) : x * un;
+    // j^n is an integer: whole turns can go.  They do where 2^10 turns per step or more (a
+    // theta_ref far from anything the grid samples) would take the sum beyond the range of cis_neg_turns64
+    if ((__double2hiint(x) & 0x7fffffff) >= 0x40900000) x -= rint(x);
+    r.X[n] = x;
     un *= u;
   }
   const double a = 8.035028173395984e-06 / kMpcS * v.amp * (sqrt(icf) * P[1]);  // |K| f_c^-7/6 without |P|
