@@ -1152,21 +1152,20 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     e.w32_current = true;
     err = launch_summary_parts(e.d_w32, e.d_is32, e.d_wexp, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref,
                                e.d_chunkq, ss ? e.d_chunks : nullptr, e.out(), s);
-  } else if (e.h0_valid || chunk64) {
+  } else if (chunk64) {
+    err = launch_summary_chunk64(in, e.d_h0, e.d_chunks, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref, e.out(),
+                                 e.n_parts, s);
+    e.h0_valid = err == cudaSuccess;
+    ++launches;
+    e.w32_current = !in_opt && e.w32_resident;
+  } else if (e.h0_valid) {
     // FP64 sums from the fiducial waveform stored by the last inline build
     // for this theta_ref: strain, PSD and h0 streamed, no waveform arithmetic;
     // its fixed-point sum starts from zero (a fast build leaves it set)
     if ((err = cudaMemsetAsync(&e.d_sync->base_acc, 0, sizeof(unsigned long long), s)) != cudaSuccess ||
         (err = cudaMemsetAsync(&e.d_sync->overflow, 0, sizeof(unsigned), s)) != cudaSuccess)
       return cuda_fail(err, "zero counters");
-    if (chunk64) {
-      err = launch_summary_chunk64(in, e.d_h0, e.d_chunks, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref, e.out(),
-                                   e.n_parts, s);
-      e.h0_valid = err == cudaSuccess;
-      ++launches;
-    } else {
-      err = launch_summary_stored(in, e.d_h0, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.out(), e.n_parts, s);
-    }
+    err = launch_summary_stored(in, e.d_h0, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.out(), e.n_parts, s);
     e.w32_current = !in_opt && e.w32_resident;
   } else {
     // FP64 waveform generated inline, and stored for the next builds

@@ -452,9 +452,10 @@ __device__ __forceinline__ int part_of_block(int n_parts) { return n_parts - 1 -
 // The end of the FP64 builds that take one block per part of a bin: the block's
 // sums of the per-thread sums acc (six per detector, terms over S without the
 // factor 4 df, moments in units of half a grid step), the parts of a bin added in index order by the last of them to
-// finish, which runs the FP64 epilogue (base log L by the fixed-point sum).
+// finish, which runs the FP64 epilogue (base log L as fixed_base says: the fixed-point
+// sum rounds every bin's share to 2^-32, the FP64 sum of the shares costs the last block ~1 us).
 template <int ND>
-__device__ __forceinline__ void stored_part_sums(const double (&acc)[6 * ND], double inv_T, int pid, const PartDesc& pd, int b, int B, const SummaryOut& so,
+__device__ __forceinline__ void stored_part_sums(bool fixed_base, const double (&acc)[6 * ND], double inv_T, int pid, const PartDesc& pd, int b, int B, const SummaryOut& so,
                                                  double (*wsum)[6 * kMaxDet], double* sblock) {
   __shared__ bool s_last;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -493,7 +494,7 @@ __device__ __forceinline__ void stored_part_sums(const double (&acc)[6 * ND], do
   }
   if (tid < 6 * ND) sblock[tid] = mine;
   __syncthreads();
-  summary_epilogue(so, b, 0, ND, B, ND, sblock, nullptr, false, (unsigned)B, so.inv_df[b], true);
+  summary_epilogue(so, b, 0, ND, B, ND, sblock, nullptr, false, (unsigned)B, so.inv_df[b], fixed_base);
 }
 
 template <int ND>
@@ -520,7 +521,7 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_stored(DataPtrs in, 
       add_terms(&acc[6 * d], w, n, dv, hv.x, hv.y, hv.x * hv.x + hv.y * hv.y);
     }
   }
-  stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, wsum, sblock);
+  stored_part_sums<ND>(true, acc, inv_T, pid, pd, b, B, so, wsum, sblock);
 }
 
 cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t N, double T, int D, int B,
@@ -762,7 +763,7 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in,
       add_terms(&acc[6 * d], rcp_newton(S[d]), n, dv[d], hr, hi, a2 * sg2[d][ci]);
     }
   }
-  stored_part_sums<ND>(acc, inv_T, pid, pd, b, B, so, wsum, sblock);
+  stored_part_sums<ND>(false, acc, inv_T, pid, pd, b, B, so, wsum, sblock);
 }
 
 cudaError_t launch_summary_chunk64(const DataPtrs& in, double* h0_out, void* scratch, int64_t kmin, int64_t N, double T, int D,
