@@ -166,10 +166,10 @@ RB_API int rb_event_free(rb_event_t ev);
  * it (16 B per point and detector, counted in device_bytes); later FP64 builds
  * with the same theta_ref stream the strain, the PSD and that stored h0
  * instead of regenerating it (the same sums in another order, within FP64
- * rounding), and a theta_ref argument discards it.  A call that brings a
- * theta_ref generates h0 from an FP64 Taylor expansion per 32-point chunk of the
- * grid (T f_low >= 1024, N <= 2^30; within FP64 rounding of the evaluation at every point that
- * other builds, and event creation, take).  RB_MIXED / RB_MIXED_F64PHASE: the
+ * rounding), and a theta_ref argument discards it.  h0 is generated from an FP64
+ * Taylor expansion per 32-point chunk of the grid where T f_low >= 1024 and N <= 2^30
+ * (at every point elsewhere), by event creation and by every rebuild alike: an event
+ * created at theta_ref and one rebuilt to it hold the same bits.  RB_MIXED / RB_MIXED_F64PHASE: the
  * fiducial phase is expanded in a Taylor series per 32-point chunk of the
  * grid (coefficients in FP64) and every grid point is evaluated in FP32 and
  * float-pair arithmetic, which keeps the per-point work off the FP64 pipe

@@ -542,7 +542,7 @@ int rb_event_rebuild(rb_event_t ev, const double* theta_ref_host, const double* 
       }
     }
   }
-  return rebuild_event(e, have ? &in : nullptr, mode, s, nullptr, theta_ref_host != nullptr);
+  return rebuild_event(e, have ? &in : nullptr, mode, s);
 }
 
 void rb_set_trace_events(void* before_main, void* after_main) { set_trace_events(before_main, after_main); }
@@ -1063,7 +1063,7 @@ int rb_strain(const double* geom, double gmst, const double* theta_host, double 
 
 namespace rb {
 
-int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t s, const SideSetup* ss, bool new_ref) {
+int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t s, const SideSetup* ss) {
   cudaError_t err;
   DataPtrs in{};
   if (in_opt) {
@@ -1075,12 +1075,13 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     }
   }
   const bool fast = mode != RB_FP64 && e.kmin >= 1024 && e.N <= (int64_t(1) << 30);
-  // FP64 sums with h0 generated: for a theta_ref given with the call from FP64
-  // Taylor chunks; otherwise (the event's creation, or a rebuild behind a change of
-  // theta_ref that kept h0 away) directly at every point, so that a saved event
-  // loads to the bits it has after an FP64 rebuild
-  const bool chunk64 = mode == RB_FP64 && new_ref && !e.h0_valid && e.kmin >= 1024 && e.N <= (int64_t(1) << 30) &&
-                       e.kmin <= (int64_t(1) << 30);
+  // FP64 sums with h0 generated: from FP64 Taylor chunks wherever the grid admits
+  // them, whatever call brought theta_ref (the event's creation, this rebuild or
+  // one before it), so that h0's bits depend on the data, theta_ref and the grid
+  // alone and a saved event loads to the bits it has after an FP64 rebuild.
+  // (k_summary_chunk64 counts points from 0 Hz in 32 bits)
+  const bool chunk64 = mode == RB_FP64 && !e.h0_valid && e.kmin >= 1024 && e.N <= (int64_t(1) << 30) &&
+                       e.kmin < (int64_t(1) << 30) - kChunk;
   if (ss && !(fast && mode == RB_MIXED)) return set_error(RB_EINVAL, "overlapped set-up needs the mixed fast rebuild");
   // Both sets of reference values are rebuilt: the float-float set (mixed
   // path, fast summary) and the FP64 set (FP64 paths, FP64 summary).  The
@@ -1153,13 +1154,14 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     err = launch_summary_parts(e.d_w32, e.d_is32, e.d_wexp, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref,
                                e.d_chunkq, ss ? e.d_chunks : nullptr, e.out(), s);
   } else if (chunk64) {
+    // h0 generated from Taylor chunks, and stored for the next builds
     err = launch_summary_chunk64(in, e.d_h0, e.d_chunks, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref, e.out(),
                                  e.n_parts, s);
     e.h0_valid = err == cudaSuccess;
     ++launches;
     e.w32_current = !in_opt && e.w32_resident;
   } else if (e.h0_valid) {
-    // FP64 sums from the fiducial waveform stored by the last inline build
+    // FP64 sums from the fiducial waveform stored by the last build that generated it
     // for this theta_ref: strain, PSD and h0 streamed, no waveform arithmetic;
     // its fixed-point sum starts from zero (a fast build leaves it set)
     if ((err = cudaMemsetAsync(&e.d_sync->base_acc, 0, sizeof(unsigned long long), s)) != cudaSuccess ||
@@ -1168,7 +1170,7 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     err = launch_summary_stored(in, e.d_h0, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.out(), e.n_parts, s);
     e.w32_current = !in_opt && e.w32_resident;
   } else {
-    // FP64 waveform generated inline, and stored for the next builds
+    // FP64 waveform evaluated at every point, and stored for the next builds
     err = launch_summary(in, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref, e.out(), e.d_h0, s);
     e.h0_valid = err == cudaSuccess;
     e.w32_current = !in_opt && e.w32_resident;

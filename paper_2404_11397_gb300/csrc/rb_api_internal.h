@@ -46,7 +46,7 @@ struct EventEntry {
   bool h0_valid = false;      // d_h0 holds h0 for the current theta_ref
   double* d_theta_ref = nullptr;
   void* d_chunkq = nullptr;   // event-constant per-chunk Taylor matrices (fast summary build)
-  void* d_chunks = nullptr;   // per-rebuild chunk records (rebuild + batch step; FP64 build with a new theta_ref)
+  void* d_chunks = nullptr;   // per-rebuild chunk records (rebuild + batch step; FP64 build that generates h0)
   double* d_invdf = nullptr;  // [B] 1 / bin width
   double* d_share = nullptr;  // [D][B] per-bin shares of log L(theta_ref)
   SummarySync* d_sync = nullptr;  // build counters (zero between builds)
@@ -140,10 +140,7 @@ struct SideSetup {
   bool grad;
   cudaEvent_t data_ready;  // if not NULL: the resident data are complete only after this event
 };
-// new_ref: the call brings a theta_ref (an FP64 build then generates h0 from FP64
-// Taylor chunks instead of evaluating it at every point).
-int rebuild_event(EventEntry& e, const DataPtrs* in, int mode, cudaStream_t s, const SideSetup* side_setup = nullptr,
-                  bool new_ref = false);
+int rebuild_event(EventEntry& e, const DataPtrs* in, int mode, cudaStream_t s, const SideSetup* side_setup = nullptr);
 // Stream-ordered allocation from the library's memory pool (see rb_api.cu).
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s);
 int rebuild_and_batch(EventEntry& e, const double* theta, int64_t W, double* logl, double* grad, int mode,

@@ -532,7 +532,7 @@ cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t 
 }
 
 // ===========================================================================
-// FP64 build with a new fiducial point: h0 from FP64 Taylor chunks.
+// FP64 build that generates h0 (event creation, a new theta_ref): FP64 Taylor chunks.
 //
 // k_summary evaluates h0_d at every grid point and detector from scratch (log, cbrt,
 // ten basis terms, sincos: ~500 FP64 operations per point with three
@@ -550,12 +550,14 @@ cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t 
 // this kernel 133 us (FP64 pipe 84 % busy) and the records 17 us; the whole rebuild call
 // 640 -> 176 us.  Before detector 0's delay went into the phase, the moments into whole
 // steps and the block sums into transposed warp sums it was ~115 operations, 161 us.
-// Errors against FP64 torch sums (2-norm) on four events: A0 1.5e-13 to 2.2e-12 (k_summary
-// 1.4e-13 to 2.2e-12), A1 1.4e-13 to 8.6e-13 (1.5e-13 to 8.6e-13).
+// Errors against quad-precision sums with the same coefficients (2-norm) on four events,
+// two reference points each: A0 1.4e-14 to 6.7e-14 (k_summary 1.1e-13 to 1.7e-13; this
+// form with the centres' powers rounded to FP64 1.2e-13 to 1.7e-13), A1 2.2e-14 to
+// 6.1e-14 (1.0e-13 to 1.7e-13; 1.0e-13 to 2.6e-13).
 // A record keeps the orders
 // that reach 2^-48 turns at the chunk's ends (up to 9 of them); X_0, up to
-// thousands of turns, is reduced to [-1/2, 1/2] before it is rounded, so the phase's
-// error stays that of the basis functions, as in k_summary.
+// thousands of turns, is formed in double-double and reduced to [-1/2, 1/2] before it is
+// rounded, so that the phase carries no rounding of its thousands of turns.
 // Needs kmin >= 1024 (|j u| <= 1/64: order 10 is below 2^-46 turns).  The records
 // take the place of the rebuild + batch step's (128 B per chunk).
 // ===========================================================================
@@ -609,12 +611,27 @@ __global__ void __launch_bounds__(kChunk64Threads) k_chunk64(const RefValues* __
   }
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n_chunks) return;
-  const double nc = (double)(kmin + (int64_t)c * kChunk + kChunk / 2), fc = nc / T, u = 1.0 / nc;
+  const double nc = (double)(kmin + (int64_t)c * kChunk + kChunk / 2), fc = nc / T, u = rcp_newton(nc);
   const double cf = cbrt(fc), lf = log(fc), icf = 1.0 / cf, icf2 = icf * icf;
-  const double P[kNBasis] = {icf2 * icf2 * icf, 1.0 / fc, icf2, icf, 1.0, cf, cf, cf * cf, fc * cf * cf, fc * fc * cf};
+  double P[kNBasis] = {icf2 * icf2 * icf, icf2 * icf, icf2, icf, 1.0, cf, cf, cf * cf, fc * cf * cf, fc * fc * cf};
   ChunkRec64& r = recs[c];
   // X_0 = [Phi0 + sum_k c_k g_k(f_c)] / 2 pi: the two largest terms (up to ~1e4 rad)
-  // added last, in double-double, and the quotient rounded after the whole turns go
+  // added last, in double-double, and the quotient rounded after the whole turns go.
+  // Their powers f_c^-5/3, f_c^-1 as P + pl: a rounding of theirs would be common to the
+  // chunk's 32 points, where the evaluation at every point averages over as many
+  const double rho = fma(-fc, T, nc) * u;  // f_c (1 + rho) = nc / T
+  double pl[2];
+  {
+    // icf^3 f_c (1 + rho) = 1 + 3 eps: icf (1 - eps) is f_c^-1/3
+    const double i2e = fma(icf, icf, -icf2), i3 = P[1], i3e = fma(icf2, icf, -i3) + i2e * icf;
+    const double o = i3 * fc, oe = fma(i3, fc, -o) + i3e * fc;
+    const double eps = ((o - 1.0) + (oe + rho)) * (1.0 / 3.0);
+    const double i4 = icf2 * icf2, i4e = fma(icf2, icf2, -i4) + 2.0 * (icf2 * i2e);
+    pl[0] = fma(i4, icf, -P[0]) + (i4e * icf - 5.0 * (eps * P[0]));
+    const double d = i3e - 3.0 * (eps * i3);
+    P[1] = i3 + d;  // (the amplitude takes it too)
+    pl[1] = d - (P[1] - i3);
+  }
   double cp[kNBasis], sh = v.phi0, sl = 0.0;
 #pragma unroll
   for (int k = kNBasis - 1; k >= 0; --k) {
@@ -623,7 +640,7 @@ __global__ void __launch_bounds__(kChunk64Threads) k_chunk64(const RefValues* __
     if (k >= 2) {
       sh = fma(v.c[k], g, sh);
     } else {
-      const double p = v.c[k] * g, pe = fma(v.c[k], g, -p);
+      const double p = v.c[k] * g, pe = fma(v.c[k], g, -p) + v.c[k] * pl[k];
       double e;
       two_sum64(sh, p, sh, e);
       sl += e + pe;
