@@ -326,8 +326,8 @@ RB_API int rb_mala_step(rb_event_t ev, double* z_dev, double* logp_dev, double* 
  * mode: RB_MIXED only.  Needs T f_low >= 1024 and n_freq <= 2^30 (the chunk
  * expansion), and, if the last rebuild read caller data in place in RB_FP64
  * mode, a rebuild in a mixed mode or from resident data first.  Asynchronous
- * on `stream`; a workspace of 224 B per walker comes from the stream-ordered
- * pool.  Errors: RB_EINVAL (NULL pointers, W < 0, bad mode, grid outside the
+ * on `stream`; a workspace of 176 B per walker and at most 64 MiB for the sums
+ * (48 B per walker and group of grid segments) comes from the stream-ordered pool.  Errors: RB_EINVAL (NULL pointers, W < 0, bad mode, grid outside the
  * expansion's range, data not available), RB_ENOMEM, RB_ECUDA. */
 RB_API int rb_loglike_full_batch(rb_event_t ev, const double* theta_dev, int64_t W, double* logl_dev, int mode,
                                  void* stream);

@@ -70,6 +70,7 @@ constexpr int full_smem(int nd) {
 
 // Segments per group: up to 64 groups.
 constexpr int kGroups = 64;
+constexpr int kTileBytes = 64 << 20;  // the groups' sums held at a time
 __host__ __device__ constexpr int group_segments(int n_seg) { return (n_seg + kGroups - 1) / kGroups; }
 
 // One level of a transposed warp sum of float pairs: lanes whose bit o is clear
@@ -447,10 +448,11 @@ extern "C" int rb_loglike_full_batch(rb_event_t ev, const double* theta_dev, int
   // group) pairs
   const int nc = (int)((e.N + kChunk - 1) / kChunk);
   const int n_seg = (nc + kSegC - 1) / kSegC, gs = group_segments(n_seg), n_groups = (n_seg + gs - 1) / gs;
-  const int64_t units = (W + kFullWarps - 1) / kFullWarps * n_groups;
-  const unsigned blocks = (unsigned)std::min<int64_t>(units, 2 * (int64_t)sm_count());
+  // the groups' sums (up to 3 KB per walker) of so many walkers at a time: a batch
+  // beyond that takes several pairs of launches, each of tens of units per block
+  const int64_t tile = std::min<int64_t>(W, kTileBytes / (int)(sizeof(double) * 6 * kFullWarps) / n_groups * kFullWarps);
   char* buf = nullptr;
-  const size_t abs_bytes = sizeof(WalkerAbs) * W, z_bytes = sizeof(double) * 6 * W * n_groups;
+  const size_t abs_bytes = sizeof(WalkerAbs) * W, z_bytes = sizeof(double) * 6 * tile * n_groups;
   err = ws_alloc(reinterpret_cast<void**>(&buf), abs_bytes + z_bytes, s);
   if (err != cudaSuccess) return cuda_fail(err, "rb_loglike_full_batch: workspace allocation");
   WalkerAbs* wabs = reinterpret_cast<WalkerAbs*>(buf);
@@ -461,13 +463,18 @@ extern "C" int rb_loglike_full_batch(rb_event_t ev, const double* theta_dev, int
   if ((err = launch_setup_abs(theta_dev, W, e.ec, wabs, s)) != cudaSuccess) {
     rc = cuda_fail(err, "rb_loglike_full_batch: set-up kernel");
   } else {
-    kz<<<blocks, kFullThreads, smem, s>>>(static_cast<const float2*>(e.d_w32), (int)e.N,
-                                          static_cast<const float*>(e.d_chunkq), nc, wabs, W, ih, il, zout);
-    constexpr int per_block = kFinishThreads / kFinishLanes;
-    k_full_finish<<<(unsigned)((W + per_block - 1) / per_block), kFinishThreads, 0, s>>>(
-        zout, n_groups, wabs, W, e.n_det, e.n_bins, e.T, e.d_wexp, e.d_summ, e.d_ref, logl_dev);
-    if ((err = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(err, "rb_loglike_full_batch: kernels");
-    else count_launches(3);
+    count_launches(1);
+    for (int64_t w0 = 0; w0 < W && rc == RB_OK; w0 += tile) {
+      const int64_t n = std::min(tile, W - w0), units = (n + kFullWarps - 1) / kFullWarps * n_groups;
+      const unsigned blocks = (unsigned)std::min<int64_t>(units, 2 * (int64_t)sm_count());
+      kz<<<blocks, kFullThreads, smem, s>>>(static_cast<const float2*>(e.d_w32), (int)e.N,
+                                            static_cast<const float*>(e.d_chunkq), nc, wabs + w0, n, ih, il, zout);
+      constexpr int per_block = kFinishThreads / kFinishLanes;
+      k_full_finish<<<(unsigned)((n + per_block - 1) / per_block), kFinishThreads, 0, s>>>(
+          zout, n_groups, wabs + w0, n, e.n_det, e.n_bins, e.T, e.d_wexp, e.d_summ, e.d_ref, logl_dev + w0);
+      if ((err = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(err, "rb_loglike_full_batch: kernels");
+      else count_launches(2);
+    }
   }
   cudaFreeAsync(buf, s);
   return rc;
