@@ -64,6 +64,7 @@ cudaError_t launch_pull32(const DataPtrs& src, int64_t N, int D, double* data, d
 // ---- diagnostics ----
 static thread_local char g_err[512] = "no error";
 static std::atomic<uint64_t> g_launches{0};
+static thread_local uint64_t t_launches = 0;  // this thread's share: what a capture on it enqueued
 static std::atomic<uint64_t> g_event_uid{0};
 
 int set_error(int code, const char* fmt, ...) {
@@ -73,7 +74,10 @@ int set_error(int code, const char* fmt, ...) {
   va_end(ap);
   return code;
 }
-void count_launches(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+void count_launches(uint64_t n) {
+  g_launches.fetch_add(n, std::memory_order_relaxed);
+  t_launches += n;
+}
 
 int cuda_fail(cudaError_t e, const char* what) {
   if (e == cudaErrorMemoryAllocation) return set_error(RB_ENOMEM, "%s: %s", what, cudaGetErrorString(e));
@@ -786,9 +790,9 @@ static bool host_batch_graph(EventEntry& e, const double* theta, int64_t W, doub
     cudaGetLastError();
     return false;
   }
-  const uint64_t n0 = g_launches.load();
+  const uint64_t n0 = t_launches;
   const int rc = run_batch(&e, theta, W, logl, grad, mode, e.hg_stream, e.hg_ws);
-  e.hg_launches = g_launches.load() - n0;
+  e.hg_launches = t_launches - n0;
   count_launches((uint64_t)0 - e.hg_launches);  // the capture launched nothing
   err = cudaStreamEndCapture(e.hg_stream, &g);
   cudaGraphExec_t exec = nullptr;
@@ -910,9 +914,9 @@ static bool host_step_graph(EventEntry& e, const DataPtrs& src, const double* th
     cudaGetLastError();
     return false;
   }
-  const uint64_t n0 = g_launches.load();
+  const uint64_t n0 = t_launches;
   const int rc = enqueue_host_step(e, src, theta, W, logl, grad, mode, e.hg_stream);
-  const uint64_t n = g_launches.load() - n0;
+  const uint64_t n = t_launches - n0;
   count_launches((uint64_t)0 - n);  // the capture launched nothing
   cudaGraph_t g = nullptr;
   err = cudaStreamEndCapture(e.hg_stream, &g);
