@@ -1215,8 +1215,11 @@ int run_batch(const EventEntry* e, const double* theta, int64_t W, double* logl,
   const bool want_grad = grad != nullptr || mala != nullptr;
   // set-up and likelihood in one launch where the batch allows it (not with
   // trace events, which bracket the likelihood kernel alone, nor for launches
-  // that share the GPU with others)
-  if (mode == RB_MIXED && spread && !mala && !trace_events_set()) {
+  // that share the GPU with others, nor into theta's own memory: some blocks of that
+  // kernel write results before others have read their walkers)
+  const size_t theta_bytes = sizeof(double) * kNPar * W;
+  if (mode == RB_MIXED && spread && !mala && !trace_events_set() && !overlap(theta, theta_bytes, logl, sizeof(double) * W) &&
+      !(grad && overlap(theta, theta_bytes, grad, theta_bytes))) {
     bool done = false;
     const cudaError_t ferr = launch_rb_fused(e->dev, e->ec, theta, W, logl, grad, s, sm_count(), nullptr, &done);
     if (ferr != cudaSuccess) return cuda_fail(ferr, "likelihood kernel");

@@ -149,6 +149,12 @@ int rebuild_and_batch(EventEntry& e, const double* theta, int64_t W, double* log
 cudaError_t launch_batch_main(const EventEntry* e, void* ws, void* tan, int64_t W, double* logl, double* grad, int mode,
                               bool spread, cudaStream_t s, const MalaArgs* mala);
 
+// Whether [a, a + na) and [b, b + nb) share a byte (NULL: no).
+inline bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x && y && x < y + nb && y < x + na;
+}
+
 // Events recorded on the launch stream right before / after the main
 // likelihood kernel of every batch (NULL disables).
 void set_trace_events(void* before, void* after);

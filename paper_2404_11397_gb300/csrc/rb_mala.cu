@@ -128,8 +128,9 @@ static int mala_run(rb_event_t ev, double* z, double* logp, double* gz, int64_t 
   cudaError_t err;
   // Mixed batches that take the set-up and likelihood in one launch (rb_loglike.cu)
   // take the proposals there too: one kernel, no workspace.  1000 chains, 3 detectors,
-  // 200 bins: a step with its copies 53 -> 47 us.  Not with trace events, which bracket the likelihood kernel.
-  if (mode == RB_MIXED && !trace_events_set()) {
+  // 200 bins: a step with its copies 53 -> 47 us.  Not with trace events, which bracket the likelihood kernel,
+  // nor with the answers in the draws' memory, which other blocks may not have read yet.
+  if (mode == RB_MIXED && !trace_events_set() && !overlap(accepted, sizeof(int) * W, u, sizeof(double) * W)) {
     bool done = false;
     if ((err = launch_rb_fused(e->dev, e->ec, nullptr, W, nullptr, nullptr, s, sm_count(), &m, &done)) != cudaSuccess)
       return cuda_fail(err, "MALA step kernel");
