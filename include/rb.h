@@ -71,6 +71,13 @@ extern "C" {
 #define RB_MIXED 0          /* phase in float-float (FP32 pairs), trig/ratio/contraction FP32, sums FP64 */
 #define RB_FP64 1           /* everything in native FP64 (comparison path) */
 #define RB_MIXED_F64PHASE 2 /* phase accumulated in native FP64, rest as RB_MIXED */
+/* Or'ed to the mode of rb_loglike_batch, rb_loglike_grad_batch, rb_mala_init or rb_mala_step
+ * (other calls refuse it): the call shares the GPU with others in flight, on other
+ * streams or on other branches of a graph.  By default a batch of up to ~32 walkers per
+ * SM is spread over all SMs, one block per SM, which is the fastest form of a call
+ * that has the GPU to itself; with the flag it takes few, dense blocks and a set-up
+ * kernel of its own, slower alone but with room for the others.  Same results, bit for bit. */
+#define RB_SHARED 0x100
 /* RB_MIXED sums each walker's phase from FP32 pairs with exact high parts
  * scaled to the walker's largest phase term |dc_k g_k(f)|, |dtau_d f| over the
  * band.  A walker with such a term beyond 2^18 turns (~1.6e6 rad: far outside

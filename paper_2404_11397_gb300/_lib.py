@@ -17,7 +17,9 @@ RB_EINVAL, RB_ENOMEM, RB_ECUDA, RB_ETIMEDOUT, RB_EBUSY, RB_ENOTFOUND, RB_ECLOSED
 RB_MIXED, RB_FP64, RB_MIXED_F64PHASE = 0, 1, 2
 RB_BINS_PN, RB_BINS_AGNOSTIC = 0, 1
 BIN_SCHEMES = {"pn": RB_BINS_PN, "agnostic": RB_BINS_AGNOSTIC}
-MODES = {"mixed": RB_MIXED, "fp64": RB_FP64, "mixed_f64phase": RB_MIXED_F64PHASE}
+RB_SHARED = 0x100  # batch and MALA calls: or'ed to the mode of calls that share the GPU with others in flight
+MODES = {"mixed": RB_MIXED, "fp64": RB_FP64, "mixed_f64phase": RB_MIXED_F64PHASE,
+         "mixed_shared": RB_MIXED | RB_SHARED, "mixed_f64phase_shared": RB_MIXED_F64PHASE | RB_SHARED}
 NPAR = 13
 MAX_DET = 3
 RB_STATIC_MAX_WALKERS = 8192

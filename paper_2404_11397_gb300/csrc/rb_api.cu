@@ -704,7 +704,8 @@ int rb_event_get_summary(rb_event_t ev, double* A0, double* A1, double* B0, doub
 int rb_loglike_grad_batch(rb_event_t ev, const double* theta_dev, int64_t W, double* logl_dev, double* grad_dev,
                           int mode, void* stream) {
   RB_NVTX("rb_loglike_grad_batch");
-  return rb::run_batch(event_entry(ev), theta_dev, W, logl_dev, grad_dev, mode, (cudaStream_t)stream, nullptr);
+  return rb::run_batch(event_entry(ev), theta_dev, W, logl_dev, grad_dev, mode & ~RB_SHARED, (cudaStream_t)stream, nullptr, nullptr,
+                       !(mode & RB_SHARED));
 }
 
 namespace rb {
@@ -732,7 +733,8 @@ int rb_rebuild_loglike_grad(rb_event_t ev, const double* theta_dev, int64_t W, d
 
 int rb_loglike_batch(rb_event_t ev, const double* theta_dev, int64_t W, double* logl_dev, int mode, void* stream) {
   RB_NVTX("rb_loglike_batch");
-  return rb::run_batch(event_entry(ev), theta_dev, W, logl_dev, nullptr, mode, (cudaStream_t)stream, nullptr);
+  return rb::run_batch(event_entry(ev), theta_dev, W, logl_dev, nullptr, mode & ~RB_SHARED, (cudaStream_t)stream, nullptr, nullptr,
+                       !(mode & RB_SHARED));
 }
 
 namespace rb {

@@ -119,7 +119,7 @@ size_t walker_ws_bytes(int mode, bool grad);
 // Set-up + likelihood kernels for one batch; scratch = NULL takes the
 // workspace from the stream-ordered allocator.  With mala, the likelihood
 // kernel finishes each walker with the MALA accept step (logl, grad unused).
-// spread = false for launches that share the GPU with others (the server's):
+// spread = false for launches that share the GPU with others (the server's, and RB_SHARED):
 // few, dense blocks instead of a small batch spread over every SM.
 int run_batch(const EventEntry* e, const double* theta, int64_t W, double* logl, double* grad, int mode,
               cudaStream_t s, void* scratch, const MalaArgs* mala = nullptr, bool spread = true);

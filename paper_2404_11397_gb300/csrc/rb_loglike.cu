@@ -1169,10 +1169,12 @@ constexpr int64_t kThinWalkers = 4;  // an SM's sub-partitions
 // Blocks of a batch of W walkers, at most n_max.  spread: a batch that does not
 // fill the SMs with 16 walkers per block takes more of them, down to one walker
 // per SM sub-partition (the warps of a block share its FP32 pipe; below four
-// walkers nothing is left to share).  GPU time of a call, 3 detectors, 500
-// bins, with the gradient: 64 walkers 24.1 -> 16.2 us, 1024 walkers 24.2 -> 18.4
-// us.  Otherwise (launches that share the GPU with others) the blocks stay
-// dense: fewer SMs are held, for longer.
+// walkers nothing is left to share).  Otherwise (launches that share the GPU with
+// others: the server's, RB_SHARED) the blocks stay dense: fewer SMs are held, for
+// longer.  A call of 1024 walkers with the gradient, 3 detectors, 500 bins, one after
+// the other on one stream: spread (and in one launch with the set-up, see FUSED) 18.4
+// us, dense 24.7; on eight branches of a graph: 15.6 and 7.9.  (64 walkers: 12.3 and
+// 25.0; 2.1 and 3.5.)
 static int64_t mixed_grid(int64_t W, bool spread, int n_sm, int64_t n_max) {
   const int64_t dense = (W * 32 + kThreads - 1) / kThreads;
   const int64_t thin = spread ? std::min<int64_t>((W + kThinWalkers - 1) / kThinWalkers, n_sm) : 0;

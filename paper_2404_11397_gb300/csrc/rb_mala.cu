@@ -99,6 +99,8 @@ static int mala_run(rb_event_t ev, double* z, double* logp, double* gz, int64_t 
   if (W == 0) return RB_OK;
   if (!z || !logp || !gz || !lo_host || !hi_host) return set_error(RB_EINVAL, "%s: NULL argument", who);
   if (!init && (!eps_host || !xi || !u)) return set_error(RB_EINVAL, "%s: NULL eps, xi or u", who);
+  const bool spread = !(mode & RB_SHARED);
+  mode &= ~RB_SHARED;
   if (mode != RB_MIXED && mode != RB_FP64 && mode != RB_MIXED_F64PHASE) return set_error(RB_EINVAL, "%s: bad mode %d", who, mode);
   MalaBox box;
   for (int j = 0; j < kNPar; ++j) {
@@ -129,8 +131,9 @@ static int mala_run(rb_event_t ev, double* z, double* logp, double* gz, int64_t 
   // Mixed batches that take the set-up and likelihood in one launch (rb_loglike.cu)
   // take the proposals there too: one kernel, no workspace.  1000 chains, 3 detectors,
   // 200 bins: a step with its copies 53 -> 47 us.  Not with trace events, which bracket the likelihood kernel,
-  // nor with the answers in the draws' memory, which other blocks may not have read yet.
-  if (mode == RB_MIXED && !trace_events_set() && !overlap(accepted, sizeof(int) * W, u, sizeof(double) * W)) {
+  // nor with the answers in the draws' memory, which other blocks may not have read yet, nor
+  // with RB_SHARED.
+  if (mode == RB_MIXED && spread && !trace_events_set() && !overlap(accepted, sizeof(int) * W, u, sizeof(double) * W)) {
     bool done = false;
     if ((err = launch_rb_fused(e->dev, e->ec, nullptr, W, nullptr, nullptr, s, sm_count(), &m, &done)) != cudaSuccess)
       return cuda_fail(err, "MALA step kernel");
@@ -160,7 +163,7 @@ static int mala_run(rb_event_t ev, double* z, double* logp, double* gz, int64_t 
     m.lu = lu;
     m.jac = jac;
     m.inside = inside;
-    rc = run_batch(e, theta, W, nullptr, nullptr, mode, s, nullptr, &m);
+    rc = run_batch(e, theta, W, nullptr, nullptr, mode, s, nullptr, &m, spread);
   }
   cudaFreeAsync(buf, s);
   return rc;
