@@ -18,6 +18,10 @@ from . import _lib
 from ._lib import MODES, NPAR, check, load
 
 
+# torch's private accessors of the current stream's handle; where a torch has none, its Stream object serves
+_raw_stream, _raw_device = (getattr(torch._C, name, None) for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+
+
 def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
     """The cudaStream_t of the given stream, or of the current one.  Addresses are
     passed to the C ABI as plain ints (its prototypes convert them): a Stream
@@ -25,9 +29,11 @@ def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
     about a third of its host time."""
     if stream is not None:
         return stream.cuda_stream
+    if _raw_stream is None or _raw_device is None:
+        return torch.cuda.current_stream().cuda_stream
     if not torch.cuda.is_initialized():
         torch.cuda.init()
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_raw_device())
 
 
 def _mode(mode) -> int:
