@@ -284,10 +284,10 @@ RB_API int rb_rebuild_loglike_grad_host(rb_event_t ev, const double* const* data
  * its gradient) for host buffers:
  * copies theta_host [W][13] to the device, evaluates, copies logl_host [W]
  * (and grad_host [W][13] unless NULL) back, and synchronises the stream.
- * pinned, mapped, 8-byte-aligned theta_host is read by the set-up kernel
+ * pinned, mapped, 8-byte-aligned theta_host is read by the kernels
  * over the host link (no copy in), and such logl_host/grad_host are written
  * by the likelihood kernel directly (no copy back).  With all three pinned,
- * the set-up and likelihood launches are captured as a CUDA graph the first
+ * the launches (one kernel for up to ~32 walkers per SM, otherwise set-up and likelihood) are captured as a CUDA graph the first
  * time for these buffers, W and mode, and replayed by the following calls
  * with the same ones (as for rb_rebuild_loglike_grad_host). */
 RB_API int rb_loglike_grad_host(rb_event_t ev, const double* theta_host, int64_t W, double* logl_host, double* grad_host,

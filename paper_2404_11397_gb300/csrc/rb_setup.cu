@@ -653,8 +653,8 @@ cudaError_t launch_tangents(const double* theta, int64_t W, const EventConst& ec
 }
 
 // Phase directions of the fiducial waveform for the bin placement without the
-// PN ansatz: dc_k / dtheta_j at theta_ref (the FP64 dual numbers of the FP64
-// set-up's tangents), out[k][j] for j = Mc, q, chi1, chi2, Lambda1, Lambda2.
+// PN ansatz: dc_k / dtheta_j at theta_ref (the mixed tangents' dual numbers in
+// FP64), out[k][j] for j = Mc, q, chi1, chi2, Lambda1, Lambda2.
 // With the basis functions g_k they give dPsi(f) / dtheta_j = sum_k out[k][j] g_k(f);
 // the constant phase does not vary with f and is not needed.
 __global__ void k_ref_phase_tangents(const double* __restrict__ theta_ref, double* __restrict__ out) {

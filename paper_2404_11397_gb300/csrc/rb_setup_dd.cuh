@@ -357,8 +357,8 @@ __device__ __forceinline__ void ddantenna(const DetGeom& g, const dd* t, dd* P) 
 }
 
 // The walkers' theta into shared memory, as doubles and float pairs (the role
-// warps).  INT: split on the integer pipe, 0.3 to 0.4 us earlier (of 8 to 13 us of a small
-// batch's launch, 0.6 us of a large one's log L).  Beside tangent warps (k_setup_dd<true>)
+// warps).  INT: split on the integer pipe, 0.2 us earlier (of 8 to 33 us of a batch in
+// one launch; 0.6 us of a large one's log L, 28 to 81 us).  Beside tangent warps (k_setup_dd<true>)
 // the longer code costs more than the FP64 pipe's waits, which let those warps run:
 // 0.7 us later.
 template <bool INT>

@@ -1143,8 +1143,8 @@ __global__ void __launch_bounds__(kSumFastThreads, INBLOCK ? 6 : 8)
   __shared__ double scale[kMaxDet][4];
   __shared__ double s_inv_df;
   __shared__ bool s_last;
-  // (beside the walkers' set-up, in one wave, the order the parts come in: 4096 walkers, 500
-  // bins, the step 55.7 us from the last one down, 55.3 from the first up)
+  // (beside the walkers' set-up, in one wave, the order the parts come in: from the last one
+  // down the step of 4096 walkers, 500 bins was 0.4 us of 56 longer, within its spread)
   const int pid = INBLOCK ? part_of_block(so.n_parts) : (int)blockIdx.x;
   const PartDesc pd = so.parts[RB_IDX(pid, so.n_parts, 201)];
   const int b = pd.bin;
