@@ -423,6 +423,13 @@ __device__ __forceinline__ double rcp_newton(double S) {
   return fma(r, fma(e, e, e), r);
 }
 
+// Point k of a detector's strain, read once.  Data read in place from the caller need not
+// start on a 16-byte boundary: one load where they do, two elsewhere.
+__device__ __forceinline__ double2 strain_at(const double* __restrict__ p, int64_t k) {
+  if ((reinterpret_cast<uintptr_t>(p) & 8) == 0) return __ldcs(reinterpret_cast<const double2*>(p) + k);
+  return make_double2(__ldcs(p + 2 * k), __ldcs(p + 2 * k + 1));
+}
+
 // Integer -> double, exactly, by one FP64 addition (the conversion instruction
 // issues on the FP64 pipe too, and the 64-bit one more than once): 1.5 2^52 + i
 // put together with integer operations.
@@ -515,7 +522,7 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_stored(DataPtrs in, 
   for (int64_t k = pd.start + tid; k < pd.end; k += kStoredThreads, n += 2.0 * kStoredThreads) {
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
-      const double2 dv = __ldcs(reinterpret_cast<const double2*>(in.data[d]) + RB_IDX(k, N, 222));
+      const double2 dv = strain_at(in.data[d], RB_IDX(k, N, 222));
       const double2 hv = __ldcs(reinterpret_cast<const double2*>(h0) + (size_t)d * N + RB_IDX(k, N, 222));
       const double w = rcp_newton(__ldcs(in.psd[d] + k));
       add_terms(&acc[6 * d], w, n, dv, hv.x, hv.y, hv.x * hv.x + hv.y * hv.y);
@@ -756,7 +763,7 @@ __global__ void __launch_bounds__(kStoredThreads) k_summary_chunk64(DataPtrs in,
     double S[ND];
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
-      dv[d] = __ldcs(reinterpret_cast<const double2*>(in.data[d]) + RB_IDX(k, N, 222));
+      dv[d] = strain_at(in.data[d], RB_IDX(k, N, 222));
       S[d] = __ldcs(in.psd[d] + k);
     }
     const int ci = RB_IDX((int)(k / kChunk) - c0, kRecs, 203);
@@ -1043,7 +1050,7 @@ __global__ void __launch_bounds__(256) k_data32(DataPtrs in, int64_t N, int D, f
     exps[2 * d + 1] = sS;
   }
   if (k >= N) return;
-  const double2 dv = __ldcs(reinterpret_cast<const double2*>(in.data[d]) + k);
+  const double2 dv = strain_at(in.data[d], k);
   const float Sp = scaled_float(__ldcs(in.psd[d] + k), (unsigned)(896 - sS) << 20);
   const float is = __frcp_rn(Sp);
   const unsigned bd = (unsigned)(896 - sd) << 20;
