@@ -173,10 +173,11 @@ RB_API int rb_event_free(rb_event_t ev);
  * it (16 B per point and detector, counted in device_bytes); later FP64 builds
  * with the same theta_ref stream the strain, the PSD and that stored h0
  * instead of regenerating it (the same sums in another order, within FP64
- * rounding), and a theta_ref argument discards it.  h0 is generated from an FP64
- * Taylor expansion per 32-point chunk of the grid where T f_low >= 1024 and N <= 2^30
- * (at every point elsewhere), by event creation and by every rebuild alike: an event
- * created at theta_ref and one rebuilt to it hold the same bits.  RB_MIXED / RB_MIXED_F64PHASE: the
+ * rounding), and a theta_ref argument discards it.  A call that brings a
+ * theta_ref generates h0 from an FP64 Taylor expansion per 32-point chunk of the
+ * grid (T f_low >= 1024, N <= 2^30); other builds, and event creation, evaluate it at
+ * every point.  The two agree within FP64 rounding, not bit for bit: an event rebuilt to
+ * theta_ref and one created at it may differ in the last bits.  RB_MIXED / RB_MIXED_F64PHASE: the
  * fiducial phase is expanded in a Taylor series per 32-point chunk of the
  * grid (coefficients in FP64) and every grid point is evaluated in FP32 and
  * float-pair arithmetic, which keeps the per-point work off the FP64 pipe
@@ -202,10 +203,11 @@ RB_API int rb_event_get_summary(rb_event_t ev, double* A0, double* A1, double* B
  * [n_det][n_freq], behind a fixed header (native byte order).  It first
  * synchronises the device, so that calls already issued on any stream are
  * included.  rb_event_load reads such a file and builds a new event from it
- * with rb_build_summary (host data, `stream` as the build stream, synchronous).
- * The build is deterministic, so the loaded event's grid, bins, summary data,
- * tables and log L values are bit-identical to those of an event built from
- * the same inputs.  Errors: RB_EINVAL (NULL argument, unreadable or unwritable
+ * as rb_build_summary does (host data, `stream` as the build stream, synchronous),
+ * with h0 generated as in the event that was saved: after rb_build_summary, and after a
+ * RB_FP64 rebuild that generated h0, the loaded event's grid, bins, summary data, tables
+ * and log L values are bit-identical to the saved one's; after other rebuilds, to those
+ * of an event built from the same inputs.  Errors: RB_EINVAL (NULL argument, unreadable or unwritable
  * path, a file that is not a complete event file, or an event whose last
  * rebuild read caller data in place: it holds no copy of that data);
  * rb_build_summary's errors on load; RB_ECUDA. */

@@ -320,8 +320,8 @@ int rb_event_free(rb_event_t ev) {
   return RB_OK;
 }
 
-int rb_build_summary(const rb_event_desc* desc, rb_event_t* out) {
-  RB_NVTX("rb_build_summary");
+// chunk_h0: h0 from Taylor chunks (rebuild_event), as the event that was saved had it.
+static int build_event(const rb_event_desc* desc, rb_event_t* out, bool chunk_h0) {
   if (!desc || !out) return set_error(RB_EINVAL, "rb_build_summary: NULL descriptor or output");
   *out = nullptr;
   const int D = desc->n_det, B = desc->n_bins;
@@ -488,7 +488,7 @@ int rb_build_summary(const rb_event_desc* desc, rb_event_t* out) {
     if ((err = launch_edge_tables(kmin, e.T, D, B, Ep, Bp, e.d_edges, e.d_tab32, edge32, e.d_tab64, e.d_invdf, e.d_slot32, NS, s)) != cudaSuccess) { rc = cuda_fail(err, "edge table kernel"); break; }
     if ((err = launch_chunk_q(kmin, e.T, N, e.d_chunkq, s)) != cudaSuccess) { rc = cuda_fail(err, "chunk matrix kernel"); break; }
     count_launches(4);
-    if ((rc = rebuild_event(e, nullptr, RB_FP64, s)) != RB_OK) break;
+    if ((rc = rebuild_event(e, nullptr, RB_FP64, s, nullptr, chunk_h0)) != RB_OK) break;
     if ((err = cudaStreamSynchronize(s)) != cudaSuccess) { rc = cuda_fail(err, "build synchronise"); break; }
     double span = 0.0;
     if ((err = cudaMemcpy(&span, d_span, sizeof(double), cudaMemcpyDeviceToHost)) != cudaSuccess) { rc = cuda_fail(err, "read bin span"); break; }
@@ -506,6 +506,11 @@ int rb_build_summary(const rb_event_desc* desc, rb_event_t* out) {
   }
   *out = ev;
   return RB_OK;
+}
+
+int rb_build_summary(const rb_event_desc* desc, rb_event_t* out) {
+  RB_NVTX("rb_build_summary");
+  return build_event(desc, out, false);
 }
 
 int rb_event_rebuild(rb_event_t ev, const double* theta_ref_host, const double* const* data, const double* const* psd,
@@ -546,7 +551,7 @@ int rb_event_rebuild(rb_event_t ev, const double* theta_ref_host, const double* 
       }
     }
   }
-  return rebuild_event(e, have ? &in : nullptr, mode, s);
+  return rebuild_event(e, have ? &in : nullptr, mode, s, nullptr, theta_ref_host != nullptr);
 }
 
 void rb_set_trace_events(void* before_main, void* after_main) { set_trace_events(before_main, after_main); }
@@ -597,7 +602,8 @@ struct EventFileHeader {  // followed by strain [n_det][n_freq][2] and PSD [n_de
   double T, f_low, f_high, gmst;
   double geom[RB_MAX_DET][5];
   double theta_ref[RB_NPAR];
-  int32_t bin_scheme, reserved;
+  int32_t bin_scheme;
+  int32_t chunk_h0;  // 1: the FP64 summary's h0 came from Taylor chunks (0 in files written before there was a choice)
 };
 }  // namespace
 
@@ -619,6 +625,7 @@ int rb_event_save(rb_event_t ev, const char* path) {
   std::memcpy(h.geom, e.geom, sizeof(h.geom));
   std::memcpy(h.theta_ref, e.theta_ref, sizeof(h.theta_ref));
   h.bin_scheme = e.bin_scheme;
+  h.chunk_h0 = e.h0_valid && e.h0_chunks ? 1 : 0;
   const size_t nd = (size_t)2 * e.n_det * e.N, np = (size_t)e.n_det * e.N;
   std::vector<double> data(nd), psd(np);
   // the resident copy, after every call already issued on any stream
@@ -679,7 +686,7 @@ int rb_event_load(const char* path, void* stream, rb_event_t* out) {
     dd.data = data.data() + (size_t)2 * d * h.n_freq;
     dd.psd = psd.data() + (size_t)d * h.n_freq;
   }
-  return rb_build_summary(&desc, out);
+  return build_event(&desc, out, h.chunk_h0 == 1);
 }
 
 int rb_event_get_summary(rb_event_t ev, double* A0, double* A1, double* B0, double* B1, int64_t* edges) {
@@ -1069,7 +1076,7 @@ int rb_strain(const double* geom, double gmst, const double* theta_host, double 
 
 namespace rb {
 
-int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t s, const SideSetup* ss) {
+int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t s, const SideSetup* ss, bool chunk_h0) {
   cudaError_t err;
   DataPtrs in{};
   if (in_opt) {
@@ -1081,12 +1088,12 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     }
   }
   const bool fast = mode != RB_FP64 && e.kmin >= 1024 && e.N <= (int64_t(1) << 30);
-  // FP64 sums with h0 generated: from FP64 Taylor chunks wherever the grid admits
-  // them, whatever call brought theta_ref (the event's creation, this rebuild or
-  // one before it), so that h0's bits depend on the data, theta_ref and the grid
-  // alone and a saved event loads to the bits it has after an FP64 rebuild.
-  // (k_summary_chunk64 counts points from 0 Hz in 32 bits)
-  const bool chunk64 = mode == RB_FP64 && !e.h0_valid && e.kmin >= 1024 && e.N <= (int64_t(1) << 30) &&
+  // FP64 sums with h0 generated: from FP64 Taylor chunks for a theta_ref given with the
+  // call, where the grid admits them; otherwise (creation, or a rebuild behind a change
+  // of theta_ref that kept h0 away) directly at every point, so that events keep the bits
+  // they are created with.  Which of the two it was is saved with the event: loading
+  // takes the same one.  (k_summary_chunk64 counts points from 0 Hz in 32 bits)
+  const bool chunk64 = mode == RB_FP64 && chunk_h0 && !e.h0_valid && e.kmin >= 1024 && e.N <= (int64_t(1) << 30) &&
                        e.kmin < (int64_t(1) << 30) - kChunk;
   if (ss && !(fast && mode == RB_MIXED)) return set_error(RB_EINVAL, "overlapped set-up needs the mixed fast rebuild");
   // Both sets of reference values are rebuilt: the float-float set (mixed
@@ -1164,6 +1171,7 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     err = launch_summary_chunk64(in, e.d_h0, e.d_chunks, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref, e.out(),
                                  e.n_parts, s);
     e.h0_valid = err == cudaSuccess;
+    e.h0_chunks = true;
     ++launches;
     e.w32_current = !in_opt && e.w32_resident;
   } else if (e.h0_valid) {
@@ -1179,6 +1187,7 @@ int rebuild_event(EventEntry& e, const DataPtrs* in_opt, int mode, cudaStream_t 
     // FP64 waveform evaluated at every point, and stored for the next builds
     err = launch_summary(in, e.kmin, e.N, e.T, e.n_det, e.n_bins, e.d_edges, e.d_ref, e.out(), e.d_h0, s);
     e.h0_valid = err == cudaSuccess;
+    e.h0_chunks = false;
     e.w32_current = !in_opt && e.w32_resident;
   }
   e.last_in_place = in_opt != nullptr;

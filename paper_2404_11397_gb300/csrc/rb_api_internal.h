@@ -44,9 +44,10 @@ struct EventEntry {
   double* d_psd = nullptr;    // resident PSD [D][N]
   double* d_h0 = nullptr;     // stored fiducial waveform h0_d(f) [D][N][2] (FP64 builds)
   bool h0_valid = false;      // d_h0 holds h0 for the current theta_ref
+  bool h0_chunks = false;     // ... generated from Taylor chunks
   double* d_theta_ref = nullptr;
   void* d_chunkq = nullptr;   // event-constant per-chunk Taylor matrices (fast summary build)
-  void* d_chunks = nullptr;   // per-rebuild chunk records (rebuild + batch step; FP64 build that generates h0)
+  void* d_chunks = nullptr;   // per-rebuild chunk records (rebuild + batch step; FP64 build with a new theta_ref)
   double* d_invdf = nullptr;  // [B] 1 / bin width
   double* d_share = nullptr;  // [D][B] per-bin shares of log L(theta_ref)
   SummarySync* d_sync = nullptr;  // build counters (zero between builds)
@@ -140,7 +141,10 @@ struct SideSetup {
   bool grad;
   cudaEvent_t data_ready;  // if not NULL: the resident data are complete only after this event
 };
-int rebuild_event(EventEntry& e, const DataPtrs* in, int mode, cudaStream_t s, const SideSetup* side_setup = nullptr);
+// chunk_h0: an FP64 build that has to generate h0 takes FP64 Taylor chunks instead of
+// evaluating it at every point.
+int rebuild_event(EventEntry& e, const DataPtrs* in, int mode, cudaStream_t s, const SideSetup* side_setup = nullptr,
+                  bool chunk_h0 = false);
 // Stream-ordered allocation from the library's memory pool (see rb_api.cu).
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t s);
 int rebuild_and_batch(EventEntry& e, const double* theta, int64_t W, double* logl, double* grad, int mode,

@@ -539,7 +539,7 @@ cudaError_t launch_summary_stored(const DataPtrs& in, const double* h0, int64_t 
 }
 
 // ===========================================================================
-// FP64 build that generates h0 (event creation, a new theta_ref): FP64 Taylor chunks.
+// FP64 build with a new fiducial point: h0 from FP64 Taylor chunks.
 //
 // k_summary evaluates h0_d at every grid point and detector from scratch (log, cbrt,
 // ten basis terms, sincos: ~500 FP64 operations per point with three
