@@ -847,13 +847,15 @@ int rb_loglike_grad_host(rb_event_t ev, const double* theta_host, int64_t W, dou
   // a graph captured for these buffers at the previous such call
   if (theta_in && out.direct && !rb::trace_events_set()) {
     bool replay;
+    uint64_t launches;
     {
       std::lock_guard<std::mutex> lk(rb::g_hg_mu);
       replay = rb::host_batch_graph(ev->e, theta_in, W, out.logl, out.grad, mode);
+      launches = ev->e.hg_launches;
       if (replay && (err = cudaGraphLaunch(ev->e.hg_exec, s)) != cudaSuccess) return cuda_fail(err, "graph launch");
     }
     if (replay) {
-      rb::count_launches(ev->e.hg_launches);
+      rb::count_launches(launches);
       err = cudaStreamSynchronize(s);
       return err == cudaSuccess ? RB_OK : cuda_fail(err, "synchronise");
     }
@@ -987,12 +989,14 @@ int rb_rebuild_loglike_grad_host(rb_event_t ev, const double* const* data_host, 
   const double* theta_in = W > 0 ? mapped_host(theta_host, 8) : nullptr;
   if (W > 0 && mapped && theta_in && out.direct && !trace_events_set()) {
     bool replay;
+    uint64_t launches;
     {
       std::lock_guard<std::mutex> lk(g_hg_mu);
       replay = host_step_graph(e, src, theta_in, W, out.logl, out.grad, mode);
+      launches = e.hs_launches;
       if (replay && (err = cudaGraphLaunch(e.hs_exec, s)) != cudaSuccess) return cuda_fail(err, "graph launch");
     }
-    if (replay) count_launches(e.hs_launches);
+    if (replay) count_launches(launches);
     else rc = enqueue_host_step(e, src, theta_in, W, out.logl, out.grad, mode, s);
     err = cudaStreamSynchronize(s);
     if (rc == RB_OK && err != cudaSuccess) rc = cuda_fail(err, "synchronise");

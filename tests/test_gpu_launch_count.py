@@ -49,3 +49,34 @@ def test_captures_do_not_count_other_threads_launches():
     assert rb.kernel_launch_count() - start == n + sum(calls)
     for e in events:
         e.free()
+
+
+def test_replays_of_one_event_from_two_threads():
+    """Two threads replay one event's captured call, one with a batch of one kernel, the
+    other with a batch of two: each replay counts its own."""
+    import torch
+    import paper_2404_11397_gb300 as rb
+    ev = small_event(sites=("H1",))
+    event = rb.Event.from_synth(ev, n_bins=70)
+    sizes, each, per_call = (64, 40_000), 300, []
+    for W in sizes:
+        n0 = rb.kernel_launch_count()
+        rb.loglike(event, torch.tensor(synth.posterior_box(ev["theta_inj"], W, seed=5), device="cuda"))
+        per_call.append(rb.kernel_launch_count() - n0)
+    assert per_call == [1, 2]
+    start = rb.kernel_launch_count()
+
+    def replays(W):
+        host = torch.empty(W, 13, dtype=torch.float64, pin_memory=True)
+        host.copy_(torch.from_numpy(synth.posterior_box(ev["theta_inj"], W, seed=5)))
+        logl = torch.empty(W, dtype=torch.float64, pin_memory=True)
+        for _ in range(each):
+            rb.loglike_grad_host(event, host, logl)
+
+    threads = [threading.Thread(target=replays, args=(W,)) for W in sizes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert rb.kernel_launch_count() - start == sum(per_call) * each
+    event.free()
