@@ -254,7 +254,8 @@ class Event:
 
     @classmethod
     def load(cls, path, stream: Optional[torch.cuda.Stream] = None) -> "Event":
-        """Build an event from a file written by save (bit-identical results)."""
+        """Build an event from a file written by save: the bits of its FP64 summary data (rb.h
+        says after which rebuilds)."""
         lib = load()
         h = ctypes.c_void_p()
         sh = _stream_handle(stream) if torch.cuda.is_available() else None
